@@ -32,10 +32,8 @@ constexpr int TAN_WARPS_PER_BLOCK = 4;   // ... and of the tangent walk (a large
 //   RECIP op:  W[t & 0x7fff] = -1 / W[a]         (t has bit 15 set)
 //   empty:     t == 0xffff
 // On the device the same op holds BYTE offsets into the cell's work array,
-// empty slots become a harmless FMA into a dummy slot, and a RECIP op (or an
-// empty slot of a pass with reciprocals) carries c == 0xffff.  A pass with
-// reciprocals may hold FMA ops in its other lanes (the interpreter runs such a
-// pass as one mixed op per lane).
+// empty slots become a harmless FMA into a dummy slot, and a RECIP op carries
+// c == 0xffff.  A pass with reciprocals may hold FMA ops in its other lanes.
 struct Op {
   uint16_t t, a, b, c;
 };
@@ -112,21 +110,25 @@ struct MechDev {
   const ushort4 *nudot_ops, *jt_ops;    // programs on the extended Wd
   const ushort4 *fwdT_ops, *bwdT_ops;   // U^T and L^T solves on WL (FP64 byte offsets)
   int nudot_npass, jt_npass, fwdT_npass, bwdT_npass;
-  const uint32_t *nudot_runs, *jt_runs, *fwdT_runs, *bwdT_runs;   // their run tables
-  int nudot_nruns, jt_nruns, fwdT_nruns, bwdT_nruns;
+  const uint32_t *nudot_runs, *jt_runs;   // run tables of nudot and jt
+  int nudot_nruns, jt_nruns;
 };
 
 // Kinds of the units a program's passes form, in its run table (one uint32 per
 // run of equal units: kind << 28 | units): a single pass of FMAs, a pair of
 // consecutive FMA passes whose 64 ops are independent of each other (the
 // interpreter loads the operands of both before it stores either result, so a
-// lane has two FMAs in flight between warp synchronisations), a pass of
-// reciprocals (and FMAs in the lanes the reciprocals leave).
+// lane has two FMAs in flight between warp synchronisations), three passes with
+// reciprocals in the first (RECIP): a lane with a reciprocal spends three FP64
+// instructions on it and has no op in the other two, every other lane runs its
+// three FMA ops; all ops of the unit are independent of each other.
 constexpr uint32_t RUN_FMA1 = 0, RUN_FMA2 = 1, RUN_RECIP = 2;
 
 struct HostProgram {
   std::vector<Op> ops;   // n_pass * 32
-  std::vector<uint8_t> unit;   // per pass: 0 single FMA pass, 1 / 2 first / second pass of a pair, 3 reciprocals
+  // per pass: 0 single FMA pass, 1 / 2 first / second pass of a pair, 3 the
+  // first pass of a reciprocal unit (the two passes after it, marked 0, belong to it)
+  std::vector<uint8_t> unit;
   int n_ops = 0;
   int n_pass() const { return (int)(ops.size() / WARP); }
   std::vector<uint32_t> runs() const {
@@ -134,6 +136,7 @@ struct HostProgram {
     uint32_t kind = 0xf, n = 0;
     for (size_t p = 0; p < unit.size(); ++p) {
       if (unit[p] == 2) continue;
+      if (p >= 1 && unit[p - 1] == 3) { ++p; continue; }   // the second and third pass of a reciprocal unit
       const uint32_t k = unit[p] == 1 ? RUN_FMA2 : unit[p] == 3 ? RUN_RECIP : RUN_FMA1;
       if (k != kind && n) r.push_back(kind << 28 | n), n = 0;
       kind = k;

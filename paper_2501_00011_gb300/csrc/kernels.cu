@@ -97,37 +97,6 @@ __device__ __forceinline__ float lds(float *, uint32_t a) {
 __device__ __forceinline__ void sts(uint32_t a, double v) { asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory"); }
 __device__ __forceinline__ void sts(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
 
-// Run a warp program (byte-offset ops, see internal.h) over the work array W,
-// the next pass's op prefetched.  The loop is deliberately not unrolled and
-// prefetches one pass only: the solve kernel is bound by instruction fetch as
-// much as by latency, and deeper prefetch (unrolled copies of the pass body at
-// every call site) measured 17% slower on the persistent driver and 33% on the
-// plain one.  Calls out of line measured slower still (register save/restore).
-template <typename T, bool NEG, bool SMEM>
-__device__ __forceinline__ void run_ops(const ushort4 *ops, const int np, T *W, const int lane) {
-  const uint32_t wb = smem_addr(W);
-  T *const tag = nullptr;
-  ops += lane;
-  uint2 next = np > 0 ? ld_op<SMEM>(ops) : make_uint2(0, 0);   // packed: x = t | a << 16, y = b | c << 16
-#pragma unroll 1
-  for (int p = 0; p < np; ++p) {
-    const uint2 op = next;
-    if (p + 1 < np) next = ld_op<SMEM>(ops + (size_t)(p + 1) * WARP);
-    const uint32_t ot = op.x & 0xffff, oa = op.x >> 16, ob = op.y & 0xffff, oc = op.y >> 16;
-    if (oc == DEV_RECIP) {
-      sts(wb + ot, -lu_recip(lds(tag, wb + oa)));
-    } else {
-      const T a = lds(tag, wb + oa), b = lds(tag, wb + ob), c = lds(tag, wb + oc);
-      sts(wb + ot, NEG ? fma(-a, b, c) : fma(a, b, c));
-    }
-    __syncwarp();
-  }
-}
-
-// The same interpreter for programs in global memory, with the ops streamed
-// RING passes ahead by cp.async into a ring of RING x 256 bytes of shared
-// memory (ring: 8-byte aligned shared address).  Each lane copies and reads
-// only its own op slots, so cp.async.wait_group alone orders them.
 __device__ __forceinline__ void cp_async8(uint32_t dst, const void *src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -135,131 +104,128 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// The next pass's op is read from the ring one pass ahead, so that shared-memory
-// load overlaps the current pass (the ring slot it reuses held the op read two
-// passes earlier).
-template <typename T, bool NEG, int RING>
-__device__ __forceinline__ void run_ops_ring(const ushort4 *ops, const int np, T *W, const int lane, const uint32_t ring) {
-  const uint32_t wb = smem_addr(W);
-  T *const tag = nullptr;
-  const uint2 *g = reinterpret_cast<const uint2 *>(ops) + lane;
-  const uint32_t rb = ring + 8u * lane;
-#pragma unroll 1
-  for (int i = 0; i < RING - 1; ++i) {
-    if (i < np) cp_async8(rb + 256u * i, g + (size_t)i * WARP);
-    cp_async_commit();
-  }
-  cp_async_wait<RING - 2>();            // pass 0's group has landed
-  uint32_t nx = 0, ny = 0;
-  if (np > 0) asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(nx), "=r"(ny) : "r"(rb) : "memory");
-#pragma unroll 1
-  for (int p = 0; p < np; ++p) {
-    const uint32_t ox = nx, oy = ny;
-    const int q = p + RING - 1;
-    if (q < np) cp_async8(rb + 256u * (q % RING), g + (size_t)q * WARP);
-    cp_async_commit();
-    cp_async_wait<RING - 2>();          // pass p+1's group has landed
-    if (p + 1 < np)
-      asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(nx), "=r"(ny) : "r"(rb + 256u * ((p + 1) % RING)) : "memory");
-    const uint32_t ot = ox & 0xffff, oa = ox >> 16, ob = oy & 0xffff, oc = oy >> 16;
-    if (oc == DEV_RECIP) {
-      sts(wb + ot, -lu_recip(lds(tag, wb + oa)));
-    } else {
-      const T a = lds(tag, wb + oa), b = lds(tag, wb + ob), c = lds(tag, wb + oc);
-      sts(wb + ot, NEG ? fma(-a, b, c) : fma(a, b, c));
-    }
-    __syncwarp();
-  }
-  cp_async_wait<0>();                   // nothing in flight once the ring's memory is reused
+// A lane's op as shared addresses: the work array's base plus the op's byte
+// offsets (packed op: x = t | a << 16, y = b | c << 16).
+struct OpAddr {
+  uint32_t t, a, b, c;
+};
+__device__ __forceinline__ OpAddr unpack(uint32_t wb, uint2 o) {
+  return OpAddr{wb + (o.x & 0xffff), wb + (o.x >> 16), wb + (o.y & 0xffff), wb + (o.y >> 16)};
 }
 
-// One FMA op / a pair of independent FMA ops / a reciprocal op of a lane
-// (packed ops: x = t | a << 16, y = b | c << 16, byte offsets into W at wb).
-template <typename T, bool NEG>
-__device__ __forceinline__ void op_fma(uint32_t wb, uint2 o) {
-  T *const tag = nullptr;
-  const T a = lds(tag, wb + (o.x >> 16)), b = lds(tag, wb + (o.y & 0xffff)), c = lds(tag, wb + (o.y >> 16));
-  sts(wb + (o.x & 0xffff), NEG ? fma(-a, b, c) : fma(a, b, c));
-}
-template <typename T, bool NEG>
-__device__ __forceinline__ void op_fma2(uint32_t wb, uint2 o, uint2 u) {
-  T *const tag = nullptr;
-  const T a = lds(tag, wb + (o.x >> 16)), b = lds(tag, wb + (o.y & 0xffff)), c = lds(tag, wb + (o.y >> 16));
-  const T a2 = lds(tag, wb + (u.x >> 16)), b2 = lds(tag, wb + (u.y & 0xffff)), c2 = lds(tag, wb + (u.y >> 16));
-  sts(wb + (o.x & 0xffff), NEG ? fma(-a, b, c) : fma(a, b, c));
-  sts(wb + (u.x & 0xffff), NEG ? fma(-a2, b2, c2) : fma(a2, b2, c2));
-}
-// A lane of a pass with reciprocals: W[t] = -1/W[a] (c == DEV_RECIP) or an
-// FMA, without a branch.  FP64: every lane forms the estimate r of 1/W[a] and
-// the cubic step's e = 1 - x r, e + e^2 (recip_nr), and the final FMA is
-// fma(-r, e + e^2, -r) = -recip_nr(x) in a reciprocal lane, the op's own FMA
-// in the others (whose r and e are discarded).
-template <typename T, bool NEG>
-__device__ __forceinline__ void op_mixed(uint32_t wb, uint2 o);
+// A lane of a reciprocal unit (three passes, ops o, u, v).  Without a
+// reciprocal: three independent FMAs.  With one (o.c is the DEV_RECIP marker,
+// u and v are empty): W[t] = -1/W[a]; the three FP64 instructions of the cubic
+// step, e = 1 - x r, e + e^2 and fma(-r, e + e^2, -r) = -recip_nr(x), are the
+// three FMAs of the lane, so the warp's other lanes lose none.  (A pass whose
+// other lanes ran one FMA each spent 383 FP64 instructions on the factorisation
+// of the 72-species mechanism; these units spend 337.)
+template <typename T>
+struct RecipUnit;
 template <>
-__device__ __forceinline__ void op_mixed<double, false>(uint32_t wb, uint2 o) {
-  double *const tag = nullptr;
-  const uint32_t oa = o.x >> 16, oc = o.y >> 16;
-  const bool rcp = oc == DEV_RECIP;
-  const double x = lds(tag, wb + oa), b = lds(tag, wb + (rcp ? oa : (o.y & 0xffff))), c = lds(tag, wb + (rcp ? oa : oc));
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  const double ee = fma(e, e, e);
-  sts(wb + (o.x & 0xffff), rcp ? fma(-r, ee, -r) : fma(x, b, c));
-}
+struct RecipUnit<double> {
+  double p1, p2, p3;
+  bool rcp;
+  __device__ __forceinline__ void load_and_run(uint32_t wb, const OpAddr &o, const OpAddr &u, const OpAddr &v) {
+    double *const tag = nullptr;
+    rcp = o.c == wb + DEV_RECIP;
+    const double x = lds(tag, o.a), b = lds(tag, rcp ? o.a : o.b), c = lds(tag, rcp ? o.a : o.c);
+    const double a2 = lds(tag, u.a), b2 = lds(tag, u.b), c2 = lds(tag, u.c);
+    const double a3 = lds(tag, v.a), b3 = lds(tag, v.b), c3 = lds(tag, v.c);
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    p1 = fma(rcp ? -x : x, rcp ? r : b, rcp ? 1.0 : c);
+    p2 = fma(rcp ? p1 : a2, rcp ? p1 : b2, rcp ? p1 : c2);
+    p3 = fma(rcp ? -r : a3, rcp ? p2 : b3, rcp ? -r : c3);
+  }
+  __device__ __forceinline__ void store(const OpAddr &o, const OpAddr &u, const OpAddr &v) const {
+    sts(o.t, rcp ? p3 : p1);
+    sts(u.t, p2);                       // a reciprocal's lane: the dummy slot
+    sts(v.t, p3);
+  }
+};
 template <>
-__device__ __forceinline__ void op_mixed<float, false>(uint32_t wb, uint2 o) {
-  float *const tag = nullptr;
-  const uint32_t oa = o.x >> 16, oc = o.y >> 16;
-  const bool rcp = oc == DEV_RECIP;
-  const float x = lds(tag, wb + oa), b = lds(tag, wb + (rcp ? oa : (o.y & 0xffff))), c = lds(tag, wb + (rcp ? oa : oc));
-  sts(wb + (o.x & 0xffff), rcp ? -__frcp_rn(x) : fmaf(x, b, c));
-}
+struct RecipUnit<float> {
+  float p1, p2, p3;
+  __device__ __forceinline__ void load_and_run(uint32_t wb, const OpAddr &o, const OpAddr &u, const OpAddr &v) {
+    float *const tag = nullptr;
+    const bool rcp = o.c == wb + DEV_RECIP;
+    const float x = lds(tag, o.a), b = lds(tag, rcp ? o.a : o.b), c = lds(tag, rcp ? o.a : o.c);
+    const float a2 = lds(tag, u.a), b2 = lds(tag, u.b), c2 = lds(tag, u.c);
+    const float a3 = lds(tag, v.a), b3 = lds(tag, v.b), c3 = lds(tag, v.c);
+    p1 = rcp ? -__frcp_rn(x) : fmaf(x, b, c);
+    p2 = fmaf(a2, b2, c2);
+    p3 = fmaf(a3, b3, c3);
+  }
+  __device__ __forceinline__ void store(const OpAddr &o, const OpAddr &u, const OpAddr &v) const {
+    sts(o.t, p1);
+    sts(u.t, p2);
+    sts(v.t, p3);
+  }
+};
 
-// A program with a run table (RUN_* units, internal.h).  The ops of the next
-// two passes are held in registers (n0, n1) and refilled as the units consume
-// them, so a unit never waits for its own ops.  Runs are read from shared
-// memory (SMEM) or global memory like the ops; WIDE / RECIP: the program has
-// pair / reciprocal units (a run table without them compiles to a plain loop).
-template <typename T, bool NEG, bool SMEM, bool WIDE, bool RECIP>
+// A program with a run table (RUN_* units, internal.h).  The addresses of the
+// next two passes' ops are held in registers (A0, A1); a unit loads the ops
+// that follow it before its own operands and turns them into addresses while
+// its FMAs are in flight, so neither the loads nor the address arithmetic sit
+// between a unit's stores and the next unit's operand loads.  Runs are read
+// from shared memory (SMEM) or global memory like the ops; WIDE / RECIP: the
+// program has pair / reciprocal units (a run table without them compiles to a
+// plain loop).
+template <typename T, bool SMEM, bool WIDE, bool RECIP>
 __device__ __forceinline__ void run_prog(const ushort4 *ops, const uint32_t *runs, const int nruns, const int np, T *W,
                                          const int lane) {
   const uint32_t wb = smem_addr(W);
+  T *const tag = nullptr;
   ops += lane;
-  uint2 n0 = np > 0 ? ld_op<SMEM>(ops) : make_uint2(0, 0);
-  uint2 n1 = np > 1 ? ld_op<SMEM>(ops + WARP) : make_uint2(0, 0);
+  uint2 r0 = np > 0 ? ld_op<SMEM>(ops) : make_uint2(0, 0);
+  uint2 r1 = np > 1 ? ld_op<SMEM>(ops + WARP) : make_uint2(0, 0);
+  OpAddr A0 = unpack(wb, r0), A1 = unpack(wb, r1);
   int p = 0;
 #pragma unroll 1
   for (int r = 0; r < nruns; ++r) {
-    const uint32_t rr = SMEM ? runs[r] : __ldg(runs + r);
+    // (without pairs and reciprocals the program is one run of all its passes)
+    const uint32_t rr = !WIDE && !RECIP ? (uint32_t)np : SMEM ? runs[r] : __ldg(runs + r);
     const uint32_t kind = rr >> 28;
     int n = (int)(rr & 0x0fffffffu);
     if (WIDE && kind == RUN_FMA2) {
 #pragma unroll 1
       for (; n > 0; --n, p += 2) {
-        const uint2 o = n0, u = n1;
-        if (p + 2 < np) n0 = ld_op<SMEM>(ops + (size_t)(p + 2) * WARP);
-        if (p + 3 < np) n1 = ld_op<SMEM>(ops + (size_t)(p + 3) * WARP);
-        op_fma2<T, NEG>(wb, o, u);
+        if (p + 2 < np) r0 = ld_op<SMEM>(ops + (size_t)(p + 2) * WARP);
+        if (p + 3 < np) r1 = ld_op<SMEM>(ops + (size_t)(p + 3) * WARP);
+        const T a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
+        const T a2 = lds(tag, A1.a), b2 = lds(tag, A1.b), c2 = lds(tag, A1.c);
+        const T v = fma(a, b, c), v2 = fma(a2, b2, c2);
+        const uint32_t t = A0.t, t2 = A1.t;
+        A0 = unpack(wb, r0);
+        A1 = unpack(wb, r1);
+        sts(t, v);
+        sts(t2, v2);
         __syncwarp();
       }
     } else if (RECIP && kind == RUN_RECIP) {
 #pragma unroll 1
-      for (; n > 0; --n, ++p) {
-        const uint2 o = n0;
-        n0 = n1;
-        if (p + 2 < np) n1 = ld_op<SMEM>(ops + (size_t)(p + 2) * WARP);
-        op_mixed<T, NEG>(wb, o);
+      for (; n > 0; --n, p += 3) {
+        const OpAddr A2 = unpack(wb, ld_op<SMEM>(ops + (size_t)(p + 2) * WARP));
+        if (p + 3 < np) r0 = ld_op<SMEM>(ops + (size_t)(p + 3) * WARP);
+        if (p + 4 < np) r1 = ld_op<SMEM>(ops + (size_t)(p + 4) * WARP);
+        RecipUnit<T> ru;
+        ru.load_and_run(wb, A0, A1, A2);
+        ru.store(A0, A1, A2);
+        A0 = unpack(wb, r0);
+        A1 = unpack(wb, r1);
         __syncwarp();
       }
     } else {
 #pragma unroll 1
       for (; n > 0; --n, ++p) {
-        const uint2 o = n0;
-        n0 = n1;
-        if (p + 2 < np) n1 = ld_op<SMEM>(ops + (size_t)(p + 2) * WARP);
-        op_fma<T, NEG>(wb, o);
+        if (p + 2 < np) r0 = ld_op<SMEM>(ops + (size_t)(p + 2) * WARP);
+        const T a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
+        const T v = fma(a, b, c);
+        const uint32_t t = A0.t;
+        A0 = A1;
+        A1 = unpack(wb, r0);
+        sts(t, v);
         __syncwarp();
       }
     }
@@ -267,64 +233,92 @@ __device__ __forceinline__ void run_prog(const ushort4 *ops, const uint32_t *run
 }
 
 // The same for programs in global memory, the ops streamed through a ring of
-// RING x 256 bytes of shared memory (ring: 8-byte aligned shared address) as
-// in run_ops_ring.  Invariant at the start of a unit at pass p: passes up to
-// p + RING - 3 are issued and the ops of passes p and p + 1 are in n0, n1.  A
-// unit issues one pass per pass it consumes, into the slots of passes p - 2
-// (and p - 1), whose ops were read into registers and used by earlier units;
-// it then waits until pass p + 2 (and p + 3) has landed and refills n0, n1.
-template <typename T, bool NEG, int RING, bool WIDE, bool RECIP>
+// RING x 256 bytes of shared memory (ring: 8-byte aligned shared address) by
+// cp.async.  Each lane copies and reads only its own op slots, so
+// cp.async.wait_group alone orders them.  Invariant at the start of a unit at
+// pass p: passes up to p + RING - 3 are issued and the ops of passes p and
+// p + 1 are in A0, A1.  A unit issues one pass per pass it consumes, into the
+// slots of passes p - 2, p - 1 (read into registers by earlier units) and, a
+// reciprocal unit, p (whose op's addresses its operand loads have used by
+// then); it waits until the passes after it have landed and refills A0, A1.
+template <typename T, int RING, bool WIDE, bool RECIP>
 __device__ __forceinline__ void run_prog_ring(const ushort4 *ops, const uint32_t *runs, const int nruns, const int np, T *W,
                                               const int lane, const uint32_t ring) {
-  static_assert(RING >= 6, "ring too shallow to run ahead");
+  static_assert(RING >= 6 && (RING & (RING - 1)) == 0, "ring too shallow to run ahead, or not a power of two");
   const uint32_t wb = smem_addr(W);
+  T *const tag = nullptr;
   const uint2 *g = reinterpret_cast<const uint2 *>(ops) + lane;
   const uint32_t rb = ring + 8u * lane;
-#pragma unroll 1
-  for (int i = 0; i < RING - 2; ++i) {
-    if (i < np) cp_async8(rb + 256u * i, g + (size_t)i * WARP);
+  auto issue = [&](int q) {             // pass q into its ring slot (nothing past the end)
+    if (q < np) cp_async8(rb + 256u * (q % RING), g + (size_t)q * WARP);
     cp_async_commit();
-  }
+  };
+  auto fetch = [&](int q) {
+    uint2 o;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(o.x), "=r"(o.y) : "r"(rb + 256u * (q % RING)) : "memory");
+    return o;
+  };
+#pragma unroll 1
+  for (int i = 0; i < RING - 2; ++i) issue(i);
   cp_async_wait<RING - 4>();            // passes 0 and 1 have landed
-  uint2 n0 = make_uint2(0, 0), n1 = make_uint2(0, 0);
-  if (np > 0) asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(n0.x), "=r"(n0.y) : "r"(rb) : "memory");
-  if (np > 1) asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(n1.x), "=r"(n1.y) : "r"(rb + 256u) : "memory");
+  uint2 r0 = make_uint2(0, 0), r1 = make_uint2(0, 0);
+  if (np > 0) r0 = fetch(0);
+  if (np > 1) r1 = fetch(1);
+  OpAddr A0 = unpack(wb, r0), A1 = unpack(wb, r1);
   int p = 0;
 #pragma unroll 1
   for (int r = 0; r < nruns; ++r) {
-    const uint32_t rr = __ldg(runs + r);
+    const uint32_t rr = !WIDE && !RECIP ? (uint32_t)np : __ldg(runs + r);
     const uint32_t kind = rr >> 28;
     int n = (int)(rr & 0x0fffffffu);
     if (WIDE && kind == RUN_FMA2) {
 #pragma unroll 1
       for (; n > 0; --n, p += 2) {
-        const uint2 o = n0, u = n1;
-        const int q = p + RING - 2;
-        if (q < np) cp_async8(rb + 256u * (q % RING), g + (size_t)q * WARP);
-        cp_async_commit();
-        if (q + 1 < np) cp_async8(rb + 256u * ((q + 1) % RING), g + (size_t)(q + 1) * WARP);
-        cp_async_commit();
+        issue(p + RING - 2);
+        issue(p + RING - 1);
         cp_async_wait<RING - 4>();      // passes p + 2 and p + 3 have landed
-        if (p + 2 < np)
-          asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(n0.x), "=r"(n0.y) : "r"(rb + 256u * ((p + 2) % RING)) : "memory");
-        if (p + 3 < np)
-          asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(n1.x), "=r"(n1.y) : "r"(rb + 256u * ((p + 3) % RING)) : "memory");
-        op_fma2<T, NEG>(wb, o, u);
+        if (p + 2 < np) r0 = fetch(p + 2);
+        if (p + 3 < np) r1 = fetch(p + 3);
+        const T a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
+        const T a2 = lds(tag, A1.a), b2 = lds(tag, A1.b), c2 = lds(tag, A1.c);
+        const T v = fma(a, b, c), v2 = fma(a2, b2, c2);
+        const uint32_t t = A0.t, t2 = A1.t;
+        A0 = unpack(wb, r0);
+        A1 = unpack(wb, r1);
+        sts(t, v);
+        sts(t2, v2);
+        __syncwarp();
+      }
+    } else if (RECIP && kind == RUN_RECIP) {
+#pragma unroll 1
+      for (; n > 0; --n, p += 3) {
+        cp_async_wait<RING - 5>();      // pass p + 2 has landed
+        const OpAddr A2 = unpack(wb, fetch(p + 2));
+        RecipUnit<T> ru;
+        ru.load_and_run(wb, A0, A1, A2);
+        issue(p + RING - 2);
+        issue(p + RING - 1);
+        issue(p + RING);
+        cp_async_wait<RING - 4>();      // passes p + 3 and p + 4 have landed
+        if (p + 3 < np) r0 = fetch(p + 3);
+        if (p + 4 < np) r1 = fetch(p + 4);
+        ru.store(A0, A1, A2);
+        A0 = unpack(wb, r0);
+        A1 = unpack(wb, r1);
         __syncwarp();
       }
     } else {
 #pragma unroll 1
       for (; n > 0; --n, ++p) {
-        const uint2 o = n0;
-        n0 = n1;
-        const int q = p + RING - 2;
-        if (q < np) cp_async8(rb + 256u * (q % RING), g + (size_t)q * WARP);
-        cp_async_commit();
+        issue(p + RING - 2);
         cp_async_wait<RING - 4>();      // pass p + 2 has landed
-        if (p + 2 < np)
-          asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(n1.x), "=r"(n1.y) : "r"(rb + 256u * ((p + 2) % RING)) : "memory");
-        if (RECIP && kind == RUN_RECIP) op_mixed<T, NEG>(wb, o);
-        else op_fma<T, NEG>(wb, o);
+        if (p + 2 < np) r0 = fetch(p + 2);
+        const T a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
+        const T v = fma(a, b, c);
+        const uint32_t t = A0.t;
+        A0 = A1;
+        A1 = unpack(wb, r0);
+        sts(t, v);
         __syncwarp();
       }
     }
@@ -368,6 +362,8 @@ __device__ __forceinline__ bool eq_fp(double a, double b) {
   const unsigned long long ua = ubits(a), ub = ubits(b);
   return (ua == ub && (ua & ABS_MASK) <= INF_BITS) || ((ua | ub) & ABS_MASK) == 0;
 }
+// +0 + x without the FP64 add: x, but -0 becomes +0
+__device__ __forceinline__ double plus0(double x) { return ubits(x) == ~ABS_MASK ? 0.0 : x; }
 // x < 0 (false for -0 and NaN; true for -inf)
 __device__ __forceinline__ bool lt0(double x) {
   const unsigned long long u = ubits(x), a = u & ABS_MASK;
@@ -508,7 +504,7 @@ __device__ __forceinline__ void f_core(const MechDev &M, const unsigned char *tb
     sts(rt + 8u * j, r);
   }
   __syncwarp();
-  run_prog<double, false, STAGED, true, false>(reinterpret_cast<const ushort4 *>(tbase + M.tab.f_ops),
+  run_prog<double, STAGED, true, false>(reinterpret_cast<const ushort4 *>(tbase + M.tab.f_ops),
                                                reinterpret_cast<const uint32_t *>(tbase + M.tab.f_runs), M.f_nruns,
                                                M.f_npass, Wd, lane);
 }
@@ -562,12 +558,12 @@ __device__ __forceinline__ void mlu_core(const MechDev &M, const unsigned char *
   // read from L2 two passes ahead.  The LU program's ops are streamed through a
   // ring in the rates and f slots of Wd, dead once M is formed (too small a
   // region: read from L2 as well).
-  run_prog<T, false, false, true, false>(M.m_ops[prec], M.m_runs, M.m_nruns, M.m_npass, reinterpret_cast<T *>(Wd), lane);
+  run_prog<T, false, true, false>(M.m_ops[prec], M.m_runs, M.m_nruns, M.m_npass, reinterpret_cast<T *>(Wd), lane);
   const uint32_t wr = smem_addr(Wd + M.d_RT);            // 8-byte aligned (a double slot)
   if ((M.R + M.S) * 8 >= 8 * 256)
-    run_prog_ring<T, false, 8, true, true>(M.lu_ops[prec], M.lu_runs, M.lu_nruns, M.lu_npass, WL, lane, wr);
+    run_prog_ring<T, 8, true, true>(M.lu_ops[prec], M.lu_runs, M.lu_nruns, M.lu_npass, WL, lane, wr);
   else
-    run_prog<T, false, false, true, true>(M.lu_ops[prec], M.lu_runs, M.lu_nruns, M.lu_npass, WL, lane);
+    run_prog<T, false, true, true>(M.lu_ops[prec], M.lu_runs, M.lu_nruns, M.lu_npass, WL, lane);
 }
 
 // a5: forward and backward substitution with the LDU factors on the vector in
@@ -582,21 +578,17 @@ __device__ __forceinline__ void solve_core(const MechDev &M, const unsigned char
   const ushort4 *bwd = reinterpret_cast<const ushort4 *>(tbase + M.tab.bwd_ops);
   T *const W = reinterpret_cast<T *>(Wd);                 // the programs address the whole per-cell slice
   if (STAGED) {
-    run_ops<T, false, true>(fwd, M.fwd_npass, W, lane);
-    run_ops<T, false, true>(bwd, M.bwd_npass, W, lane);
+    run_prog<T, true, false, false>(fwd, nullptr, 1, M.fwd_npass, W, lane);
+    run_prog<T, true, false, false>(bwd, nullptr, 1, M.bwd_npass, W, lane);
     return;
   }
   const uint32_t rb = smem_addr(Wd + M.d_RT);            // the rates and f slots: dead during a solve
-  const int cap = (M.R + M.S) * 8;
-  if (cap >= 8 * 256) {
-    run_ops_ring<T, false, 8>(fwd, M.fwd_npass, W, lane, rb);
-    run_ops_ring<T, false, 8>(bwd, M.bwd_npass, W, lane, rb);
-  } else if (cap >= 4 * 256) {
-    run_ops_ring<T, false, 4>(fwd, M.fwd_npass, W, lane, rb);
-    run_ops_ring<T, false, 4>(bwd, M.bwd_npass, W, lane, rb);
+  if ((M.R + M.S) * 8 >= 8 * 256) {
+    run_prog_ring<T, 8, false, false>(fwd, nullptr, 1, M.fwd_npass, W, lane, rb);
+    run_prog_ring<T, 8, false, false>(bwd, nullptr, 1, M.bwd_npass, W, lane, rb);
   } else {
-    run_ops<T, false, false>(fwd, M.fwd_npass, W, lane);
-    run_ops<T, false, false>(bwd, M.bwd_npass, W, lane);
+    run_prog<T, false, false, false>(fwd, nullptr, 1, M.fwd_npass, W, lane);
+    run_prog<T, false, false, false>(bwd, nullptr, 1, M.bwd_npass, W, lane);
   }
 }
 
@@ -730,16 +722,19 @@ __device__ __forceinline__ void get_row(const double (&D)[NROW][KS], int r, doub
 #undef CHEM_ROW_CASE
 }
 
-// Accepted step at order q: D_{q+2} = d - D_{q+1}, D_{q+1} = d, then
-// D_m += D_{m+1} for m = q .. 0.
+// Accepted step at order q: D_{q+2} = d - D_{q+1} (only with `top`), D_{q+1} = d,
+// then D_m += D_{m+1} for m = q .. 0.  D_{q+2} is read by the order selection
+// after the step and, when that raises the order, by the next step; a step
+// without a selection need not form it (the next accepted step at this order
+// overwrites it, and at a lower order the row is above those it touches).
 template <int KS>
-__device__ __forceinline__ void accept_update(double (&D)[NROW][KS], int q, const double (&d)[KS]) {
+__device__ __forceinline__ void accept_update(double (&D)[NROW][KS], int q, const double (&d)[KS], bool top = true) {
 #define CHEM_UPD_CASE(Q_)                                                      \
   case Q_:                                                                    \
-    _Pragma("unroll") for (int k = 0; k < KS; ++k) {                          \
-      D[Q_ + 2][k] = d[k] - D[Q_ + 1][k];                                     \
-      D[Q_ + 1][k] = d[k];                                                    \
+    if (top) {                                                                \
+      _Pragma("unroll") for (int k = 0; k < KS; ++k) D[Q_ + 2][k] = d[k] - D[Q_ + 1][k]; \
     }                                                                         \
+    _Pragma("unroll") for (int k = 0; k < KS; ++k) D[Q_ + 1][k] = d[k];       \
     _Pragma("unroll") for (int m = Q_; m >= 0; --m)                           \
       _Pragma("unroll") for (int k = 0; k < KS; ++k) D[m][k] += D[m + 1][k];  \
     break;
@@ -965,6 +960,9 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
     rec.push_row(EV_INIT, q, h, y0, lane);
 
     double t = 0.0, cM = 0.0, icM = 0.0, rho2 = 1.0;   // rho2: squared convergence-rate estimate
+    // the correction's scale 2/(1 + c/c_M) and the c it belongs to (with this
+    // M): steps at an unchanged c reuse both it and its test |c/c_M - 1| <= DGMAX
+    double scale = 1.0, scale_c = 0.0;
     int n_eq = 0, have_M = 0, force_M = 0, n_since_M = 0, nef = 0, ncf = 0, last = 0;
     const int qmax = P.max_order;
     double ypred[KS], psi[KS], d[KS], y[KS], x[KS];
@@ -973,23 +971,34 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
     const double *gfac = gtab<double>(tb, M.tab.g), *lim = gtab<double>(tb, M.tab.lim);
     for (;;) {
       if (st.steps >= P.max_steps) { status = CHEM_CELL_MAX_STEPS; break; }
+      // dt - t, h (1 + STRETCH), t + h and c = h / gamma_q are one FP64 instruction
+      // over four lanes (each costs the warp as much as 32): fma(-1, t, dt),
+      // fma(1 + STRETCH, h, 0), fma(1, h, t), fma(1/gamma_q, h, 0), all with the
+      // rounding of the plain operation (h > 0)
+      const double iq = c_igam[q];
+      double rem, hs, tn, c;
+      {
+        const double a = lane == 0 ? -1.0 : lane == 1 ? 1.0 + STRETCH : lane == 2 ? 1.0 : iq;
+        const double r = fma(a, lane == 0 ? t : h, lane == 0 ? dt : lane == 2 ? t : 0.0);
+        rem = __shfl_sync(FULL, r, 0);
+        hs = __shfl_sync(FULL, r, 1);
+        tn = __shfl_sync(FULL, r, 2);
+        c = __shfl_sync(FULL, r, 3);
+      }
       // dt - t >= +0 always (t < dt inside the loop)
-      if (le_nn(dt - t, h * (1.0 + STRETCH))) {
-        const double hn = dt - t;
-        if (!eq_fp(hn, h)) {
-          rescale<KS>(D, q, hn / h, M.rescale_coef, lane);
-          rec.push(EV_RESCALE, q, hn / h, lane);
-          h = hn;
+      if (le_nn(rem, hs)) {
+        if (!eq_fp(rem, h)) {
+          rescale<KS>(D, q, rem / h, M.rescale_coef, lane);
+          rec.push(EV_RESCALE, q, rem / h, lane);
+          h = rem;
+          c = h * iq;
           n_eq = 0;
         }
         last = 1;
       } else {
         last = 0;
       }
-      if (!last && eq_fp(t + h, t)) { status = CHEM_CELL_H_TOO_SMALL; break; }
-
-      const double iq = c_igam[q];
-      const double c = h * iq;
+      if (!last && eq_fp(tn, t)) { status = CHEM_CELL_H_TOO_SMALL; break; }
 #pragma unroll
       for (int k = 0; k < KS; ++k) {
         ypred[k] = D[0][k];
@@ -1009,7 +1018,9 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
       for (int k = 0; k < KS; ++k) psi[k] *= iq;
 
       int fresh = 0;
-      if (!have_M || force_M || gt_nn(__longlong_as_double(__double_as_longlong(fma(c, icM, -1.0)) & ABS_MASK), DGMAX) ||
+      const bool same_c = eq_fp(c, scale_c);
+      if (!have_M || force_M ||
+          (!same_c && gt_nn(__longlong_as_double(__double_as_longlong(fma(c, icM, -1.0)) & ABS_MASK), DGMAX)) ||
           n_since_M >= MSBP) {
         cl.form_and_factor(c, ypred);
         have_M = 1;
@@ -1023,8 +1034,10 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
       }
       force_M = 0;
       const bool scaled = !eq_fp(c, cM);
-      double scale = 1.0;
-      if (scaled) scale = 2.0 * recip_nr(fma(c, icM, 1.0));
+      if (fresh || !same_c) {
+        scale_c = c;
+        if (scaled) scale = 2.0 * recip_nr(fma(c, icM, 1.0));
+      }
       const double tol2 = lim[8 + q];     // S (0.1 (q+1))^2
 
 #pragma unroll
@@ -1041,7 +1054,11 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
         cl.eval_f(y, f);
         st.f_evals++;
 #pragma unroll
-        for (int k = 0; k < KS; ++k) tmp[k] = c * f[k] - psi[k] - d[k];
+        for (int k = 0; k < KS; ++k) tmp[k] = fma(c, f[k], -psi[k]);
+        if (it > 0) {                      // d = +0 before the first correction
+#pragma unroll
+          for (int k = 0; k < KS; ++k) tmp[k] -= d[k];
+        }
         cl.solve(tmp, x);
         st.solves++;
         if (scaled) {
@@ -1050,14 +1067,18 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
         }
         del2 = grp.sum(cl.sumsq(x, w));
         if (COUPLED) del2 *= gsc;
+        if (it > 0) {
 #pragma unroll
-        for (int k = 0; k < KS; ++k) {
-          d[k] += x[k];
-          y[k] = ypred[k] + d[k];
+          for (int k = 0; k < KS; ++k) d[k] += x[k];
+        } else {
+#pragma unroll
+          for (int k = 0; k < KS; ++k) d[k] = plus0(x[k]);
         }
+#pragma unroll
+        for (int k = 0; k < KS; ++k) y[k] = ypred[k] + d[k];
         st.newton_iters++;
         if (it > 0) rho2 = max_nn(CRDOWN * CRDOWN * rho2, del2 * idel2_prev);
-        if (le_nn(le_nn(rho2, 1.0) ? del2 * rho2 : del2, tol2)) { conv = 1; break; }
+        if (le_nn(gt_nn(1.0, rho2) ? del2 * rho2 : del2, tol2)) { conv = 1; break; }
         if (it > 0 && gt_nn(del2, RDIV * RDIV * del2_prev)) break;
         // not converged, so del2 > tol2 >= 1e-2 S (q >= 1): a normal number
         del2_prev = del2;
@@ -1079,6 +1100,7 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
       }
 
       // inequality constraint y >= 0
+      bool projected = false;   // d changed after the last correction
       unsigned pm[KS];          // species projected onto y = 0 (ballot per register slot)
 #pragma unroll
       for (int k = 0; k < KS; ++k) pm[k] = 0u;
@@ -1100,6 +1122,7 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
           if (COUPLED) vs *= gsc;
           eta_c = grp.min(warp_min(eta_c));
           if (le_nn(vs, tol2)) {
+            projected = true;
 #pragma unroll
             for (int k = 0; k < KS; ++k) {
               const bool p = cl.own[k] && lt0(y[k]);
@@ -1125,8 +1148,12 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
       }
 
       // local error test: (||d|| / (q+1))^2 <= 1, as the raw sum against S (q+1)^2
-      double err2 = grp.sum(cl.sumsq(d, w));
-      if (COUPLED) err2 *= gsc;
+      // (after a single correction d is that correction, whose sum is del2)
+      double err2 = del2;
+      if (n_it > 1 || projected) {
+        err2 = grp.sum(cl.sumsq(d, w));
+        if (COUPLED) err2 *= gsc;
+      }
       const int ie = grid_idx(thr2, err2, q, lane);
       if (!le_nn(err2, lim[q])) {
         st.rejects++;
@@ -1143,18 +1170,18 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
       }
 
       // accept: update the backward differences
-      t = last ? dt : t + h;
+      t = last ? dt : tn;
       st.steps++;
       st.order_sum += q;
       n_since_M++;
       nef = 0;
       ncf = 0;
-      accept_update<KS>(D, q, d);
+      n_eq++;
+      accept_update<KS>(D, q, d, n_eq >= q + 1);
       rec.accept_iters(n_it, lane);
       rec.accept_projections(pm, lane);
       rec.push(EV_STEP, q, c, lane);
       if (last) break;
-      n_eq++;
 
       // next factor: grid indices compare as the factors do (g_i increasing)
       int ieta = ie;
@@ -1556,8 +1583,8 @@ __device__ __forceinline__ void jt_and_theta(const MechDev &M, double *Wd, const
   for (int k = 0; k < KS; ++k)
     if (own[k]) Wd[M.a_MU + lane + WARP * k] = v[k];
   __syncwarp();
-  run_prog<double, false, false, true, false>(M.nudot_ops, M.nudot_runs, M.nudot_nruns, M.nudot_npass, Wd, lane);
-  run_prog<double, false, false, true, false>(M.jt_ops, M.jt_runs, M.jt_nruns, M.jt_npass, Wd, lane);
+  run_prog<double, false, true, false>(M.nudot_ops, M.nudot_runs, M.nudot_nruns, M.nudot_npass, Wd, lane);
+  run_prog<double, false, true, false>(M.jt_ops, M.jt_runs, M.jt_nruns, M.jt_npass, Wd, lane);
   for (int j = lane; j < M.R; j += WARP) Wd[M.a_G + j] = fma(scale * Wd[M.d_RT + j], Wd[M.a_NM + j], Wd[M.a_G + j]);
 #pragma unroll
   for (int k = 0; k < KS; ++k) out[k] = own[k] ? Wd[M.a_JTM + lane + WARP * k] : 0.0;
@@ -1671,8 +1698,8 @@ __device__ void backward_cell(const MechDev &M, const CellsDev &C, const AdjDev 
       for (int k = 0; k < KS; ++k)
         if (cl.own[k]) Wd[M.d_Y + cl.pos[k]] = lamd[k];   // the solve vector: y's slots (y was consumed)
       __syncwarp();
-      run_prog<double, false, false, false, false>(M.fwdT_ops, M.fwdT_runs, M.fwdT_nruns, M.fwdT_npass, Wd, lane);
-      run_prog<double, false, false, false, false>(M.bwdT_ops, M.bwdT_runs, M.bwdT_nruns, M.bwdT_npass, Wd, lane);
+      run_prog<double, false, false, false>(M.fwdT_ops, nullptr, 1, M.fwdT_npass, Wd, lane);
+      run_prog<double, false, false, false>(M.bwdT_ops, nullptr, 1, M.bwdT_npass, Wd, lane);
 #pragma unroll
       for (int k = 0; k < KS; ++k) g[k] = cl.own[k] ? -ss * Wd[M.d_Y + cl.pos[k]] : 0.0;   // the programs leave -M^{-T} lambda
       __syncwarp();
@@ -1803,7 +1830,7 @@ __device__ __forceinline__ void tangent_f(const MechDev &M, const Tabs &tb, doub
     Wd[M.d_RT + j] = sj;
   }
   __syncwarp();
-  run_prog<double, false, false, true, false>(tab<ushort4>(tb, M.tab.f_ops), tab<uint32_t>(tb, M.tab.f_runs), M.f_nruns,
+  run_prog<double, false, true, false>(tab<ushort4>(tb, M.tab.f_ops), tab<uint32_t>(tb, M.tab.f_runs), M.f_nruns,
                                               M.f_npass, Wd, lane);
 #pragma unroll
   for (int k = 0; k < KS; ++k) out[k] = own[k] ? Wd[M.d_F + lane + WARP * k] : 0.0;

@@ -36,7 +36,7 @@ namespace {
 // finish() then packs the recorded graph afresh by list scheduling: pass by
 // pass it takes the ready ops with the longest remaining dependency chain
 // first (a reciprocal weighs RECIP_WEIGHT, the FP64 instructions of its pass),
-// and a pass holds reciprocals only when the most urgent ready op is one.
+// and a unit holds reciprocals only when the most urgent ready op is one.
 struct Scheduler {
   static constexpr int RECIP_WEIGHT = 4;
   std::vector<int> lastw, lastr;
@@ -130,17 +130,32 @@ struct Scheduler {
         pass.push_back(ready[k].top());
         ready[k].pop();
       }
-      // wide: a pass of reciprocals takes the most urgent ready FMAs into its
-      // other lanes (the kernels run such a pass as one mixed op per lane)
-      while (wide && k == 1 && !ready[0].empty() && pass.size() < (size_t)WARP) {
-        pass.push_back(ready[0].top());
-        ready[0].pop();
+      // A reciprocal costs its lane three FP64 instructions, and so the warp:
+      // its unit is three passes, the lanes without a reciprocal running an FMA
+      // op in each (the most urgent ready ones, all independent of each other),
+      // the lanes with one leaving their slots of the second and third empty
+      if (k == 1) {
+        const size_t nr = pass.size();
+        std::vector<int> all = pass;
+        for (int sub = 0; sub < 3; ++sub) {
+          std::vector<int> fill;
+          while (!ready[0].empty() && fill.size() + nr < (size_t)WARP) {
+            fill.push_back(ready[0].top());
+            ready[0].pop();
+          }
+          for (size_t i = 0; i < nr; ++i) hp.ops.push_back(sub == 0 ? rec_op[pass[i]] : Op{OP_EMPTY, 0, 0, 0});
+          for (int i : fill) hp.ops.push_back(rec_op[i]);
+          for (size_t i = nr + fill.size(); i < (size_t)WARP; ++i) hp.ops.push_back(Op{OP_EMPTY, 0, 0, 0});
+          hp.unit.push_back(sub == 0 ? 3 : 0);
+          all.insert(all.end(), fill.begin(), fill.end());
+        }
+        pass = std::move(all);
+      } else {
+        for (int i : pass) hp.ops.push_back(rec_op[i]);
+        for (size_t i = pass.size(); i < width; ++i) hp.ops.push_back(Op{OP_EMPTY, 0, 0, 0});
+        if (width == WARP) hp.unit.push_back(0);
+        else hp.unit.insert(hp.unit.end(), {1, 2});
       }
-      for (int i : pass) hp.ops.push_back(rec_op[i]);
-      for (size_t i = pass.size(); i < (size_t)WARP; ++i) hp.ops.push_back(Op{OP_EMPTY, 0, 0, 0});
-      if (k == 1) hp.unit.push_back(3);
-      else if (width == WARP) hp.unit.push_back(0);
-      else hp.unit.insert(hp.unit.end(), {1, 2});
       done += (int)pass.size();
       for (int i : pass)
         for (int s2 : succ[i])
@@ -185,28 +200,17 @@ uint32_t xorshift(uint32_t &s) {
 }
 
 // element of role r (0 t, 1 a, 2 b, 3 c) of an op as the device runs it (-1: no access)
-int role_elem(const Op &o, bool recip, int r, int dummy, int zero, int one) {
-  if (o.t == OP_EMPTY) {
-    if (recip) return r == 0 ? dummy : r == 1 ? one : -1;
-    return r == 0 ? dummy : zero;
-  }
+int role_elem(const Op &o, int r, int dummy, int zero) {
+  if (o.t == OP_EMPTY) return r == 0 ? dummy : zero;
   if (o.t & OP_RECIP) return r == 0 ? (o.t & 0x7fff) : r == 1 ? o.a : -1;
   return r == 0 ? o.t : r == 1 ? o.a : r == 2 ? o.b : o.c;
-}
-
-bool recip_pass(const HostProgram &hp, int p) {
-  for (int l = 0; l < WARP; ++l) {
-    const Op &o = hp.ops[(size_t)p * WARP + l];
-    if (o.t != OP_EMPTY && (o.t & OP_RECIP)) return true;
-  }
-  return false;
 }
 
 // The slot search: a permutation of the slots [0, n_perm) (perm[e] = new
 // position of e), improved in place.  A group is the distinct slots of one
 // operand of one pass, per half-warp in the pass's current lane order (16 bank
 // pairs: position mod 16) and whole (32 banks: position mod 32).
-void bank_permutation(const std::vector<BankProg> &progs, int n_perm, int dummy, int zero, int one, long iters,
+void bank_permutation(const std::vector<BankProg> &progs, int n_perm, int dummy, int zero, long iters,
                       std::vector<int> &perm) {
   constexpr int NB = 32;
   if (n_perm < 2 * NB) return;
@@ -232,13 +236,12 @@ void bank_permutation(const std::vector<BankProg> &progs, int n_perm, int dummy,
   for (const BankProg &bp : progs) {
     const HostProgram &hp = *bp.hp;
     for (int p = 0; p < hp.n_pass(); ++p) {
-      const bool rc = recip_pass(hp, p);
       for (int r = 0; r < 4; ++r) {
         std::vector<int> whole;
         for (int h = 0; h < 2; ++h) {
           std::vector<int> half;
           for (int l = 16 * h; l < 16 * h + 16; ++l) {
-            const int e = role_elem(hp.ops[(size_t)p * WARP + l], rc, r, dummy, zero, one);
+            const int e = role_elem(hp.ops[(size_t)p * WARP + l], r, dummy, zero);
             if (e >= 0) half.push_back(e);
           }
           whole.insert(whole.end(), half.begin(), half.end());
@@ -317,13 +320,12 @@ int half_cost(const std::vector<int> (&el)[4], const std::vector<int> &lane_op) 
 }
 
 // The lane search over every pass of hp.
-void bank_lanes(HostProgram &hp, int dummy, int zero, int one) {
+void bank_lanes(HostProgram &hp, int dummy, int zero) {
   for (int p = 0; p < hp.n_pass(); ++p) {
-    const bool rc = recip_pass(hp, p);
     Op *ops = &hp.ops[(size_t)p * WARP];
     std::vector<int> el[4];
     for (int r = 0; r < 4; ++r)
-      for (int l = 0; l < WARP; ++l) el[r].push_back(role_elem(ops[l], rc, r, dummy, zero, one));
+      for (int l = 0; l < WARP; ++l) el[r].push_back(role_elem(ops[l], r, dummy, zero));
     std::vector<int> lane_op(WARP);
     for (int l = 0; l < WARP; ++l) lane_op[l] = l;
     int best = half_cost(el, lane_op);
@@ -345,6 +347,24 @@ void bank_lanes(HostProgram &hp, int dummy, int zero, int one) {
     Op tmp[WARP];
     for (int l = 0; l < WARP; ++l) tmp[l] = ops[lane_op[l]];
     for (int l = 0; l < WARP; ++l) ops[l] = tmp[l];
+  }
+  // a reciprocal's lane has no op in the two passes after it (its unit): move
+  // those passes' empty slots there, within the half-warp where one is
+  auto is_recip = [](const Op &o) { return o.t != OP_EMPTY && (o.t & OP_RECIP); };
+  for (int p = 0; p < hp.n_pass(); ++p) {
+    if (hp.unit[p] != 3) continue;
+    const Op *rop = &hp.ops[(size_t)p * WARP];
+    for (int sub = 1; sub < 3; ++sub) {
+      Op *ops = &hp.ops[(size_t)(p + sub) * WARP];
+      for (int l = 0; l < WARP; ++l) {
+        if (!is_recip(rop[l]) || ops[l].t == OP_EMPTY) continue;
+        int to = -1;
+        for (int pref = 0; pref < 2 && to < 0; ++pref)
+          for (int x = 0; x < WARP && to < 0; ++x)
+            if (!is_recip(rop[x]) && ops[x].t == OP_EMPTY && (pref == 1 || (x < 16) == (l < 16))) to = x;
+        std::swap(ops[l], ops[to]);      // one exists: the pass holds at most WARP - reciprocals ops
+      }
+    }
   }
 }
 
@@ -854,16 +874,15 @@ int compile_mechanism(int S, int R, const chem_reaction *rx, Mechanism &m, std::
   }
   // ---- bank layout (see bank_permutation): the LU slots, then every pass's lanes
   {
-    const int L_ONE = d.L_ZERO + 1;
     // weights: runs per formation of M (about 4.6 Newton solves per factorisation
     // on the 72/186 workload; the adjoint's transposed solves once per iteration walked)
     const std::vector<BankProg> bp = {{&m.m_prog, 1.0},   {&m.lu_prog, 1.0},   {&m.fwd_prog, 4.6},
                                       {&m.bwd_prog, 4.6}, {&m.fwdT_prog, 1.0}, {&m.bwdT_prog, 1.0}};
     // lanes for the slots as numbered, then the permutation for those lanes, then the lanes again
-    for (const BankProg &b : bp) bank_lanes(*b.hp, d.L_DUMMY, d.L_ZERO, L_ONE);
+    for (const BankProg &b : bp) bank_lanes(*b.hp, d.L_DUMMY, d.L_ZERO);
     std::vector<int> perm(nnz);
     for (int e = 0; e < nnz; ++e) perm[e] = e;
-    bank_permutation(bp, nnz, d.L_DUMMY, d.L_ZERO, L_ONE, std::min<long>(700L * nnz, 2000000L), perm);
+    bank_permutation(bp, nnz, d.L_DUMMY, d.L_ZERO, std::min<long>(700L * nnz, 2000000L), perm);
     auto remap = [&](uint16_t &f) {
       if (f < nnz) f = (uint16_t)perm[f];
     };
@@ -883,8 +902,8 @@ int compile_mechanism(int S, int R, const chem_reaction *rx, Mechanism &m, std::
         }
       }
     for (int &x : m.lu_diag) x = d.L_LU + perm[x - d.L_LU];
-    for (const BankProg &b : bp) bank_lanes(*b.hp, d.L_DUMMY, d.L_ZERO, L_ONE);
-    bank_lanes(m.f_prog, d.d_DUMMY, d.d_ZERO, d.d_ONE);
+    for (const BankProg &b : bp) bank_lanes(*b.hp, d.L_DUMMY, d.L_ZERO);
+    bank_lanes(m.f_prog, d.d_DUMMY, d.d_ZERO);
   }
   m.rx_slot_idx.assign((size_t)R * 3, d.d_ONE);
   for (int j = 0; j < R; ++j)
@@ -906,38 +925,23 @@ int put(Mechanism &m, const std::vector<T> &v, const T **dst, std::string &msg) 
   return 0;
 }
 
-// Device form of a program: byte offsets (off(element index)), empty slots
-// as FMAs into the dummy slot (in a pass with reciprocals: a reciprocal of one
-// into it), RECIP ops marked by c == DEV_RECIP.
+// Device form of a program: byte offsets (off(element index)), empty slots as
+// FMAs into the dummy slot, RECIP ops marked by c == DEV_RECIP.
 template <typename Off>
-std::vector<ushort4> device_ops_at(const HostProgram &hp, Off off, int dummy, int zero, int one) {
+std::vector<ushort4> device_ops_at(const HostProgram &hp, Off off, int dummy, int zero) {
   std::vector<ushort4> v(hp.ops.size());
-  const int np = hp.n_pass();
-  for (int p = 0; p < np; ++p) {
-    bool recip = false;
-    for (int l = 0; l < WARP; ++l) {
-      const Op &o = hp.ops[(size_t)p * WARP + l];
-      if (o.t != OP_EMPTY && (o.t & OP_RECIP)) recip = true;
-    }
-    for (int l = 0; l < WARP; ++l) {
-      const Op &o = hp.ops[(size_t)p * WARP + l];
-      ushort4 &d = v[(size_t)p * WARP + l];
-      if (o.t == OP_EMPTY) {
-        d = recip ? make_ushort4(off(dummy), off(one), 0, DEV_RECIP)
-                  : make_ushort4(off(dummy), off(zero), off(zero), off(zero));
-      } else if (o.t & OP_RECIP) {
-        d = make_ushort4(off(o.t & 0x7fff), off(o.a), 0, DEV_RECIP);
-      } else {
-        d = make_ushort4(off(o.t), off(o.a), off(o.b), off(o.c));
-      }
-    }
+  for (size_t i = 0; i < v.size(); ++i) {
+    const Op &o = hp.ops[i];
+    if (o.t == OP_EMPTY) v[i] = make_ushort4(off(dummy), off(zero), off(zero), off(zero));
+    else if (o.t & OP_RECIP) v[i] = make_ushort4(off(o.t & 0x7fff), off(o.a), 0, DEV_RECIP);
+    else v[i] = make_ushort4(off(o.t), off(o.a), off(o.b), off(o.c));
   }
   return v;
 }
 
 // ... with byte offsets elem * index from the program's own array
-std::vector<ushort4> device_ops(const HostProgram &hp, int elem, int dummy, int zero, int one) {
-  return device_ops_at(hp, [elem](int e) { return (unsigned short)(e * elem); }, dummy, zero, one);
+std::vector<ushort4> device_ops(const HostProgram &hp, int elem, int dummy, int zero) {
+  return device_ops_at(hp, [elem](int e) { return (unsigned short)(e * elem); }, dummy, zero);
 }
 
 // polynomial coefficients (in eta) of R(eta)_{jm} = prod_{l<m} (l - j eta)/(l+1)
@@ -1009,7 +1013,7 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
     const int el = prec == 0 ? 8 : 4;     // bytes per WL element
     BlobWriter bw;
     TableOffsets t;
-    t.f_ops = bw.add(device_ops(m.f_prog, 8, d.d_DUMMY, d.d_ZERO, d.d_ONE));
+    t.f_ops = bw.add(device_ops(m.f_prog, 8, d.d_DUMMY, d.d_ZERO));
     t.f_runs = bw.add(m.f_prog.runs());
     // the M and solve programs run on the whole per-cell slice: WL slots after Wd
     // (rounded to an even length), the pair products in Wd from the rates' first
@@ -1020,9 +1024,9 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
                               : e >= X_VIRTUAL ? x_off + (e - X_VIRTUAL) * el
                                                : wl_off + e * el);
     };
-    const std::vector<ushort4> m_dev = device_ops_at(m.m_prog, coff, d.L_DUMMY, d.L_ZERO, d.L_ZERO + 1);
-    t.fwd_ops = bw.add(device_ops_at(m.fwd_prog, coff, d.L_DUMMY, d.L_ZERO, d.L_ZERO + 1));
-    t.bwd_ops = bw.add(device_ops_at(m.bwd_prog, coff, d.L_DUMMY, d.L_ZERO, d.L_ZERO + 1));
+    const std::vector<ushort4> m_dev = device_ops_at(m.m_prog, coff, d.L_DUMMY, d.L_ZERO);
+    t.fwd_ops = bw.add(device_ops_at(m.fwd_prog, coff, d.L_DUMMY, d.L_ZERO));
+    t.bwd_ops = bw.add(device_ops_at(m.bwd_prog, coff, d.L_DUMMY, d.L_ZERO));
     std::vector<uint2> slots(R);
     for (int j = 0; j < R; ++j)
       slots[j] = make_uint2((unsigned)(m.rx_slot_idx[j * 3] * 8) | ((unsigned)(m.rx_slot_idx[j * 3 + 1] * 8) << 16),
@@ -1052,7 +1056,7 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
     d.tab = t;
     int rc = put(m, bw.buf, &d.blob[prec], msg);
     if (!rc) rc = put(m, m_dev, &d.m_ops[prec], msg);
-    if (!rc) rc = put(m, device_ops(m.lu_prog, el, d.L_DUMMY, d.L_ZERO, d.L_ZERO + 1), &d.lu_ops[prec], msg);
+    if (!rc) rc = put(m, device_ops(m.lu_prog, el, d.L_DUMMY, d.L_ZERO), &d.lu_ops[prec], msg);
     if (!rc && prec == 0) rc = put(m, m.m_prog.runs(), &d.m_runs, msg);
     if (!rc && prec == 0) rc = put(m, m.lu_prog.runs(), &d.lu_runs, msg);
     if (rc) {
@@ -1068,12 +1072,11 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
     std::vector<int> aoff(m.a_consts_i.size());
     for (size_t k = 0; k < aoff.size(); ++k) aoff[k] = m.a_consts_i[k] * 8;
     if ((rc = put(m, aoff, &d.a_const_off, msg)) || (rc = put(m, m.a_consts_v, &d.a_const_val, msg)) ||
-        (rc = put(m, device_ops(m.nudot_prog, 8, d.d_DUMMY, d.d_ZERO, d.d_ONE), &d.nudot_ops, msg)) ||
-        (rc = put(m, device_ops(m.jt_prog, 8, d.d_DUMMY, d.d_ZERO, d.d_ONE), &d.jt_ops, msg)) ||
-        (rc = put(m, device_ops_at(m.fwdT_prog, xoff64, d.L_DUMMY, d.L_ZERO, d.L_ZERO + 1), &d.fwdT_ops, msg)) ||
-        (rc = put(m, device_ops_at(m.bwdT_prog, xoff64, d.L_DUMMY, d.L_ZERO, d.L_ZERO + 1), &d.bwdT_ops, msg)) ||
-        (rc = put(m, m.nudot_prog.runs(), &d.nudot_runs, msg)) || (rc = put(m, m.jt_prog.runs(), &d.jt_runs, msg)) ||
-        (rc = put(m, m.fwdT_prog.runs(), &d.fwdT_runs, msg)) || (rc = put(m, m.bwdT_prog.runs(), &d.bwdT_runs, msg))) {
+        (rc = put(m, device_ops(m.nudot_prog, 8, d.d_DUMMY, d.d_ZERO), &d.nudot_ops, msg)) ||
+        (rc = put(m, device_ops(m.jt_prog, 8, d.d_DUMMY, d.d_ZERO), &d.jt_ops, msg)) ||
+        (rc = put(m, device_ops_at(m.fwdT_prog, xoff64, d.L_DUMMY, d.L_ZERO), &d.fwdT_ops, msg)) ||
+        (rc = put(m, device_ops_at(m.bwdT_prog, xoff64, d.L_DUMMY, d.L_ZERO), &d.bwdT_ops, msg)) ||
+        (rc = put(m, m.nudot_prog.runs(), &d.nudot_runs, msg)) || (rc = put(m, m.jt_prog.runs(), &d.jt_runs, msg))) {
       free_mechanism(m);
       return rc;
     }
@@ -1084,8 +1087,6 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
     d.bwdT_npass = m.bwdT_prog.n_pass();
     d.nudot_nruns = (int)m.nudot_prog.runs().size();
     d.jt_nruns = (int)m.jt_prog.runs().size();
-    d.fwdT_nruns = (int)m.fwdT_prog.runs().size();
-    d.bwdT_nruns = (int)m.bwdT_prog.runs().size();
   }
   d.f_npass = m.f_prog.n_pass();
   d.f_nruns = (int)m.f_prog.runs().size();
