@@ -210,13 +210,18 @@ int chem_cells_create(const chem_mech *mech, int64_t n_cells, const chem_opts *o
     if (o.record_adjoint) return fail(CHEM_EINVAL, "coupled cells have no adjoint");
     const int wmax = max_warps_per_block(mech->m.dev, o.lu_precision, o.driver);
     if (o.couple_cells > wmax) return fail(CHEM_EINVAL, "couple_cells exceeds the cells a block can hold");
-    if (o.cells_per_block == 0) o.cells_per_block = (wmax / o.couple_cells) * o.couple_cells;   // whole groups per block
     if (o.cells_per_block % o.couple_cells) return fail(CHEM_EINVAL, "cells_per_block must be a multiple of couple_cells");
   }
   const int wmax = max_warps_per_block(mech->m.dev, o.lu_precision, o.driver);
   if (wmax < 1) return fail(CHEM_EINVAL, "mechanism working set does not fit in shared memory");
   if (o.cells_per_block > wmax) return fail(CHEM_EINVAL, "cells_per_block exceeds the shared-memory limit");
-  if (o.cells_per_block == 0) o.cells_per_block = best_warps_per_block(mech->m.dev, o.lu_precision, o.driver);
+  if (o.cells_per_block == 0) {
+    if (o.blocks_per_sm > 0)
+      o.cells_per_block = o.couple_cells > 1 ? (wmax / o.couple_cells) * o.couple_cells   // whole groups per block
+                                             : best_warps_per_block(mech->m.dev, o.lu_precision, o.driver);
+    else
+      auto_shape(mech->m.dev, o.lu_precision, o.driver, o.couple_cells, n_cells, &o.cells_per_block, &o.blocks_per_sm);
+  }
   if (o.cells_per_block < 1) return fail(CHEM_EINVAL, "no launch shape fits on this device");
   if (o.record_adjoint && o.lu_precision != 64)
     return fail(CHEM_EINVAL, "record_adjoint needs lu_precision 64 (the adjoint differentiates the FP64 iteration)");

@@ -2417,12 +2417,7 @@ int best_warps_per_block(const MechDev &M, int lu_precision, int driver) {
   // block against 64.1 ms at 11).
   if (!staged_driver(driver)) return (wmax >= 1 && occupancy(M, lu_precision, driver, 1) >= 1) ? 1 : 0;
   // The persistent driver stages the tables once per block: most resident
-  // cells per SM, ties to the larger block.  (The walks' narrow-batch bound
-  // was measured here too: a single first solve of 1,024 / 2,048 cells of the
-  // 72/186 mechanism gains 10% / 8% at 8 cells per SM, but the four recorded
-  // steps of the 2,048-cell differentiation workload lose 3%, 15.9 -> 16.4
-  // ms: after the first step the queue is keyed by exact costs and the
-  // throughput of the full occupancy wins.)
+  // cells per SM, ties to the larger block.
   int best_w = 0, best_cells = 0;
   for (int w = 1; w <= wmax; ++w) {
     const int cells = w * occupancy(M, lu_precision, driver, w);
@@ -2432,6 +2427,32 @@ int best_warps_per_block(const MechDev &M, int lu_precision, int driver) {
     }
   }
   return best_w;
+}
+
+// Launch shape of a batch whose caller gave none.  The persistent driver fills
+// the SMs with best_warps_per_block cells each; a batch with fewer cells than
+// that (coupled: whole groups) spreads evenly instead, one block of
+// ceil(units / SMs) cells or groups on every SM, since a cell runs the faster
+// the fewer share its SM (72/186, first solve of 301 cells: 5.5 ms against
+// 7.3 ms as 26 full blocks of 12; 1,824 cells fill every SM either way).
+// Between one and two cells per resident warp the full occupancy stays: 8
+// cells per SM gain 8% on a first solve of 2,048 cells but lose 3% on four
+// consecutive steps, whose queue is keyed by exact costs.
+void auto_shape(const MechDev &M, int lu_precision, int driver, int couple, int64_t n_cells, int *warps_per_block,
+                int *blocks_per_sm) {
+  const int full = couple > 1 ? (max_warps_per_block(M, lu_precision, driver) / couple) * couple
+                              : best_warps_per_block(M, lu_precision, driver);
+  *warps_per_block = full;
+  if (!staged_driver(driver) || full < 1) return;
+  int dev = 0, n_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  if (n_sm < 1) return;
+  const int64_t units = (n_cells + couple - 1) / couple;
+  const int64_t w = (units + n_sm - 1) / n_sm * couple;
+  if (w < 1 || w >= full) return;
+  *warps_per_block = (int)w;
+  *blocks_per_sm = 1;
 }
 
 cudaError_t launch_probe(const MechDev &M, const CellsDev &C, int lu_precision, int mode, double c, const double *y,
