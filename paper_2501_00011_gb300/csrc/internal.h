@@ -66,6 +66,12 @@ struct TableOffsets {
 
 constexpr int RX_EXT = 8;   // extra rate parameters per reaction
 
+// Terms of the tile derivative (MechDev::tl_term): coefficient +1, -1, another
+constexpr uint32_t TILE_PLUS = 0, TILE_MINUS = 1, TILE_GENERAL = 2;
+constexpr int TILE_CHUNK = 8;     // terms per chunk: the f program's
+constexpr int TILE_WARPS = 12;    // warps per group of the tile derivative
+constexpr int TILE_GROUPS = 2;    // groups per block
+
 // Everything a solve kernel needs about a mechanism; passed by value.
 struct MechDev {
   int S, R, max_reac, n_phot, n_pairs;
@@ -81,6 +87,18 @@ struct MechDev {
   const chem_reaction *rx_aos;
   const int *rx_reac, *rx_nprod, *rx_prod;
   const double *rx_yld;
+  // f for tiles of 32 cells, one lane per cell (deriv_gather_kernel): the
+  // reactions by their number of reactants; per species the terms of its sum in
+  // the f program's order (reaction | TILE_* << 16) with their coefficients; the
+  // species dealt to the block's warps
+  const uint2 *tl_rx;      // [R] reactions with 1, then 2, then 3 reactants: j | r0 << 16, r1 | r2 << 16
+  int tl_rx_end[3];        // ends of those three ranges
+  const uint32_t *tl_term; // (two words past the last term are readable)
+  const double *tl_nu;     // read for TILE_GENERAL terms
+  const int *tl_ptr;       // [S + 1] first term of each species
+  const int *tl_list;      // [S] species, warp by warp
+  const int *tl_warp;      // [TILE_WARPS + 1] first entry of each warp in tl_list
+  int tl_cost, ga_cost;    // FP64 warp instructions per tile, and per cell by the f program
   // species permutation: position of species s in the pivot order
   const int *sp_pos;       // [S]
   // per-cell double array Wd (element indices)
@@ -165,6 +183,7 @@ struct Mechanism {
   std::vector<std::pair<int, int>> pair_other;   // Wd element indices
   std::vector<int> lu_diag;                      // WL element indices
   std::vector<int> rx_slot_idx;                  // [R][3] Wd element indices of the reactants' y
+  std::vector<std::vector<std::pair<double, int>>> f_terms;   // f_i = sum nu_ij r_j: (nu, j) in the f program's order
   std::vector<chem_reaction> rx;
   MechDev dev{};                     // device pointers filled in upload()
   std::vector<void *> allocations;   // device buffers owned

@@ -103,6 +103,7 @@ __device__ __forceinline__ void cp_async8(uint32_t dst, const void *src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // A lane's op as shared addresses: the work array's base plus the op's byte
 // offsets (packed op: x = t | a << 16, y = b | c << 16).
@@ -335,6 +336,14 @@ __device__ __forceinline__ double warp_min(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(FULL, v, o));
   return v;
+}
+
+// An FMA that stays one (the compiler would turn a factor 1 into an add) and is
+// not executed ahead of the branch it stands in.
+__device__ __forceinline__ double fma_now(double a, double b, double c) {
+  double d;
+  asm volatile("fma.rn.f64 %0, %1, %2, %3;" : "=d"(d) : "d"(a), "d"(b), "d"(c));
+  return d;
 }
 
 // Comparisons of non-negative doubles on the integer pipe.  FP64 compares,
@@ -2292,49 +2301,189 @@ cudaError_t launch_order_t(const MechDev &M, const CellsDev &C, const SolveParam
 }
 
 // ----------------------------------------------------- derivative only
-// a2 for every cell with the rate constants given (kt[R][C]): a block of
-// GATHER_CELLS cells copies the hot table prefix into shared memory, reads its
-// y and k~ tiles with the cells fastest (coalesced), transposes them into the
-// cells' Wd slices, runs the rates and the f program one warp per cell, and
-// writes f back the same way.
-constexpr int GATHER_CELLS = 16;
+// a2 for every cell with the rate constants given (kt[R][C]).  The FP64 unit
+// bounds it, so what counts is FP64 warp instructions per cell and their even
+// spread over the SMs: one block per SM, its warps in two groups that run side
+// by side:
+//   tiles   two groups of TILE_WARPS warps take 32 cells at a time each, one lane
+//           per cell: they bring y and k~ into shared memory, form the rates
+//           there, then each warp sums its species' terms in the f program's
+//           order (chunks of 8, added up in order: the same bits).  The groups run
+//           apart, so one's loads and barriers pass under the other's FMAs (one
+//           group of 16 warps with two buffers: 25.2 us for 10,000 cells).  Every
+//           lane works, and the first term of a chunk with coefficient +-1 costs
+//           nothing: 72/186 spends 946 FP64 instructions per tile, 30 per cell, so
+//           10,000 cells need 14.7 us.
+//   gather  more warps run the compiled f program, one warp per cell (36
+//           instructions): the cells beyond the last whole round of one tile per
+//           SM, spread over the SMs, and batches too small for tiles.
+// 10,000 cells: 24.9 us a call against 38.9 us with every cell by the gather in
+// blocks of 16 cells.
+constexpr int TILE_CELLS = WARP;
+constexpr int GATHER_BAR = 1, TILE_BAR = 2;     // named barriers: the gather warps, the first tile group
+constexpr int GATHER_WARPS = 16;                // most gather warps of a block
 
-template <int KS>
-__global__ void __launch_bounds__(GATHER_CELLS * WARP) deriv_gather_kernel(const __grid_constant__ MechDev M, const int64_t NC,
-                                                                             const double *kt, const double *y, double *f,
-                                                                             const int cell_doubles) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  // the hot table prefix (f program, reactant slots), then the cells' slices
-  const int tb = M.tab.staged;
-  for (int i = threadIdx.x; i < tb / 16; i += blockDim.x)
-    reinterpret_cast<uint4 *>(smem)[i] = __ldg(reinterpret_cast<const uint4 *>(M.blob[0]) + i);
-  double *sm = reinterpret_cast<double *>(smem + tb);
-  const int lane = threadIdx.x & (WARP - 1);
-  const int warp = threadIdx.x / WARP;
-  const int64_t c0 = (int64_t)blockIdx.x * GATHER_CELLS;
-  const int nb = (int)((NC - c0) < GATHER_CELLS ? (NC - c0) : GATHER_CELLS);    // cells of this block
-  // tiles in: element (row, cell) -> slice of cell, slot row
-  for (int i = threadIdx.x; i < M.S * GATHER_CELLS; i += blockDim.x) {
-    const int r = i / GATHER_CELLS, cl = i % GATHER_CELLS;
-    if (cl < nb) sm[(size_t)cl * cell_doubles + M.d_Y + r] = y[(int64_t)r * NC + c0 + cl];
+struct DerivSplit {
+  int64_t n_tiles;         // tiles of 32 cells, dealt to the blocks in turn, then to a block's groups
+  int tile_warps;          // of a block: TILE_GROUPS * TILE_WARPS, or 0 without tiles
+  int gather_cells;        // gather warps (one cell each) per block
+  int cell_doubles;        // a gather cell's slice
+  int tile_doubles;        // a tile buffer
+};
+
+__device__ __forceinline__ void group_sync(int bar, int warps) {
+  asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(warps * WARP) : "memory");
+}
+
+// the tile's y [S][32] and k~ [R][32] into the buffer at sm, asynchronously (cells past the end: zero)
+__device__ __forceinline__ void deriv_tile_load(const MechDev &M, const int64_t NC, const int64_t c, const double *kt,
+                                                const double *y, double *sm, int lane, int warp) {
+  const uint32_t base = smem_addr(sm) + 8u * lane;
+  if (c < NC) {
+#pragma unroll 4
+    for (int i = warp; i < M.S; i += TILE_WARPS) cp_async8(base + i * (TILE_CELLS * 8u), y + (int64_t)i * NC + c);
+#pragma unroll 4
+    for (int j = warp; j < M.R; j += TILE_WARPS) cp_async8(base + (M.S + j) * (TILE_CELLS * 8u), kt + (int64_t)j * NC + c);
+  } else {
+    for (int i = warp; i < M.S + M.R; i += TILE_WARPS) sts(base + i * (TILE_CELLS * 8u), 0.0);
   }
-  for (int i = threadIdx.x; i < M.R * GATHER_CELLS; i += blockDim.x) {
-    const int r = i / GATHER_CELLS, cl = i % GATHER_CELLS;
-    if (cl < nb) sm[(size_t)cl * cell_doubles + M.d_KT + r] = kt[(int64_t)r * NC + c0 + cl];
+}
+
+__device__ __forceinline__ void deriv_tile(const MechDev &M, const int64_t NC, const int64_t c, double *f, double *sm,
+                                           int lane, int warp, int bar) {
+  const bool in = c < NC;
+  double *const ys = sm, *const rs = sm + (size_t)M.S * TILE_CELLS;      // [S][32], [R][32]
+  // (no predicated FP64 instruction: one with every lane off still takes the
+  // unit's time, so what does not apply is skipped by loop bounds)
+  const uint32_t yb = smem_addr(ys + lane), rb = smem_addr(rs + lane);
+  constexpr uint32_t ROW = TILE_CELLS * 8u;
+  double *const tag = nullptr;
+  // a product as fma(a, b, -0): the same bits, and an FP64 multiplication takes
+  // the unit 76 cycles where an FMA takes 64
+  auto mul = [](double a, double b) { return fma_now(a, b, -0.0); };
+  int e = warp;
+#pragma unroll 2
+  for (; e < M.tl_rx_end[0]; e += TILE_WARPS) {
+    const uint2 x = __ldg(M.tl_rx + e);
+    const uint32_t ra = rb + (x.x & 0xffffu) * ROW;
+    sts(ra, mul(lds(tag, ra), lds(tag, yb + (x.x >> 16) * ROW)));
+  }
+#pragma unroll 2
+  for (; e < M.tl_rx_end[1]; e += TILE_WARPS) {
+    const uint2 x = __ldg(M.tl_rx + e);
+    const uint32_t ra = rb + (x.x & 0xffffu) * ROW;
+    const double k = lds(tag, ra), y0 = lds(tag, yb + (x.x >> 16) * ROW), y1 = lds(tag, yb + (x.y & 0xffffu) * ROW);
+    sts(ra, mul(mul(k, y0), y1));
+  }
+  for (; e < M.tl_rx_end[2]; e += TILE_WARPS) {
+    const uint2 x = __ldg(M.tl_rx + e);
+    const uint32_t ra = rb + (x.x & 0xffffu) * ROW;
+    const double k = lds(tag, ra), y0 = lds(tag, yb + (x.x >> 16) * ROW), y1 = lds(tag, yb + (x.y & 0xffffu) * ROW);
+    sts(ra, mul(mul(mul(k, y0), y1), lds(tag, yb + (x.y >> 16) * ROW)));
+  }
+  group_sync(bar, TILE_WARPS);
+  const int e1 = __ldg(M.tl_warp + warp + 1);
+#pragma unroll 1
+  for (int e = __ldg(M.tl_warp + warp); e < e1; ++e) {
+    const int i = __ldg(M.tl_list + e);
+    const int k1 = __ldg(M.tl_ptr + i + 1);
+    int k = __ldg(M.tl_ptr + i);
+    double total = 0.0;
+    if (k < k1) {
+      // term k: word w, rate r; word wn of term k + 1 and the rate it names are
+      // loaded while term k's FMA runs
+      uint32_t w = __ldg(M.tl_term + k), wn = __ldg(M.tl_term + k + 1);
+      double r = lds(tag, rb + (w & 0xffffu) * ROW), rn;
+      auto advance = [&]() {
+        rn = lds(tag, rb + (wn & 0xffffu) * ROW);
+        return __ldg(M.tl_term + k + 2);
+      };
+      // one chunk up to term ke: fma(nu, r, acc) in order, nu = +-1 put together on
+      // the integer pipe; its first term, fma(+-1, r, +0), is the signed rate with
+      // -0 as +0
+      auto chunk = [&](const int ke) {
+        double acc = 0.0;
+        if ((w >> 16) != TILE_GENERAL) {
+          acc = plus0(__longlong_as_double(__double_as_longlong(r) ^ ((long long)((w >> 16) == TILE_MINUS) << 63)));
+          const uint32_t w2 = advance();
+          w = wn;
+          wn = w2;
+          r = rn;
+          ++k;
+        }
+#pragma unroll 1
+        for (; k < ke; ++k) {
+          const uint32_t w2 = advance();
+          double nu = __hiloint2double((w >> 16) == TILE_MINUS ? 0xbff00000 : 0x3ff00000, 0);
+          if ((w >> 16) == TILE_GENERAL) nu = __ldg(M.tl_nu + k);
+          acc = fma_now(nu, r, acc);
+          w = wn;
+          wn = w2;
+          r = rn;
+        }
+        return acc;
+      };
+      const double one = 1.0;
+      total = chunk(k + TILE_CHUNK < k1 ? k + TILE_CHUNK : k1);
+#pragma unroll 1
+      while (k < k1) total = fma_now(one, chunk(k + TILE_CHUNK < k1 ? k + TILE_CHUNK : k1), total);
+    }
+    if (in) f[(int64_t)i * NC + c] = total;
+  }
+}
+
+__global__ void __launch_bounds__(32 * WARP) deriv_gather_kernel(const __grid_constant__ MechDev M, const int64_t NC,
+                                                                             const double *kt, const double *y, double *f,
+                                                                             const DerivSplit D) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & (WARP - 1);
+  int warp = threadIdx.x / WARP;
+  if (warp < D.tile_warps) {
+    const int g = warp / TILE_WARPS;
+    warp -= g * TILE_WARPS;
+    double *const sm = reinterpret_cast<double *>(smem) + (size_t)g * D.tile_doubles;
+    for (int64_t t = blockIdx.x + (int64_t)g * gridDim.x; t < D.n_tiles; t += (int64_t)TILE_GROUPS * gridDim.x) {
+      const int64_t c = t * TILE_CELLS + lane;
+      deriv_tile_load(M, NC, c, kt, y, sm, lane, warp);
+      cp_async_wait_all();
+      group_sync(TILE_BAR + g, TILE_WARPS);
+      deriv_tile(M, NC, c, f, sm, lane, warp, TILE_BAR + g);
+      group_sync(TILE_BAR + g, TILE_WARPS);
+    }
+    return;
+  }
+  warp -= D.tile_warps;
+  const int64_t c0 = D.n_tiles * TILE_CELLS + (int64_t)blockIdx.x * D.gather_cells;
+  if (c0 >= NC) return;                         // all the block's gather warps
+  const int nb = (int)((NC - c0) < D.gather_cells ? (NC - c0) : D.gather_cells);    // cells of this block
+  // the hot table prefix (f program, reactant slots), then the cells' slices
+  unsigned char *const gs = smem + (D.tile_warps ? (size_t)TILE_GROUPS * D.tile_doubles * sizeof(double) : 0);
+  const int tid = warp * WARP + lane, nt = D.gather_cells * WARP;
+  const int tb = M.tab.staged;
+  for (int i = tid; i < tb / 16; i += nt)
+    reinterpret_cast<uint4 *>(gs)[i] = __ldg(reinterpret_cast<const uint4 *>(M.blob[0]) + i);
+  double *sm = reinterpret_cast<double *>(gs + tb);
+  // element (row, cell) -> slice of cell, slot row
+  for (int i = tid; i < M.S * D.gather_cells; i += nt) {
+    const int r = i / D.gather_cells, cl = i % D.gather_cells;
+    if (cl < nb) sm[(size_t)cl * D.cell_doubles + M.d_Y + r] = y[(int64_t)r * NC + c0 + cl];
+  }
+  for (int i = tid; i < M.R * D.gather_cells; i += nt) {
+    const int r = i / D.gather_cells, cl = i % D.gather_cells;
+    if (cl < nb) sm[(size_t)cl * D.cell_doubles + M.d_KT + r] = kt[(int64_t)r * NC + c0 + cl];
   }
   if (warp < nb) {
-    double *Wd = sm + (size_t)warp * cell_doubles;
-    unsigned char *wd = reinterpret_cast<unsigned char *>(Wd);
+    unsigned char *wd = reinterpret_cast<unsigned char *>(sm + (size_t)warp * D.cell_doubles);
     const unsigned char *gb = M.blob[0];
     for (int k = lane; k < M.d_nconst; k += WARP)
       at<double>(wd, reinterpret_cast<const int *>(gb + M.tab.dconst_off)[k]) = reinterpret_cast<const double *>(gb + M.tab.dconst_val)[k];
   }
-  __syncthreads();
-  if (warp < nb) f_core<true>(M, smem, sm + (size_t)warp * cell_doubles, lane);
-  __syncthreads();
-  for (int i = threadIdx.x; i < M.S * GATHER_CELLS; i += blockDim.x) {
-    const int r = i / GATHER_CELLS, cl = i % GATHER_CELLS;
-    if (cl < nb) f[(int64_t)r * NC + c0 + cl] = sm[(size_t)cl * cell_doubles + M.d_F + r];
+  group_sync(GATHER_BAR, D.gather_cells);
+  if (warp < nb) f_core<true>(M, gs, sm + (size_t)warp * D.cell_doubles, lane);
+  group_sync(GATHER_BAR, D.gather_cells);
+  for (int i = tid; i < M.S * D.gather_cells; i += nt) {
+    const int r = i / D.gather_cells, cl = i % D.gather_cells;
+    if (cl < nb) f[(int64_t)r * NC + c0 + cl] = sm[(size_t)cl * D.cell_doubles + M.d_F + r];
   }
 }
 
@@ -2566,21 +2715,49 @@ cudaError_t launch_tangent(const MechDev &M, const CellsDev &C, const TanDev &A,
 cudaError_t launch_deriv_gather(const MechDev &M, const CellsDev &C, const double *kt, const double *y, double *f,
                                 cudaStream_t stream) {
   if (C.n_cells <= 0) return cudaSuccess;
-  const int cell_doubles = (M.Wd_len + 1) & ~1;
-  const size_t smem = (size_t)M.tab.staged + (size_t)cell_doubles * sizeof(double) * GATHER_CELLS;
-  cudaError_t e;
-  const unsigned blocks = (unsigned)((C.n_cells + GATHER_CELLS - 1) / GATHER_CELLS);
-  switch ((M.S + WARP - 1) / WARP) {
-#define CHEM_GATHER_CASE(K_)                                                                                      \
-    case K_:                                                                                                      \
-      if ((e = allow_max_smem<deriv_gather_kernel<K_>>()) != cudaSuccess) return e;                          \
-      deriv_gather_kernel<K_><<<blocks, GATHER_CELLS * WARP, smem, stream>>>(M, C.n_cells, kt, y, f, cell_doubles); \
-      break;
-    CHEM_GATHER_CASE(1) CHEM_GATHER_CASE(2) CHEM_GATHER_CASE(3) CHEM_GATHER_CASE(4)
-#undef CHEM_GATHER_CASE
-    default:
-      return cudaErrorInvalidValue;
+  int dev = 0, n_sm = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (n_sm < 1) return cudaErrorInvalidValue;
+  DerivSplit D{};
+  D.cell_doubles = (M.Wd_len + 1) & ~1;
+  D.tile_doubles = (M.S + M.R) * TILE_CELLS;
+  const long avail = (long)optin;
+  const size_t tile_smem = (size_t)TILE_GROUPS * D.tile_doubles * sizeof(double);
+  auto gather_fit = [&](size_t used) {          // gather cells that fit beside `used` bytes
+    const long fit = (avail - (long)used - (long)M.tab.staged) / (long)(D.cell_doubles * sizeof(double));
+    const int warps = used ? 32 - TILE_GROUPS * TILE_WARPS : GATHER_WARPS;
+    return fit < 0 ? 0 : fit < warps ? (int)fit : warps;
+  };
+  // whole rounds of one tile per SM; the cells beyond them one gather warp each
+  // where they fit and cost less than another round, else as tiles
+  const int64_t round = (int64_t)n_sm * TILE_CELLS;
+  int64_t blocks = n_sm;
+  if (tile_smem <= (size_t)avail) {
+    D.n_tiles = C.n_cells / round * n_sm;
+    const int64_t per_sm = (C.n_cells - D.n_tiles * TILE_CELLS + n_sm - 1) / n_sm;
+    if (per_sm > gather_fit(D.n_tiles > 0 ? tile_smem : 0) || per_sm * M.ga_cost >= M.tl_cost)
+      D.n_tiles = (C.n_cells + TILE_CELLS - 1) / TILE_CELLS;
   }
+  D.tile_warps = D.n_tiles > 0 ? TILE_GROUPS * TILE_WARPS : 0;
+  const size_t used = D.n_tiles > 0 ? tile_smem : 0;
+  const int64_t rest = C.n_cells - D.n_tiles * TILE_CELLS;
+  if (rest > 0) {
+    const int fit = gather_fit(used);
+    if (fit < 1) return cudaErrorInvalidValue;
+    const int64_t per_sm = (rest + n_sm - 1) / n_sm;
+    D.gather_cells = (int)(per_sm < fit ? per_sm : fit);
+    const int64_t need = (rest + D.gather_cells - 1) / D.gather_cells;
+    blocks = D.n_tiles > 0 && need < n_sm ? n_sm : need;      // with tiles per_sm <= fit, so need <= n_sm
+  }
+  if (D.n_tiles > 0 && D.gather_cells == 0 && D.n_tiles < blocks) blocks = D.n_tiles;
+  const size_t smem = used + (D.gather_cells > 0
+                                  ? (size_t)M.tab.staged + (size_t)D.cell_doubles * sizeof(double) * D.gather_cells
+                                  : 0);
+  const cudaError_t e = allow_max_smem<deriv_gather_kernel>();
+  if (e != cudaSuccess) return e;
+  deriv_gather_kernel<<<(unsigned)blocks, (D.tile_warps + D.gather_cells) * WARP, smem, stream>>>(M, C.n_cells, kt, y, f, D);
   return cudaGetLastError();
 }
 

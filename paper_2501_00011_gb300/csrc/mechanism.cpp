@@ -490,7 +490,7 @@ struct ConstTable {
   }
 };
 
-constexpr int CHUNK = 8;
+constexpr int CHUNK = TILE_CHUNK;
 constexpr int X_VIRTUAL = 0x5000;   // the solve programs' name for the solve vector's slot 0 (above every WL slot)
 constexpr int P_VIRTUAL = 0x6000;   // the M program's name for pair product 0 (above every WL slot)
 constexpr int NSTMP = 16;   // temporaries of the triangular solves
@@ -646,6 +646,7 @@ int compile_mechanism(int S, int R, const chem_reaction *rx, Mechanism &m, std::
     int temp_next = d_temp;
     for (int i = 0; i < S; ++i) add_sum(sch, d.d_F + i, true, terms[i], CHUNK, temp_next, d.d_ZERO, d.d_ONE);
     m.f_prog = sch.finish(true);
+    m.f_terms = by_species;
     m.flops_f = flops;
     d.Wd_len = std::max(d_temp + n_temp, d.d_RT + n_pairs);   // the pair products' slots (8 bytes at most)
     m.d_consts_v = {1.0, 0.0};
@@ -1099,6 +1100,56 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
   d.d_nconst = (int)m.d_consts_v.size();
   d.L_nconst = (int)m.L_consts_v.size();
 
+  // tile derivative tables
+  std::vector<uint2> trx;
+  std::vector<int> tptr(1, 0), tlist, twarp;
+  std::vector<uint32_t> tterm;
+  std::vector<double> tnu;
+  {
+    d.tl_cost = 0;
+    for (int nr = 1; nr <= CHEM_MAX_REAC; ++nr) {
+      for (int j = 0; j < R; ++j)
+        if (m.rx[j].n_reac == nr)
+          trx.push_back(make_uint2((unsigned)j | (unsigned)m.rx[j].reac[0] << 16,
+                                   (nr > 1 ? (unsigned)m.rx[j].reac[1] : 0u) | (nr > 2 ? (unsigned)m.rx[j].reac[2] << 16 : 0u)));
+      d.tl_rx_end[nr - 1] = (int)trx.size();
+    }
+    for (int j = 0; j < R; ++j) d.tl_cost += m.rx[j].n_reac;
+    std::vector<std::pair<int, int>> cost(S);      // (FP64 instructions, species)
+    for (int i = 0; i < S; ++i) {
+      int c = 0;
+      for (size_t k = 0; k < m.f_terms[i].size(); ++k) {
+        const double v = m.f_terms[i][k].first;
+        const uint32_t code = v == 1.0 ? TILE_PLUS : v == -1.0 ? TILE_MINUS : TILE_GENERAL;
+        tterm.push_back((uint32_t)m.f_terms[i][k].second | code << 16);
+        tnu.push_back(v);
+        const bool first = k % TILE_CHUNK == 0;
+        c += (!first || code == TILE_GENERAL) + (first && k > 0);
+      }
+      tptr.push_back((int)tterm.size());
+      cost[i] = {c, i};
+      d.tl_cost += c;
+    }
+    tterm.resize(tterm.size() + 2, 0u);      // the kernel reads two terms ahead
+    // the longest sums first, each to the least loaded warp
+    std::sort(cost.begin(), cost.end(), [](const std::pair<int, int> &a, const std::pair<int, int> &b) {
+      return a.first != b.first ? a.first > b.first : a.second < b.second;
+    });
+    std::vector<std::vector<int>> bin(TILE_WARPS);
+    std::vector<int> load(TILE_WARPS, 0);
+    for (auto &cs : cost) {
+      const int b = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+      bin[b].push_back(cs.second);
+      load[b] += cs.first + 1;
+    }
+    for (int b = 0; b < TILE_WARPS; ++b) {
+      twarp.push_back((int)tlist.size());
+      tlist.insert(tlist.end(), bin[b].begin(), bin[b].end());
+    }
+    twarp.push_back((int)tlist.size());
+    d.ga_cost = m.f_prog.n_pass() + (R + WARP - 1) / WARP * m.max_reac;
+  }
+
   // T(eta) = U R(eta), U = R(1): coefficients of each entry as a polynomial in eta
   std::vector<double> coef(QMAX * QMAX * (QMAX + 1), 0.0);
   for (int i = 1; i <= QMAX; ++i)
@@ -1114,7 +1165,10 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
       }
     }
   int rc = 0;
-  if ((rc = put(m, kind, &d.rx_kind, msg)) || (rc = put(m, nreac, &d.rx_nreac, msg)) ||
+  if ((rc = put(m, trx, &d.tl_rx, msg)) || (rc = put(m, tterm, &d.tl_term, msg)) || (rc = put(m, tnu, &d.tl_nu, msg)) ||
+      (rc = put(m, tptr, &d.tl_ptr, msg)) ||
+      (rc = put(m, tlist, &d.tl_list, msg)) || (rc = put(m, twarp, &d.tl_warp, msg)) ||
+      (rc = put(m, kind, &d.rx_kind, msg)) || (rc = put(m, nreac, &d.rx_nreac, msg)) ||
       (rc = put(m, phot, &d.rx_phot, msg)) || (rc = put(m, A, &d.rx_A, msg)) ||
       (rc = put(m, Ea, &d.rx_Ea, msg)) || (rc = put(m, B, &d.rx_B, msg)) || (rc = put(m, J, &d.rx_J, msg)) ||
       (rc = put(m, ext, &d.rx_ext, msg)) ||
