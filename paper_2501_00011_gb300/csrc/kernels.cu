@@ -52,7 +52,31 @@ struct SolveParams {
   int couple;          // coupled group size (warps_per_block is a multiple of it); 1: independent cells
   long long stage_wait;   // iterations of the first bounded wait for the staged tables
   long long smem_bytes;   // host side: the launch's dynamic shared memory (0: tables + cells)
+  // constants the compiler must not see through (see Opaque)
+  double one = 1.0, mzero = -0.0;
+  int zero = 0;
 };
+
+// With four or more warps on an SM an FP64 add or multiplication takes a
+// sub-partition's FP64 unit 76 cycles where an FMA takes 64 (dependent chains,
+// 152 blocks of 4 to 24 warps: add 76.1, mul 76.1, fma 64.0 cycles per warp
+// instruction), so sums and products are written as FMAs with a factor 1 or an
+// addend -0, which have the same bits; the compiler would turn either back, so
+// both come from the launch parameters.  A predicated FP64 instruction takes
+// the unit's time even with every lane off, and the compiler predicates short
+// branches: CHEM_BRANCH(cond) { ... } is a loop that runs at most once, with a
+// trip count the compiler does not know, and so a real branch.
+#define CHEM_BRANCH(cond) for (int chem_br = (cond) ? 1 : 0; chem_br != 0; chem_br = P.zero)
+struct Opaque {
+  const SolveParams &P;
+  __device__ __forceinline__ double add(double a, double b) const { return fma(P.one, a, b); }
+  __device__ __forceinline__ double sub(double a, double b) const { return fma(P.one, a, -b); }
+  __device__ __forceinline__ double mul(double a, double b) const { return fma(a, b, P.mzero); }
+};
+
+// -x and |x| on the integer pipe (as FP64 instructions they cost what an add does)
+__device__ __forceinline__ double neg_i(double x) { return __hiloint2double(__double2hiint(x) ^ (int)0x80000000, __double2loint(x)); }
+__device__ __forceinline__ double abs_i(double x) { return __hiloint2double(__double2hiint(x) & 0x7fffffff, __double2loint(x)); }
 
 // Reciprocal from the hardware estimate r (relative error e = 1 - x r of
 // about 2^-23) refined by one cubically convergent Newton-Raphson step
@@ -135,9 +159,10 @@ struct RecipUnit<double> {
     const double a3 = lds(tag, v.a), b3 = lds(tag, v.b), c3 = lds(tag, v.c);
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    p1 = fma(rcp ? -x : x, rcp ? r : b, rcp ? 1.0 : c);
+    const double nr = neg_i(r);
+    p1 = fma(rcp ? nr : x, rcp ? x : b, rcp ? 1.0 : c);
     p2 = fma(rcp ? p1 : a2, rcp ? p1 : b2, rcp ? p1 : c2);
-    p3 = fma(rcp ? -r : a3, rcp ? p2 : b3, rcp ? -r : c3);
+    p3 = fma(rcp ? nr : a3, rcp ? p2 : b3, rcp ? nr : c3);
   }
   __device__ __forceinline__ void store(const OpAddr &o, const OpAddr &u, const OpAddr &v) const {
     sts(o.t, rcp ? p3 : p1);
@@ -481,58 +506,67 @@ __device__ __forceinline__ const X *gtab(const Tabs &tb, int off) {
 
 // Phase bodies that touch only the cell's shared-memory arrays and the tables.
 
-// a2: r_j = k~_j prod y, then f = the f program, from y in Wd[Y]
-template <bool STAGED>
-__device__ __forceinline__ void f_core(const MechDev &M, const unsigned char *tbase, double *Wd, const int lane) {
-  const uint2 *slots = reinterpret_cast<const uint2 *>(tbase + M.tab.rx_slots);
-  // two reactions per lane and iteration, so each lane has two products' loads in flight
-  const uint32_t wb = smem_addr(Wd), kt = wb + 8u * M.d_KT, rt = wb + 8u * M.d_RT;
+// r_j = k~_j prod y over the lane's reactions, two per iteration so that each
+// lane has two products' loads in flight.  NR: the most reactants of a reaction
+// (the mechanism's, so products that no reaction needs are not issued at all;
+// those a reaction lacks multiply by the constant 1).
+template <int NR>
+__device__ __forceinline__ void rates(const MechDev &M, const SolveParams &P, const uint2 *slots, const uint32_t wb,
+                                      const int lane) {
+  const Opaque o{P};
+  const uint32_t kt = wb + 8u * M.d_KT, rt = wb + 8u * M.d_RT;
   double *const tag = nullptr;
   int j = lane;
 #pragma unroll 1
   for (; j + WARP < M.R; j += 2 * WARP) {
     const uint2 s0 = slots[j], s1 = slots[j + WARP];
-    double r0 = lds(tag, kt + 8u * j) * lds(tag, wb + (s0.x & 0xffff));
-    double r1 = lds(tag, kt + 8u * (j + WARP)) * lds(tag, wb + (s1.x & 0xffff));
-    if (M.max_reac > 1) {
-      r0 *= lds(tag, wb + (s0.x >> 16));
-      r1 *= lds(tag, wb + (s1.x >> 16));
+    double r0 = o.mul(lds(tag, kt + 8u * j), lds(tag, wb + (s0.x & 0xffff)));
+    double r1 = o.mul(lds(tag, kt + 8u * (j + WARP)), lds(tag, wb + (s1.x & 0xffff)));
+    if (NR > 1) {
+      r0 = o.mul(r0, lds(tag, wb + (s0.x >> 16)));
+      r1 = o.mul(r1, lds(tag, wb + (s1.x >> 16)));
     }
-    if (M.max_reac > 2) {
-      r0 *= lds(tag, wb + (s0.y & 0xffff));
-      r1 *= lds(tag, wb + (s1.y & 0xffff));
+    if (NR > 2) {
+      r0 = o.mul(r0, lds(tag, wb + (s0.y & 0xffff)));
+      r1 = o.mul(r1, lds(tag, wb + (s1.y & 0xffff)));
     }
     sts(rt + 8u * j, r0);
     sts(rt + 8u * (j + WARP), r1);
   }
-  if (j < M.R) {
+#pragma unroll 1
+  for (; j < M.R; j += WARP) {
     const uint2 sl = slots[j];
-    double r = lds(tag, kt + 8u * j) * lds(tag, wb + (sl.x & 0xffff));
-    if (M.max_reac > 1) r *= lds(tag, wb + (sl.x >> 16));
-    if (M.max_reac > 2) r *= lds(tag, wb + (sl.y & 0xffff));
+    double r = o.mul(lds(tag, kt + 8u * j), lds(tag, wb + (sl.x & 0xffff)));
+    if (NR > 1) r = o.mul(r, lds(tag, wb + (sl.x >> 16)));
+    if (NR > 2) r = o.mul(r, lds(tag, wb + (sl.y & 0xffff)));
     sts(rt + 8u * j, r);
   }
+}
+
+// a2: the rates, then f = the f program, from y in Wd[Y]
+template <bool STAGED>
+__device__ __forceinline__ void f_core(const MechDev &M, const SolveParams &P, const unsigned char *tbase, double *Wd,
+                                       const int lane) {
+  const uint2 *slots = reinterpret_cast<const uint2 *>(tbase + M.tab.rx_slots);
+  const uint32_t wb = smem_addr(Wd);
+  if (M.max_reac > 2) rates<3>(M, P, slots, wb, lane);
+  else rates<2>(M, P, slots, wb, lane);
   __syncwarp();
   run_prog<double, STAGED, true, false>(reinterpret_cast<const ushort4 *>(tbase + M.tab.f_ops),
                                                reinterpret_cast<const uint32_t *>(tbase + M.tab.f_runs), M.f_nruns,
                                                M.f_npass, Wd, lane);
 }
 
-// a3-a5: M = I - c J(y) in the LU slots from y in Wd[Y], then factor
-template <typename T>
-__device__ __forceinline__ void mlu_core(const MechDev &M, const unsigned char *tbase, const int prec, double *Wd, T *WL,
-                                      const double c, const int lane) {
-  for (int i = lane; i < M.m_clear; i += WARP) WL[i] = (T)0;
-  __syncwarp();
-  unsigned char *wl = reinterpret_cast<unsigned char *>(WL);
-  unsigned char *wd = reinterpret_cast<unsigned char *>(Wd);
-  const int *diag = reinterpret_cast<const int *>(tbase + M.tab.lu_diag);
+// -c dr_j/dy_l of the lane's (reaction, reactant) pairs, two per iteration as
+// the rates; NR as there
+template <typename T, int NR>
+__device__ __forceinline__ void pair_products(const MechDev &M, const SolveParams &P, const unsigned char *tbase,
+                                              double *Wd, const double c, const int lane) {
+  const Opaque o{P};
   const int *prx = reinterpret_cast<const int *>(tbase + M.tab.pair_rx);
   const unsigned *pother = reinterpret_cast<const unsigned *>(tbase + M.tab.pair_other);
-  for (int k = lane; k < M.S; k += WARP) at<T>(wl, diag[k]) = (T)1;
-  const double mc = -c;
-  // two pairs per lane and iteration (loads in flight together); the pair
-  // products go to the slots of the rates, f and f temps, dead while M is formed
+  const double mc = neg_i(c);
+  // into the slots of the rates, f and f temps, dead while M is formed
   T *const pp = reinterpret_cast<T *>(Wd + M.d_RT);
   const uint32_t wdb = smem_addr(Wd), kt = wdb + 8u * M.d_KT;
   double *const tag = nullptr;
@@ -541,26 +575,41 @@ __device__ __forceinline__ void mlu_core(const MechDev &M, const unsigned char *
   for (; pr + WARP < M.n_pairs; pr += 2 * WARP) {
     const int j0 = prx[pr], j1 = prx[pr + WARP];
     const unsigned o0 = pother[pr], o1 = pother[pr + WARP];
-    double p0 = mc * lds(tag, kt + 8u * j0), p1 = mc * lds(tag, kt + 8u * j1);
-    if (M.max_reac > 1) {
-      p0 *= lds(tag, wdb + (o0 & 0xffff));
-      p1 *= lds(tag, wdb + (o1 & 0xffff));
+    double p0 = o.mul(mc, lds(tag, kt + 8u * j0)), p1 = o.mul(mc, lds(tag, kt + 8u * j1));
+    if (NR > 1) {
+      p0 = o.mul(p0, lds(tag, wdb + (o0 & 0xffff)));
+      p1 = o.mul(p1, lds(tag, wdb + (o1 & 0xffff)));
     }
-    if (M.max_reac > 2) {
-      p0 *= lds(tag, wdb + (o0 >> 16));
-      p1 *= lds(tag, wdb + (o1 >> 16));
+    if (NR > 2) {
+      p0 = o.mul(p0, lds(tag, wdb + (o0 >> 16)));
+      p1 = o.mul(p1, lds(tag, wdb + (o1 >> 16)));
     }
     pp[pr] = (T)p0;
     pp[pr + WARP] = (T)p1;
   }
-  if (pr < M.n_pairs) {
+#pragma unroll 1
+  for (; pr < M.n_pairs; pr += WARP) {
     const int j = prx[pr];
-    const unsigned o = pother[pr];
-    double p = mc * lds(tag, kt + 8u * j);
-    if (M.max_reac > 1) p *= lds(tag, wdb + (o & 0xffff));
-    if (M.max_reac > 2) p *= lds(tag, wdb + (o >> 16));
+    const unsigned oo = pother[pr];
+    double p = o.mul(mc, lds(tag, kt + 8u * j));
+    if (NR > 1) p = o.mul(p, lds(tag, wdb + (oo & 0xffff)));
+    if (NR > 2) p = o.mul(p, lds(tag, wdb + (oo >> 16)));
     pp[pr] = (T)p;
   }
+}
+
+// a3-a5: M = I - c J(y) in the LU slots from y in Wd[Y], then factor
+template <typename T>
+__device__ __forceinline__ void mlu_core(const MechDev &M, const SolveParams &P, const unsigned char *tbase, double *Wd,
+                                         T *WL, const double c, const int lane) {
+  const int prec = P.prec;
+  for (int i = lane; i < M.m_clear; i += WARP) WL[i] = (T)0;
+  __syncwarp();
+  unsigned char *wl = reinterpret_cast<unsigned char *>(WL);
+  const int *diag = reinterpret_cast<const int *>(tbase + M.tab.lu_diag);
+  for (int k = lane; k < M.S; k += WARP) at<T>(wl, diag[k]) = (T)1;
+  if (M.max_reac > 2) pair_products<T, 3>(M, P, tbase, Wd, c, lane);
+  else pair_products<T, 2>(M, P, tbase, Wd, c, lane);
   __syncwarp();
   // The M program runs on the whole per-cell slice (its operands are the pair
   // products in Wd and the LU slots, constants and temporaries in WL), its ops
@@ -637,7 +686,7 @@ struct Cell {
 #pragma unroll
     for (int k = 0; k < KS; ++k)
       if (own[k]) {
-        const double t = v[k] * w[k];
+        const double t = fma(v[k], w[k], P.mzero);
         s = fma(t, t, s);
       }
     return warp_sum_nn(s);
@@ -645,7 +694,7 @@ struct Cell {
 
   __device__ __forceinline__ void weights(const double (&y)[KS], double (&w)[KS]) const {
 #pragma unroll
-    for (int k = 0; k < KS; ++k) w[k] = own[k] ? recip_nr(fma(P.rtol, fabs(y[k]), P.atol)) : 0.0;
+    for (int k = 0; k < KS; ++k) w[k] = own[k] ? recip_nr(fma(P.rtol, abs_i(y[k]), P.atol)) : 0.0;
   }
 
   // a2: f(y) into registers
@@ -654,7 +703,7 @@ struct Cell {
     for (int k = 0; k < KS; ++k)
       if (own[k]) Wd[M.d_Y + lane + WARP * k] = y[k];
     __syncwarp();
-    f_core<STAGED>(M, tb.base, Wd, lane);
+    f_core<STAGED>(M, P, tb.base, Wd, lane);
 #pragma unroll
     for (int k = 0; k < KS; ++k) f[k] = own[k] ? Wd[M.d_F + lane + WARP * k] : 0.0;
     __syncwarp();
@@ -665,7 +714,7 @@ struct Cell {
 #pragma unroll
     for (int k = 0; k < KS; ++k)
       if (own[k]) Wd[M.d_Y + lane + WARP * k] = y[k];
-    mlu_core<T>(M, tb.base, P.prec, Wd, WL, c, lane);
+    mlu_core<T>(M, P, tb.base, Wd, WL, c, lane);
   }
 
   // a5: x = M^{-1} b with the factored M
@@ -676,7 +725,7 @@ struct Cell {
     __syncwarp();
     solve_core<T, STAGED>(M, tb.base, Wd, WL, lane);
 #pragma unroll
-    for (int k = 0; k < KS; ++k) x[k] = own[k] ? -(double)reinterpret_cast<const T *>(Wd + M.d_Y)[pos[k]] : 0.0;
+    for (int k = 0; k < KS; ++k) x[k] = own[k] ? neg_i((double)reinterpret_cast<const T *>(Wd + M.d_Y)[pos[k]]) : 0.0;
     __syncwarp();
   }
 };
@@ -684,7 +733,8 @@ struct Cell {
 // History rescale for a step ratio eta at order q: D'_i = sum_{m>=i} T_im(eta) D_m,
 // T_im a polynomial in eta whose coefficients the host precomputed.
 template <int KS>
-__device__ __forceinline__ void rescale(double (&D)[NROW][KS], int q, double eta, const double *coef, int lane) {
+__device__ __forceinline__ void rescale(const SolveParams &P, double (&D)[NROW][KS], int q, double eta, const double *coef,
+                                        int lane) {
   // lane (i-1)*QMAX + (m-1) evaluates T_im
   double tv = 0.0;
   if (lane < QMAX * QMAX) {
@@ -696,20 +746,21 @@ __device__ __forceinline__ void rescale(double (&D)[NROW][KS], int q, double eta
   // in place, rows ascending: row i reads only rows m >= i, still unchanged
 #pragma unroll
   for (int i = 1; i <= QMAX; ++i) {
-    if (i > q) break;
-    double nd[KS];
+    CHEM_BRANCH(i <= q) {
+      double nd[KS];
 #pragma unroll
-    for (int k = 0; k < KS; ++k) nd[k] = 0.0;
+      for (int k = 0; k < KS; ++k) nd[k] = 0.0;
 #pragma unroll
-    for (int mm = 1; mm <= QMAX; ++mm) {
-      if (mm > q) break;
-      if (mm < i) continue;
-      const double t = __shfl_sync(FULL, tv, (i - 1) * QMAX + (mm - 1));
+      for (int mm = i; mm <= QMAX; ++mm) {
+        CHEM_BRANCH(mm <= q) {
+          const double t = __shfl_sync(FULL, tv, (i - 1) * QMAX + (mm - 1));
 #pragma unroll
-      for (int k = 0; k < KS; ++k) nd[k] = fma(t, D[mm][k], nd[k]);
+          for (int k = 0; k < KS; ++k) nd[k] = fma(t, D[mm][k], nd[k]);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < KS; ++k) D[i][k] = nd[k];
     }
-#pragma unroll
-    for (int k = 0; k < KS; ++k) D[i][k] = nd[k];
   }
 }
 
@@ -737,15 +788,17 @@ __device__ __forceinline__ void get_row(const double (&D)[NROW][KS], int r, doub
 // without a selection need not form it (the next accepted step at this order
 // overwrites it, and at a lower order the row is above those it touches).
 template <int KS>
-__device__ __forceinline__ void accept_update(double (&D)[NROW][KS], int q, const double (&d)[KS], bool top = true) {
+__device__ __forceinline__ void accept_update(const SolveParams &P, double (&D)[NROW][KS], int q, const double (&d)[KS],
+                                              bool top = true) {
+  const Opaque o{P};
 #define CHEM_UPD_CASE(Q_)                                                      \
   case Q_:                                                                    \
-    if (top) {                                                                \
-      _Pragma("unroll") for (int k = 0; k < KS; ++k) D[Q_ + 2][k] = d[k] - D[Q_ + 1][k]; \
+    CHEM_BRANCH(top) {                                                        \
+      _Pragma("unroll") for (int k = 0; k < KS; ++k) D[Q_ + 2][k] = o.sub(d[k], D[Q_ + 1][k]); \
     }                                                                         \
     _Pragma("unroll") for (int k = 0; k < KS; ++k) D[Q_ + 1][k] = d[k];       \
     _Pragma("unroll") for (int m = Q_; m >= 0; --m)                           \
-      _Pragma("unroll") for (int k = 0; k < KS; ++k) D[m][k] += D[m + 1][k];  \
+      _Pragma("unroll") for (int k = 0; k < KS; ++k) D[m][k] = o.add(D[m][k], D[m + 1][k]); \
     break;
   switch (q) {
     CHEM_UPD_CASE(1) CHEM_UPD_CASE(2) CHEM_UPD_CASE(3) CHEM_UPD_CASE(4) CHEM_UPD_CASE(5)
@@ -932,6 +985,7 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
   const bool bad = grp.any(phantom ? false : load_cell<KS>(M, C, Wd, lane, cell, cl.own, y0));
   Recorder<KS, REC> rec(C, cell, M.S);
 
+  const Opaque op{P};
   const double dt = P.dt;
   int q = 1;
   double h = 0.0;
@@ -997,7 +1051,7 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
       // dt - t >= +0 always (t < dt inside the loop)
       if (le_nn(rem, hs)) {
         if (!eq_fp(rem, h)) {
-          rescale<KS>(D, q, rem / h, M.rescale_coef, lane);
+          rescale<KS>(P, D, q, rem / h, M.rescale_coef, lane);
           rec.push(EV_RESCALE, q, rem / h, lane);
           h = rem;
           c = h * iq;
@@ -1015,16 +1069,17 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
       }
 #pragma unroll
       for (int m = 1; m <= QMAX; ++m) {
-        if (m > q) break;
-        const double gm = c_gam[m];
+        CHEM_BRANCH(m <= q) {
+          const double gm = c_gam[m];
 #pragma unroll
-        for (int k = 0; k < KS; ++k) {
-          ypred[k] += D[m][k];
-          psi[k] = fma(gm, D[m][k], psi[k]);
+          for (int k = 0; k < KS; ++k) {
+            ypred[k] = op.add(D[m][k], ypred[k]);
+            psi[k] = fma(gm, D[m][k], psi[k]);
+          }
         }
       }
 #pragma unroll
-      for (int k = 0; k < KS; ++k) psi[k] *= iq;
+      for (int k = 0; k < KS; ++k) psi[k] = op.mul(psi[k], iq);
 
       int fresh = 0;
       const bool same_c = eq_fp(c, scale_c);
@@ -1064,30 +1119,33 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
         st.f_evals++;
 #pragma unroll
         for (int k = 0; k < KS; ++k) tmp[k] = fma(c, f[k], -psi[k]);
-        if (it > 0) {                      // d = +0 before the first correction
+        CHEM_BRANCH(it > 0) {              // d = +0 before the first correction
 #pragma unroll
-          for (int k = 0; k < KS; ++k) tmp[k] -= d[k];
+          for (int k = 0; k < KS; ++k) tmp[k] = op.sub(tmp[k], d[k]);
         }
         cl.solve(tmp, x);
         st.solves++;
-        if (scaled) {
+        CHEM_BRANCH(scaled) {
 #pragma unroll
-          for (int k = 0; k < KS; ++k) x[k] *= scale;
+          for (int k = 0; k < KS; ++k) x[k] = op.mul(x[k], scale);
         }
         del2 = grp.sum(cl.sumsq(x, w));
         if (COUPLED) del2 *= gsc;
-        if (it > 0) {
-#pragma unroll
-          for (int k = 0; k < KS; ++k) d[k] += x[k];
-        } else {
+        if (it == 0) {
 #pragma unroll
           for (int k = 0; k < KS; ++k) d[k] = plus0(x[k]);
         }
+        CHEM_BRANCH(it > 0) {
 #pragma unroll
-        for (int k = 0; k < KS; ++k) y[k] = ypred[k] + d[k];
+          for (int k = 0; k < KS; ++k) d[k] = op.add(x[k], d[k]);
+          rho2 = max_nn(op.mul(CRDOWN * CRDOWN, rho2), op.mul(del2, idel2_prev));
+        }
+#pragma unroll
+        for (int k = 0; k < KS; ++k) y[k] = op.add(d[k], ypred[k]);
         st.newton_iters++;
-        if (it > 0) rho2 = max_nn(CRDOWN * CRDOWN * rho2, del2 * idel2_prev);
-        if (le_nn(gt_nn(1.0, rho2) ? del2 * rho2 : del2, tol2)) { conv = 1; break; }
+        double dr = del2;
+        CHEM_BRANCH(gt_nn(1.0, rho2)) dr = op.mul(del2, rho2);
+        if (le_nn(dr, tol2)) { conv = 1; break; }
         if (it > 0 && gt_nn(del2, RDIV * RDIV * del2_prev)) break;
         // not converged, so del2 > tol2 >= 1e-2 S (q >= 1): a normal number
         del2_prev = del2;
@@ -1100,7 +1158,7 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
         if (!fresh) {
           force_M = 1;
         } else {
-          rescale<KS>(D, q, ETA_CF, M.rescale_coef, lane);
+          rescale<KS>(P, D, q, ETA_CF, M.rescale_coef, lane);
           rec.push(EV_RESCALE, q, ETA_CF, lane);
           h *= ETA_CF;
           n_eq = 0;
@@ -1147,7 +1205,7 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
             if (nef >= MXNEF) { status = CHEM_CELL_ERR_FAIL; break; }
             double eta = ETA_CST_SAFETY * eta_c;
             if (eta < ETA_CST_MIN) eta = ETA_CST_MIN;
-            rescale<KS>(D, q, eta, M.rescale_coef, lane);
+            rescale<KS>(P, D, q, eta, M.rescale_coef, lane);
             rec.push(EV_RESCALE, q, eta, lane);
             h *= eta;
             n_eq = 0;
@@ -1171,7 +1229,7 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
         double eta = gfac[ie];
         if (nef >= 2 && gt_nn(eta, ETA_MXF)) eta = ETA_MXF;
         if (nef >= 3 && q > 1) q -= 1;
-        rescale<KS>(D, q, eta, M.rescale_coef, lane);
+        rescale<KS>(P, D, q, eta, M.rescale_coef, lane);
         rec.push(EV_RESCALE, q, eta, lane);
         h *= eta;
         n_eq = 0;
@@ -1186,7 +1244,7 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
       nef = 0;
       ncf = 0;
       n_eq++;
-      accept_update<KS>(D, q, d, n_eq >= q + 1);
+      accept_update<KS>(P, D, q, d, n_eq >= q + 1);
       rec.accept_iters(n_it, lane);
       rec.accept_projections(pm, lane);
       rec.push(EV_STEP, q, c, lane);
@@ -1216,7 +1274,7 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
       const double eta = gfac[ieta];
       if (le_nn(THRESH, eta)) {
         q = qn;
-        rescale<KS>(D, q, eta, M.rescale_coef, lane);
+        rescale<KS>(P, D, q, eta, M.rescale_coef, lane);
         rec.push(EV_RESCALE, q, eta, lane);
         h *= eta;
         n_eq = 0;
@@ -1509,7 +1567,8 @@ cudaError_t launch_ks(const MechDev &M, const CellsDev &C, const SolveParams &P,
 
 // lambda_{1..q} <- T(eta)^T lambda_{1..q}: lambda'_m = sum_{i<=m} T_im lambda_i
 template <int KS>
-__device__ __forceinline__ void rescale_adjoint(double (&L)[NROW][KS], int q, double eta, const double *coef, int lane) {
+__device__ __forceinline__ void rescale_adjoint(const SolveParams &P, double (&L)[NROW][KS], int q, double eta,
+                                                const double *coef, int lane) {
   double tv = 0.0;
   if (lane < QMAX * QMAX) {
     const double *cp = coef + lane * (QMAX + 1);
@@ -1520,19 +1579,19 @@ __device__ __forceinline__ void rescale_adjoint(double (&L)[NROW][KS], int q, do
   // m descending: row m reads rows i <= m, still unchanged
 #pragma unroll
   for (int mm = QMAX; mm >= 1; --mm) {
-    if (mm > q) continue;
-    double nl[KS];
+    CHEM_BRANCH(mm <= q) {
+      double nl[KS];
 #pragma unroll
-    for (int k = 0; k < KS; ++k) nl[k] = 0.0;
+      for (int k = 0; k < KS; ++k) nl[k] = 0.0;
 #pragma unroll
-    for (int i = 1; i <= QMAX; ++i) {
-      if (i > mm) continue;
-      const double t = __shfl_sync(FULL, tv, (i - 1) * QMAX + (mm - 1));
+      for (int i = 1; i <= mm; ++i) {
+        const double t = __shfl_sync(FULL, tv, (i - 1) * QMAX + (mm - 1));
 #pragma unroll
-      for (int k = 0; k < KS; ++k) nl[k] = fma(t, L[i][k], nl[k]);
+        for (int k = 0; k < KS; ++k) nl[k] = fma(t, L[i][k], nl[k]);
+      }
+#pragma unroll
+      for (int k = 0; k < KS; ++k) L[mm][k] = nl[k];
     }
-#pragma unroll
-    for (int k = 0; k < KS; ++k) L[mm][k] = nl[k];
   }
 }
 
@@ -1540,17 +1599,18 @@ __device__ __forceinline__ void rescale_adjoint(double (&L)[NROW][KS], int q, do
 // lambda_d = lambda_{q+2} + lambda_{q+1} + sum_{m<=q} lambda_m; lambda_i (i<=q)
 // = prefix sums, lambda_{q+1} = -lambda_{q+2}, lambda_{q+2} = 0.
 template <int KS>
-__device__ __forceinline__ void step_adjoint_linear(double (&L)[NROW][KS], int q, double (&lamd)[KS]) {
+__device__ __forceinline__ void step_adjoint_linear(const SolveParams &P, double (&L)[NROW][KS], int q, double (&lamd)[KS]) {
+  const Opaque o{P};
 #define CHEM_ADJ_CASE(Q_)                                                           \
   case Q_:                                                                         \
     _Pragma("unroll") for (int k = 0; k < KS; ++k) {                               \
       double acc = 0.0;                                                            \
       _Pragma("unroll") for (int m = 0; m <= Q_; ++m) {                            \
-        acc += L[m][k];                                                            \
+        acc = o.add(L[m][k], acc);                                                 \
         L[m][k] = acc;                                                             \
       }                                                                            \
-      lamd[k] = L[Q_ + 2][k] + L[Q_ + 1][k] + acc;                                 \
-      L[Q_ + 1][k] = -L[Q_ + 2][k];                                                \
+      lamd[k] = o.add(o.add(L[Q_ + 2][k], L[Q_ + 1][k]), acc);                     \
+      L[Q_ + 1][k] = neg_i(L[Q_ + 2][k]);                                          \
       L[Q_ + 2][k] = 0.0;                                                          \
     }                                                                              \
     break;
@@ -1562,31 +1622,33 @@ __device__ __forceinline__ void step_adjoint_linear(double (&L)[NROW][KS], int q
 #undef CHEM_ADJ_CASE
 }
 
-// rates RT and partials PP = dr_j/dy_l at the y stored in Wd[Y]
-template <int KS>
-__device__ __forceinline__ void rates_partials(const MechDev &M, const Tabs &tb, double *Wd, int lane) {
-  unsigned char *wd = reinterpret_cast<unsigned char *>(Wd);
-  for (int j = lane; j < M.R; j += WARP) {
-    const uint2 sl = tab<uint2>(tb, M.tab.rx_slots)[j];
-    double r = Wd[M.d_KT + j] * at<double>(wd, sl.x & 0xffff);
-    if (M.max_reac > 1) r *= at<double>(wd, sl.x >> 16);
-    if (M.max_reac > 2) r *= at<double>(wd, sl.y & 0xffff);
-    Wd[M.d_RT + j] = r;
-  }
+// rates RT and partials PP = dr_j/dy_l at the y stored in Wd[Y]; NR: the most
+// reactants of a reaction
+template <int NR>
+__device__ __forceinline__ void rates_partials(const MechDev &M, const SolveParams &P, const Tabs &tb, double *Wd, int lane) {
+  const Opaque o{P};
+  const uint32_t wb = smem_addr(Wd);
+  double *const tag = nullptr;
+  rates<NR>(M, P, tab<uint2>(tb, M.tab.rx_slots), wb, lane);
+#pragma unroll 2
   for (int pr = lane; pr < M.n_pairs; pr += WARP) {
     const int j = tab<int>(tb, M.tab.pair_rx)[pr];
-    const unsigned o = tab<unsigned>(tb, M.tab.pair_other)[pr];
-    double p = Wd[M.d_KT + j];
-    if (M.max_reac > 1) p *= at<double>(wd, o & 0xffff);
-    if (M.max_reac > 2) p *= at<double>(wd, o >> 16);
-    Wd[M.a_PP + pr] = p;
+    const unsigned oo = tab<unsigned>(tb, M.tab.pair_other)[pr];
+    double p = lds(tag, wb + 8u * (M.d_KT + j));
+    if (NR > 1) p = o.mul(p, lds(tag, wb + (oo & 0xffff)));
+    if (NR > 2) p = o.mul(p, lds(tag, wb + (oo >> 16)));
+    sts(wb + 8u * (M.a_PP + pr), p);
   }
   __syncwarp();
+}
+__device__ __forceinline__ void rates_partials(const MechDev &M, const SolveParams &P, const Tabs &tb, double *Wd, int lane) {
+  if (M.max_reac > 2) rates_partials<3>(M, P, tb, Wd, lane);
+  else rates_partials<2>(M, P, tb, Wd, lane);
 }
 
 // Wd[MU] = v; runs nu.mu and J^T mu programs; theta gradient += scale * r_j * (nu_j . v); out = J^T v
 template <int KS>
-__device__ __forceinline__ void jt_and_theta(const MechDev &M, double *Wd, const bool (&own)[KS], const double (&v)[KS],
+__device__ __forceinline__ void jt_and_theta(const MechDev &M, const SolveParams &P, double *Wd, const bool (&own)[KS], const double (&v)[KS],
                                              double scale, double (&out)[KS], int lane) {
 #pragma unroll
   for (int k = 0; k < KS; ++k)
@@ -1594,7 +1656,9 @@ __device__ __forceinline__ void jt_and_theta(const MechDev &M, double *Wd, const
   __syncwarp();
   run_prog<double, false, true, false>(M.nudot_ops, M.nudot_runs, M.nudot_nruns, M.nudot_npass, Wd, lane);
   run_prog<double, false, true, false>(M.jt_ops, M.jt_runs, M.jt_nruns, M.jt_npass, Wd, lane);
-  for (int j = lane; j < M.R; j += WARP) Wd[M.a_G + j] = fma(scale * Wd[M.d_RT + j], Wd[M.a_NM + j], Wd[M.a_G + j]);
+#pragma unroll 2
+  for (int j = lane; j < M.R; j += WARP)
+    Wd[M.a_G + j] = fma(Opaque{P}.mul(scale, Wd[M.d_RT + j]), Wd[M.a_NM + j], Wd[M.a_G + j]);
 #pragma unroll
   for (int k = 0; k < KS; ++k) out[k] = own[k] ? Wd[M.a_JTM + lane + WARP * k] : 0.0;
   __syncwarp();
@@ -1610,6 +1674,7 @@ template <int KS>
 __device__ void backward_cell(const MechDev &M, const CellsDev &C, const AdjDev &A, const SolveParams &P, const Tabs &tb,
                               double *Wd, double *WL, const int lane, const int64_t cell) {
   const int64_t NC = C.n_cells;
+  const Opaque op{P};
   Cell<double, KS, false> cl(M, P, tb, Wd, WL, lane);
   cl.init_constants();
   unsigned char *wd = reinterpret_cast<unsigned char *>(Wd);
@@ -1660,9 +1725,9 @@ __device__ void backward_cell(const MechDev &M, const CellsDev &C, const AdjDev 
     const double val = __ldg(vals + e);
     const int kind = kq & 0xff, q = kq >> 8;
     if (kind == EV_RESCALE) {
-      rescale_adjoint<KS>(L, q, val, M.rescale_coef, lane);
+      rescale_adjoint<KS>(P, L, q, val, M.rescale_coef, lane);
     } else if (kind == EV_STEP) {
-      step_adjoint_linear<KS>(L, q, lamd);
+      step_adjoint_linear<KS>(P, L, q, lamd);
 #pragma unroll
       for (int k = 0; k < KS; ++k) lyp[k] = lpsi[k] = 0.0;
       sq = q;
@@ -1687,7 +1752,7 @@ __device__ void backward_cell(const MechDev &M, const CellsDev &C, const AdjDev 
 #pragma unroll
       for (int k = 0; k < KS; ++k)
         if (q == lane + WARP * k) {
-          lyp[k] = -lamd[k];
+          lyp[k] = neg_i(lamd[k]);
           lamd[k] = 0.0;
         }
     } else if (kind == EV_ITER) {
@@ -1701,7 +1766,7 @@ __device__ void backward_cell(const MechDev &M, const CellsDev &C, const AdjDev 
       for (int k = 0; k < KS; ++k)
         if (cl.own[k]) Wd[M.d_Y + lane + WARP * k] = y[k];
       __syncwarp();
-      rates_partials<KS>(M, tb, Wd, lane);
+      rates_partials(M, P, tb, Wd, lane);
       // g = s M^{-T} lambda_d
 #pragma unroll
       for (int k = 0; k < KS; ++k)
@@ -1710,25 +1775,25 @@ __device__ void backward_cell(const MechDev &M, const CellsDev &C, const AdjDev 
       run_prog<double, false, false, false>(M.fwdT_ops, nullptr, 1, M.fwdT_npass, Wd, lane);
       run_prog<double, false, false, false>(M.bwdT_ops, nullptr, 1, M.bwdT_npass, Wd, lane);
 #pragma unroll
-      for (int k = 0; k < KS; ++k) g[k] = cl.own[k] ? -ss * Wd[M.d_Y + cl.pos[k]] : 0.0;   // the programs leave -M^{-T} lambda
+      for (int k = 0; k < KS; ++k) g[k] = cl.own[k] ? op.mul(neg_i(ss), Wd[M.d_Y + cl.pos[k]]) : 0.0;   // the programs leave -M^{-T} lambda
       __syncwarp();
-      jt_and_theta<KS>(M, Wd, cl.own, g, sc, jtg, lane);
+      jt_and_theta<KS>(M, P, Wd, cl.own, g, sc, jtg, lane);
 #pragma unroll
       for (int k = 0; k < KS; ++k) {
-        const double cj = sc * jtg[k];
-        lamd[k] += cj - g[k];
-        lyp[k] += cj;
-        lpsi[k] -= g[k];
+        lamd[k] = op.add(fma(sc, jtg[k], -g[k]), lamd[k]);
+        lyp[k] = fma(sc, jtg[k], lyp[k]);
+        lpsi[k] = op.sub(lpsi[k], g[k]);
       }
       if (q == 0) {
         // the predictor: y_pred = sum_{m<=q} D_m, psi = (1/gamma_q) sum gamma_m D_m
         const double iq = c_igam[sq];
 #pragma unroll
         for (int m = 0; m <= QMAX; ++m) {
-          if (m > sq) continue;
-          const double gm = (m >= 1) ? c_gam[m] * iq : 0.0;
+          CHEM_BRANCH(m <= sq) {
+            const double gm = (m >= 1) ? op.mul(c_gam[m], iq) : 0.0;
 #pragma unroll
-          for (int k = 0; k < KS; ++k) L[m][k] += fma(gm, lpsi[k], lyp[k]);
+            for (int k = 0; k < KS; ++k) L[m][k] = op.add(fma(gm, lpsi[k], lyp[k]), L[m][k]);
+          }
         }
       }
     } else if (kind == EV_REFACTOR) {
@@ -1745,10 +1810,10 @@ __device__ void backward_cell(const MechDev &M, const CellsDev &C, const AdjDev 
       for (int k = 0; k < KS; ++k)
         if (cl.own[k]) Wd[M.d_Y + lane + WARP * k] = y[k];
       __syncwarp();
-      rates_partials<KS>(M, tb, Wd, lane);
+      rates_partials(M, P, tb, Wd, lane);
 #pragma unroll
       for (int k = 0; k < KS; ++k) l1[k] = L[1][k];
-      jt_and_theta<KS>(M, Wd, cl.own, l1, val, jtl, lane);
+      jt_and_theta<KS>(M, P, Wd, cl.own, l1, val, jtl, lane);
 #pragma unroll
       for (int k = 0; k < KS; ++k) L[0][k] = fma(val, jtl[k], L[0][k]);
 #pragma unroll
@@ -1875,6 +1940,7 @@ __device__ void tangent_cell(const MechDev &M, const CellsDev &C, const TanDev &
     for (int k = 0; k < KS; ++k) y[k] = pre[k];
     if (++row < nrows) read_row<KS>(yt, row, M.S, cl.own, lane, pre);
   };
+  const Opaque op{P};
   bool in_step = false, have_M = false, bad = false;
   double cM = 0.0, sc = 0.0, ss = 1.0;
   int sq = 1;
@@ -1918,20 +1984,21 @@ __device__ void tangent_cell(const MechDev &M, const CellsDev &C, const TanDev &
       }
 #pragma unroll
       for (int m = 1; m <= QMAX; ++m) {
-        if (m > sq) continue;
-        const double gm = c_gam[m];
+        CHEM_BRANCH(m <= sq) {
+          const double gm = c_gam[m];
 #pragma unroll
-        for (int k = 0; k < KS; ++k) {
-          dyp[k] += dD[m][k];
-          dpsi[k] = fma(gm, dD[m][k], dpsi[k]);
+          for (int k = 0; k < KS; ++k) {
+            dyp[k] = op.add(dD[m][k], dyp[k]);
+            dpsi[k] = fma(gm, dD[m][k], dpsi[k]);
+          }
         }
       }
 #pragma unroll
-      for (int k = 0; k < KS; ++k) dpsi[k] *= iq;
+      for (int k = 0; k < KS; ++k) dpsi[k] = op.mul(dpsi[k], iq);
       in_step = true;
     }
     if (kind == EV_RESCALE) {
-      rescale<KS>(dD, q, val, M.rescale_coef, lane);
+      rescale<KS>(P, dD, q, val, M.rescale_coef, lane);
     } else if (kind == EV_INIT) {
       // D_0 = y, D_1 = h0 f(y), higher rows reset
       if (row >= nrows) {
@@ -1972,22 +2039,22 @@ __device__ void tangent_cell(const MechDev &M, const CellsDev &C, const TanDev &
       next_row(y);
 #pragma unroll
       for (int k = 0; k < KS; ++k) {
-        v[k] = dyp[k] + dd[k];
+        v[k] = op.add(dd[k], dyp[k]);
         if (cl.own[k]) Wd[M.d_Y + lane + WARP * k] = y[k];
       }
       tangent_f<KS>(M, tb, Wd, A.dtheta, cl.own, v, g, lane);
 #pragma unroll
-      for (int k = 0; k < KS; ++k) b[k] = sc * g[k] - dpsi[k] - dd[k];
+      for (int k = 0; k < KS; ++k) b[k] = op.sub(fma(sc, g[k], -dpsi[k]), dd[k]);
       cl.solve(b, x);
 #pragma unroll
       for (int k = 0; k < KS; ++k) dd[k] = fma(ss, x[k], dd[k]);
     } else if (kind == EV_STEP) {
 #pragma unroll
       for (int k = 0; k < KS; ++k) {
-        if (pm[k]) dd[k] = -dyp[k];          // projected onto y = 0
+        if (pm[k]) dd[k] = neg_i(dyp[k]);          // projected onto y = 0
         pm[k] = false;
       }
-      accept_update<KS>(dD, sq, dd);
+      accept_update<KS>(P, dD, sq, dd);
       in_step = false;
     }
     // PROJECT events were read with their step's predictor
@@ -2350,7 +2417,7 @@ __device__ __forceinline__ void deriv_tile_load(const MechDev &M, const int64_t 
 }
 
 __device__ __forceinline__ void deriv_tile(const MechDev &M, const int64_t NC, const int64_t c, double *f, double *sm,
-                                           int lane, int warp, int bar) {
+                                           int lane, int warp, int bar, const SolveParams &P) {
   const bool in = c < NC;
   double *const ys = sm, *const rs = sm + (size_t)M.S * TILE_CELLS;      // [S][32], [R][32]
   // (no predicated FP64 instruction: one with every lane off still takes the
@@ -2360,7 +2427,7 @@ __device__ __forceinline__ void deriv_tile(const MechDev &M, const int64_t NC, c
   double *const tag = nullptr;
   // a product as fma(a, b, -0): the same bits, and an FP64 multiplication takes
   // the unit 76 cycles where an FMA takes 64
-  auto mul = [](double a, double b) { return fma_now(a, b, -0.0); };
+  auto mul = [&](double a, double b) { return fma_now(a, b, P.mzero); };
   int e = warp;
 #pragma unroll 2
   for (; e < M.tl_rx_end[0]; e += TILE_WARPS) {
@@ -2423,10 +2490,9 @@ __device__ __forceinline__ void deriv_tile(const MechDev &M, const int64_t NC, c
         }
         return acc;
       };
-      const double one = 1.0;
       total = chunk(k + TILE_CHUNK < k1 ? k + TILE_CHUNK : k1);
 #pragma unroll 1
-      while (k < k1) total = fma_now(one, chunk(k + TILE_CHUNK < k1 ? k + TILE_CHUNK : k1), total);
+      while (k < k1) total = fma_now(P.one, chunk(k + TILE_CHUNK < k1 ? k + TILE_CHUNK : k1), total);
     }
     if (in) f[(int64_t)i * NC + c] = total;
   }
@@ -2434,7 +2500,7 @@ __device__ __forceinline__ void deriv_tile(const MechDev &M, const int64_t NC, c
 
 __global__ void __launch_bounds__(32 * WARP) deriv_gather_kernel(const __grid_constant__ MechDev M, const int64_t NC,
                                                                              const double *kt, const double *y, double *f,
-                                                                             const DerivSplit D) {
+                                                                             const DerivSplit D, const SolveParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & (WARP - 1);
   int warp = threadIdx.x / WARP;
@@ -2447,7 +2513,7 @@ __global__ void __launch_bounds__(32 * WARP) deriv_gather_kernel(const __grid_co
       deriv_tile_load(M, NC, c, kt, y, sm, lane, warp);
       cp_async_wait_all();
       group_sync(TILE_BAR + g, TILE_WARPS);
-      deriv_tile(M, NC, c, f, sm, lane, warp, TILE_BAR + g);
+      deriv_tile(M, NC, c, f, sm, lane, warp, TILE_BAR + g, P);
       group_sync(TILE_BAR + g, TILE_WARPS);
     }
     return;
@@ -2479,7 +2545,7 @@ __global__ void __launch_bounds__(32 * WARP) deriv_gather_kernel(const __grid_co
       at<double>(wd, reinterpret_cast<const int *>(gb + M.tab.dconst_off)[k]) = reinterpret_cast<const double *>(gb + M.tab.dconst_val)[k];
   }
   group_sync(GATHER_BAR, D.gather_cells);
-  if (warp < nb) f_core<true>(M, gs, sm + (size_t)warp * D.cell_doubles, lane);
+  if (warp < nb) f_core<true>(M, P, gs, sm + (size_t)warp * D.cell_doubles, lane);
   group_sync(GATHER_BAR, D.gather_cells);
   for (int i = tid; i < M.S * D.gather_cells; i += nt) {
     const int r = i / D.gather_cells, cl = i % D.gather_cells;
@@ -2757,7 +2823,8 @@ cudaError_t launch_deriv_gather(const MechDev &M, const CellsDev &C, const doubl
                                   : 0);
   const cudaError_t e = allow_max_smem<deriv_gather_kernel>();
   if (e != cudaSuccess) return e;
-  deriv_gather_kernel<<<(unsigned)blocks, (D.tile_warps + D.gather_cells) * WARP, smem, stream>>>(M, C.n_cells, kt, y, f, D);
+  deriv_gather_kernel<<<(unsigned)blocks, (D.tile_warps + D.gather_cells) * WARP, smem, stream>>>(M, C.n_cells, kt, y, f, D,
+                                                                                                SolveParams{});
   return cudaGetLastError();
 }
 
