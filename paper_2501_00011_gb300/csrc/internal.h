@@ -107,7 +107,7 @@ struct MechDev {
   int WL_len, L_LU, L_X, L_P, L_ZERO, L_DUMMY, nnz_lu;
   int d_nconst, L_nconst;
   int m_clear;             // WL entries [0, m_clear) are cleared before forming M
-  int f_npass, fwd_npass, bwd_npass, m_npass, lu_npass;
+  int fwd_npass, bwd_npass;
   int f_nruns, m_nruns, lu_nruns;  // run tables (f: in the staged blob; M, LU: m_runs, lu_runs)
   const uint32_t *m_runs, *lu_runs;
   // staged tables: blob[0] for an FP64 LU, blob[1] for an FP32 LU (global memory)
@@ -127,20 +127,27 @@ struct MechDev {
   const double *a_const_val;
   const ushort4 *nudot_ops, *jt_ops;    // programs on the extended Wd
   const ushort4 *fwdT_ops, *bwdT_ops;   // U^T and L^T solves on WL (FP64 byte offsets)
-  int nudot_npass, jt_npass, fwdT_npass, bwdT_npass;
+  int fwdT_npass, bwdT_npass;
   const uint32_t *nudot_runs, *jt_runs;   // run tables of nudot and jt
   int nudot_nruns, jt_nruns;
 };
 
-// Kinds of the units a program's passes form, in its run table (one uint32 per
-// run of equal units: kind << 28 | units): a single pass of FMAs, a pair of
-// consecutive FMA passes whose 64 ops are independent of each other (the
-// interpreter loads the operands of both before it stores either result, so a
-// lane has two FMAs in flight between warp synchronisations), three passes with
-// reciprocals in the first (RECIP): a lane with a reciprocal spends three FP64
-// instructions on it and has no op in the other two, every other lane runs its
-// three FMA ops; all ops of the unit are independent of each other.
-constexpr uint32_t RUN_FMA1 = 0, RUN_FMA2 = 1, RUN_RECIP = 2;
+// On the device a program is a sequence of groups of two passes, lane by lane:
+// 32 x (op of the first pass, op of the second), so one 16-byte load brings a
+// lane's ops of both.  Its run table holds one uint32 per run of equal groups
+// (kind << 28 | groups):
+//   RUN_SEQ2   two passes, one after the other
+//   RUN_FMA2   a pair: 64 mutually independent FMAs; the operands of both passes
+//              are loaded before either result is stored, so a lane has two FMAs
+//              in flight between warp synchronisations
+//   RUN_RECIP  two groups, three passes, reciprocals in the first: a lane with a
+//              reciprocal spends three FP64 instructions on it and has no op in the
+//              other two, every other lane runs its three FMA ops; all ops of the
+//              unit are independent of each other
+//   RUN_FMA1   one pass (the second op slot is not used)
+constexpr uint32_t RUN_SEQ2 = 0, RUN_FMA2 = 1, RUN_RECIP = 2, RUN_FMA1 = 3;
+constexpr int GROUP_BYTES = 2 * WARP * 8;
+constexpr int PAD_GROUPS = 5;     // readable groups past a program's last (the interpreters read ahead unconditionally)
 
 struct HostProgram {
   std::vector<Op> ops;   // n_pass * 32
@@ -149,19 +156,29 @@ struct HostProgram {
   std::vector<uint8_t> unit;
   int n_ops = 0;
   int n_pass() const { return (int)(ops.size() / WARP); }
-  std::vector<uint32_t> runs() const {
-    std::vector<uint32_t> r;
-    uint32_t kind = 0xf, n = 0;
-    for (size_t p = 0; p < unit.size(); ++p) {
-      if (unit[p] == 2) continue;
-      if (p >= 1 && unit[p - 1] == 3) { ++p; continue; }   // the second and third pass of a reciprocal unit
-      const uint32_t k = unit[p] == 1 ? RUN_FMA2 : unit[p] == 3 ? RUN_RECIP : RUN_FMA1;
-      if (k != kind && n) r.push_back(kind << 28 | n), n = 0;
-      kind = k;
-      n++;
+  // the device form's groups: the passes in each (-1: none), and the run table
+  void groups(std::vector<std::pair<int, int>> &g, std::vector<uint32_t> &runs) const {
+    auto push = [&](uint32_t kind, int a, int b) {
+      g.push_back({a, b});
+      if (!runs.empty() && runs.back() >> 28 == kind) runs.back()++;
+      else runs.push_back(kind << 28 | 1u);
+    };
+    for (int p = 0; p < (int)unit.size();) {
+      if (unit[p] == 1) {
+        push(RUN_FMA2, p, p + 1);
+        p += 2;
+      } else if (unit[p] == 3) {
+        push(RUN_RECIP, p, p + 1);       // runs count units: two groups each
+        g.push_back({p + 2, -1});
+        p += 3;
+      } else if (p + 1 < (int)unit.size() && unit[p + 1] == 0) {
+        push(RUN_SEQ2, p, p + 1);
+        p += 2;
+      } else {
+        push(RUN_FMA1, p, -1);
+        p += 1;
+      }
     }
-    if (n) r.push_back(kind << 28 | n);
-    return r;
   }
 };
 

@@ -94,12 +94,6 @@ __device__ __forceinline__ double recip_nr(double x) {
 __device__ __forceinline__ double lu_recip(double x) { return recip_nr(x); }
 __device__ __forceinline__ float lu_recip(float x) { return __frcp_rn(x); }
 
-template <bool SMEM>
-__device__ __forceinline__ uint2 ld_op(const ushort4 *p) {
-  if (SMEM) return *reinterpret_cast<const uint2 *>(p);
-  return __ldg(reinterpret_cast<const uint2 *>(p));
-}
-
 template <typename T>
 __device__ __forceinline__ T &at(unsigned char *base, unsigned off) {
   return *reinterpret_cast<T *>(base + off);
@@ -190,166 +184,187 @@ struct RecipUnit<float> {
   }
 };
 
-// A program with a run table (RUN_* units, internal.h).  The addresses of the
-// next two passes' ops are held in registers (A0, A1); a unit loads the ops
-// that follow it before its own operands and turns them into addresses while
-// its FMAs are in flight, so neither the loads nor the address arithmetic sit
-// between a unit's stores and the next unit's operand loads.  Runs are read
-// from shared memory (SMEM) or global memory like the ops; WIDE / RECIP: the
-// program has pair / reciprocal units (a run table without them compiles to a
-// plain loop).
-template <typename T, bool SMEM, bool WIDE, bool RECIP>
-__device__ __forceinline__ void run_prog(const ushort4 *ops, const uint32_t *runs, const int nruns, const int np, T *W,
-                                         const int lane) {
-  const uint32_t wb = smem_addr(W);
-  T *const tag = nullptr;
-  ops += lane;
-  uint2 r0 = np > 0 ? ld_op<SMEM>(ops) : make_uint2(0, 0);
-  uint2 r1 = np > 1 ? ld_op<SMEM>(ops + WARP) : make_uint2(0, 0);
-  OpAddr A0 = unpack(wb, r0), A1 = unpack(wb, r1);
-  int p = 0;
-#pragma unroll 1
-  for (int r = 0; r < nruns; ++r) {
-    // (without pairs and reciprocals the program is one run of all its passes)
-    const uint32_t rr = !WIDE && !RECIP ? (uint32_t)np : SMEM ? runs[r] : __ldg(runs + r);
-    const uint32_t kind = rr >> 28;
-    int n = (int)(rr & 0x0fffffffu);
-    if (WIDE && kind == RUN_FMA2) {
-#pragma unroll 1
-      for (; n > 0; --n, p += 2) {
-        if (p + 2 < np) r0 = ld_op<SMEM>(ops + (size_t)(p + 2) * WARP);
-        if (p + 3 < np) r1 = ld_op<SMEM>(ops + (size_t)(p + 3) * WARP);
-        const T a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
-        const T a2 = lds(tag, A1.a), b2 = lds(tag, A1.b), c2 = lds(tag, A1.c);
-        const T v = fma(a, b, c), v2 = fma(a2, b2, c2);
-        const uint32_t t = A0.t, t2 = A1.t;
-        A0 = unpack(wb, r0);
-        A1 = unpack(wb, r1);
-        sts(t, v);
-        sts(t2, v2);
-        __syncwarp();
-      }
-    } else if (RECIP && kind == RUN_RECIP) {
-#pragma unroll 1
-      for (; n > 0; --n, p += 3) {
-        const OpAddr A2 = unpack(wb, ld_op<SMEM>(ops + (size_t)(p + 2) * WARP));
-        if (p + 3 < np) r0 = ld_op<SMEM>(ops + (size_t)(p + 3) * WARP);
-        if (p + 4 < np) r1 = ld_op<SMEM>(ops + (size_t)(p + 4) * WARP);
-        RecipUnit<T> ru;
-        ru.load_and_run(wb, A0, A1, A2);
-        ru.store(A0, A1, A2);
-        A0 = unpack(wb, r0);
-        A1 = unpack(wb, r1);
-        __syncwarp();
-      }
-    } else {
-#pragma unroll 1
-      for (; n > 0; --n, ++p) {
-        if (p + 2 < np) r0 = ld_op<SMEM>(ops + (size_t)(p + 2) * WARP);
-        const T a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
-        const T v = fma(a, b, c);
-        const uint32_t t = A0.t;
-        A0 = A1;
-        A1 = unpack(wb, r0);
-        sts(t, v);
-        __syncwarp();
-      }
-    }
-  }
-}
-
-// The same for programs in global memory, the ops streamed through a ring of
-// RING x 256 bytes of shared memory (ring: 8-byte aligned shared address) by
-// cp.async.  Each lane copies and reads only its own op slots, so
-// cp.async.wait_group alone orders them.  Invariant at the start of a unit at
-// pass p: passes up to p + RING - 3 are issued and the ops of passes p and
-// p + 1 are in A0, A1.  A unit issues one pass per pass it consumes, into the
-// slots of passes p - 2, p - 1 (read into registers by earlier units) and, a
-// reciprocal unit, p (whose op's addresses its operand loads have used by
-// then); it waits until the passes after it have landed and refills A0, A1.
-template <typename T, int RING, bool WIDE, bool RECIP>
-__device__ __forceinline__ void run_prog_ring(const ushort4 *ops, const uint32_t *runs, const int nruns, const int np, T *W,
-                                              const int lane, const uint32_t ring) {
-  static_assert(RING >= 6 && (RING & (RING - 1)) == 0, "ring too shallow to run ahead, or not a power of two");
-  const uint32_t wb = smem_addr(W);
-  T *const tag = nullptr;
-  const uint2 *g = reinterpret_cast<const uint2 *>(ops) + lane;
-  const uint32_t rb = ring + 8u * lane;
-  auto issue = [&](int q) {             // pass q into its ring slot (nothing past the end)
-    if (q < np) cp_async8(rb + 256u * (q % RING), g + (size_t)q * WARP);
-    cp_async_commit();
-  };
-  auto fetch = [&](int q) {
-    uint2 o;
-    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(o.x), "=r"(o.y) : "r"(rb + 256u * (q % RING)) : "memory");
+// Where a program's groups come from: first() gives a lane's ops of the first
+// group, next() those of the following one.  All read ahead without asking for the
+// end (programs are padded): the instructions between an FMA and the next bound a
+// lone warp (one op load per pass with bounds checks: 194 cycles a pass of the
+// factorisation, 65k cycles in all) and a full SM in part.  301 cells of the
+// 72-species mechanism 6.4 -> 5.6 ms, 10 cells of 20 species 1.2x faster, 10,000
+// cells first solve 22.2 -> 21.6 ms, FP32 LU 14.8 -> 14.1 ms, tangent of 2,048
+// cells 11.4 -> 8.9 ms, with this form.
+// Shared memory: one load, in flight beside the group's operand loads.
+struct SmemStream {
+  uint32_t p;
+  __device__ __forceinline__ SmemStream(const ushort4 *ops, int lane) : p(smem_addr(ops) + 16u * lane) {}
+  __device__ __forceinline__ uint4 get() const {
+    uint4 o;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(o.x), "=r"(o.y), "=r"(o.z), "=r"(o.w) : "r"(p) : "memory");
     return o;
-  };
-#pragma unroll 1
-  for (int i = 0; i < RING - 2; ++i) issue(i);
-  cp_async_wait<RING - 4>();            // passes 0 and 1 have landed
-  uint2 r0 = make_uint2(0, 0), r1 = make_uint2(0, 0);
-  if (np > 0) r0 = fetch(0);
-  if (np > 1) r1 = fetch(1);
-  OpAddr A0 = unpack(wb, r0), A1 = unpack(wb, r1);
-  int p = 0;
+  }
+  __device__ __forceinline__ uint4 first() const { return get(); }
+  __device__ __forceinline__ uint4 next() {
+    p += GROUP_BYTES;
+    return get();
+  }
+  __device__ __forceinline__ void end() const {}
+};
+// Global memory: two groups ahead in registers.
+struct GlobalStream {
+  const uint4 *p;
+  uint4 n1, n2;
+  __device__ __forceinline__ GlobalStream(const ushort4 *ops, int lane) : p(reinterpret_cast<const uint4 *>(ops) + lane) {}
+  __device__ __forceinline__ uint4 first() {
+    n1 = __ldg(p + WARP);
+    n2 = __ldg(p + 2 * WARP);
+    return __ldg(p);
+  }
+  __device__ __forceinline__ uint4 next() {
+    const uint4 o = n1;
+    n1 = n2;
+    p += WARP;
+    n2 = __ldg(p + 2 * WARP);
+    return o;
+  }
+  __device__ __forceinline__ void end() const {}
+};
+// Global memory through a ring of RING groups of shared memory (at a 16-byte
+// aligned shared address) filled by cp.async.  Each lane copies and reads only
+// its own ops, so cp.async.wait_group alone orders them.  next() at group g
+// refills the slot of group g, whose ops were turned into addresses a group ago,
+// with group g + RING and takes group g + 1, which was asked for RING - 1 groups
+// ago.
+constexpr int RING = 4, RING_BYTES = RING * GROUP_BYTES;
+struct RingStream {
+  const uint4 *p;             // the group that goes into the ring next
+  uint32_t base, off;         // the ring; the slot it goes to
+  __device__ __forceinline__ RingStream(const ushort4 *ops, int lane, uint32_t ring)
+      : p(reinterpret_cast<const uint4 *>(ops) + lane), base(ring + 16u * lane), off(0) {}
+  __device__ __forceinline__ void issue() {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(base + off), "l"(p) : "memory");
+    cp_async_commit();
+    p += WARP;
+    off = (off + GROUP_BYTES) & (RING_BYTES - 1);
+  }
+  __device__ __forceinline__ uint4 get(uint32_t at) const {
+    uint4 o;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(o.x), "=r"(o.y), "=r"(o.z), "=r"(o.w) : "r"(base + at) : "memory");
+    return o;
+  }
+  __device__ __forceinline__ uint4 first() {
+#pragma unroll
+    for (int i = 0; i < RING; ++i) issue();
+    cp_async_wait<RING - 1>();
+    return get(0);
+  }
+  __device__ __forceinline__ uint4 next() {
+    issue();
+    cp_async_wait<RING - 1>();
+    return get(off);          // the slot after the one just refilled
+  }
+  __device__ __forceinline__ void end() const { cp_async_wait<0>(); }   // nothing in flight once the ring's memory is reused
+};
+
+// The interpreter.  A unit's operand addresses are ready before it starts; it
+// loads its operands, then the next group's ops, and turns those into addresses
+// while its FMAs are in flight.
+template <typename T>
+struct Pass {
+  uint32_t wb;
+  OpAddr A0, A1;              // the current group's ops
+  __device__ __forceinline__ void set(const uint4 &o) {
+    A0 = unpack(wb, make_uint2(o.x, o.y));
+    A1 = unpack(wb, make_uint2(o.z, o.w));
+  }
+  template <class S>
+  __device__ __forceinline__ void pair(S &st) {
+    T *const tag = nullptr;
+    const T a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
+    const T a2 = lds(tag, A1.a), b2 = lds(tag, A1.b), c2 = lds(tag, A1.c);
+    const uint4 o = st.next();
+    const T v = fma(a, b, c), v2 = fma(a2, b2, c2);
+    const uint32_t t = A0.t, t2 = A1.t;
+    set(o);
+    sts(t, v);
+    sts(t2, v2);
+    __syncwarp();
+  }
+  template <class S>
+  __device__ __forceinline__ void seq(S &st) {
+    T *const tag = nullptr;
+    {
+      const T a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
+      sts(A0.t, fma(a, b, c));
+      __syncwarp();
+    }
+    const T a = lds(tag, A1.a), b = lds(tag, A1.b), c = lds(tag, A1.c);
+    const uint4 o = st.next();
+    const T v = fma(a, b, c);
+    const uint32_t t = A1.t;
+    set(o);
+    sts(t, v);
+    __syncwarp();
+  }
+  template <class S>
+  __device__ __forceinline__ void one(S &st) {
+    T *const tag = nullptr;
+    const T a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
+    const uint4 o = st.next();
+    const T v = fma(a, b, c);
+    const uint32_t t = A0.t;
+    set(o);
+    sts(t, v);
+    __syncwarp();
+  }
+  template <class S>
+  __device__ __forceinline__ void recip(S &st) {
+    const uint4 o2 = st.next();
+    const OpAddr A2 = unpack(wb, make_uint2(o2.x, o2.y));
+    RecipUnit<T> ru;
+    ru.load_and_run(wb, A0, A1, A2);
+    const uint4 o = st.next();
+    ru.store(A0, A1, A2);
+    set(o);
+    __syncwarp();
+  }
+};
+
+// A program with a run table (in shared or global memory); RECIP: it has
+// reciprocals.  The loops are deliberately not unrolled: the kernels are bound by
+// instruction fetch as well.
+template <typename T, bool RECIP, class S>
+__device__ __forceinline__ void run_prog(S st, const uint32_t *runs, const int nruns, T *W) {
+  Pass<T> ps{smem_addr(W)};
+  ps.set(st.first());
 #pragma unroll 1
   for (int r = 0; r < nruns; ++r) {
-    const uint32_t rr = !WIDE && !RECIP ? (uint32_t)np : __ldg(runs + r);
-    const uint32_t kind = rr >> 28;
+    const uint32_t rr = runs[r], kind = rr >> 28;
     int n = (int)(rr & 0x0fffffffu);
-    if (WIDE && kind == RUN_FMA2) {
+    if (kind == RUN_FMA2) {
 #pragma unroll 1
-      for (; n > 0; --n, p += 2) {
-        issue(p + RING - 2);
-        issue(p + RING - 1);
-        cp_async_wait<RING - 4>();      // passes p + 2 and p + 3 have landed
-        if (p + 2 < np) r0 = fetch(p + 2);
-        if (p + 3 < np) r1 = fetch(p + 3);
-        const T a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
-        const T a2 = lds(tag, A1.a), b2 = lds(tag, A1.b), c2 = lds(tag, A1.c);
-        const T v = fma(a, b, c), v2 = fma(a2, b2, c2);
-        const uint32_t t = A0.t, t2 = A1.t;
-        A0 = unpack(wb, r0);
-        A1 = unpack(wb, r1);
-        sts(t, v);
-        sts(t2, v2);
-        __syncwarp();
-      }
+      for (; n > 0; --n) ps.pair(st);
     } else if (RECIP && kind == RUN_RECIP) {
 #pragma unroll 1
-      for (; n > 0; --n, p += 3) {
-        cp_async_wait<RING - 5>();      // pass p + 2 has landed
-        const OpAddr A2 = unpack(wb, fetch(p + 2));
-        RecipUnit<T> ru;
-        ru.load_and_run(wb, A0, A1, A2);
-        issue(p + RING - 2);
-        issue(p + RING - 1);
-        issue(p + RING);
-        cp_async_wait<RING - 4>();      // passes p + 3 and p + 4 have landed
-        if (p + 3 < np) r0 = fetch(p + 3);
-        if (p + 4 < np) r1 = fetch(p + 4);
-        ru.store(A0, A1, A2);
-        A0 = unpack(wb, r0);
-        A1 = unpack(wb, r1);
-        __syncwarp();
-      }
+      for (; n > 0; --n) ps.recip(st);
+    } else if (kind == RUN_SEQ2) {
+#pragma unroll 1
+      for (; n > 0; --n) ps.seq(st);
     } else {
 #pragma unroll 1
-      for (; n > 0; --n, ++p) {
-        issue(p + RING - 2);
-        cp_async_wait<RING - 4>();      // pass p + 2 has landed
-        if (p + 2 < np) r0 = fetch(p + 2);
-        const T a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
-        const T v = fma(a, b, c);
-        const uint32_t t = A0.t;
-        A0 = A1;
-        A1 = unpack(wb, r0);
-        sts(t, v);
-        __syncwarp();
-      }
+      for (; n > 0; --n) ps.one(st);
     }
   }
-  cp_async_wait<0>();                   // nothing in flight once the ring's memory is reused
+  st.end();
+}
+// A program of np single passes
+template <typename T, class S>
+__device__ __forceinline__ void run_single(S st, const int np, T *W) {
+  Pass<T> ps{smem_addr(W)};
+  ps.set(st.first());
+#pragma unroll 1
+  for (int n = np >> 1; n > 0; --n) ps.seq(st);
+#pragma unroll 1
+  for (int n = np & 1; n > 0; --n) ps.one(st);
+  st.end();
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -552,10 +567,16 @@ __device__ __forceinline__ void f_core(const MechDev &M, const SolveParams &P, c
   if (M.max_reac > 2) rates<3>(M, P, slots, wb, lane);
   else rates<2>(M, P, slots, wb, lane);
   __syncwarp();
-  run_prog<double, STAGED, true, false>(reinterpret_cast<const ushort4 *>(tbase + M.tab.f_ops),
-                                               reinterpret_cast<const uint32_t *>(tbase + M.tab.f_runs), M.f_nruns,
-                                               M.f_npass, Wd, lane);
+  const ushort4 *ops = reinterpret_cast<const ushort4 *>(tbase + M.tab.f_ops);
+  const uint32_t *runs = reinterpret_cast<const uint32_t *>(tbase + M.tab.f_runs);
+  if (STAGED) run_prog<double, false>(SmemStream(ops, lane), runs, M.f_nruns, Wd);
+  else run_prog<double, false>(GlobalStream(ops, lane), runs, M.f_nruns, Wd);
 }
+
+// The ring of a program streamed from global memory: the slots of the rates and f
+// in Wd, dead while M is factored and during a solve
+__device__ __forceinline__ bool ring_fits(const MechDev &M) { return (M.R + M.S) * 8 - 8 >= RING_BYTES; }
+__device__ __forceinline__ uint32_t ring_addr(const MechDev &M, const double *Wd) { return (smem_addr(Wd + M.d_RT) + 15u) & ~15u; }
 
 // -c dr_j/dy_l of the lane's (reaction, reactant) pairs, two per iteration as
 // the rates; NR as there
@@ -616,12 +637,11 @@ __device__ __forceinline__ void mlu_core(const MechDev &M, const SolveParams &P,
   // read from L2 two passes ahead.  The LU program's ops are streamed through a
   // ring in the rates and f slots of Wd, dead once M is formed (too small a
   // region: read from L2 as well).
-  run_prog<T, false, true, false>(M.m_ops[prec], M.m_runs, M.m_nruns, M.m_npass, reinterpret_cast<T *>(Wd), lane);
-  const uint32_t wr = smem_addr(Wd + M.d_RT);            // 8-byte aligned (a double slot)
-  if ((M.R + M.S) * 8 >= 8 * 256)
-    run_prog_ring<T, 8, true, true>(M.lu_ops[prec], M.lu_runs, M.lu_nruns, M.lu_npass, WL, lane, wr);
+  run_prog<T, false>(GlobalStream(M.m_ops[prec], lane), M.m_runs, M.m_nruns, reinterpret_cast<T *>(Wd));
+  if (ring_fits(M))
+    run_prog<T, true>(RingStream(M.lu_ops[prec], lane, ring_addr(M, Wd)), M.lu_runs, M.lu_nruns, WL);
   else
-    run_prog<T, false, true, true>(M.lu_ops[prec], M.lu_runs, M.lu_nruns, M.lu_npass, WL, lane);
+    run_prog<T, true>(GlobalStream(M.lu_ops[prec], lane), M.lu_runs, M.lu_nruns, WL);
 }
 
 // a5: forward and backward substitution with the LDU factors on the vector in
@@ -636,17 +656,15 @@ __device__ __forceinline__ void solve_core(const MechDev &M, const unsigned char
   const ushort4 *bwd = reinterpret_cast<const ushort4 *>(tbase + M.tab.bwd_ops);
   T *const W = reinterpret_cast<T *>(Wd);                 // the programs address the whole per-cell slice
   if (STAGED) {
-    run_prog<T, true, false, false>(fwd, nullptr, 1, M.fwd_npass, W, lane);
-    run_prog<T, true, false, false>(bwd, nullptr, 1, M.bwd_npass, W, lane);
-    return;
-  }
-  const uint32_t rb = smem_addr(Wd + M.d_RT);            // the rates and f slots: dead during a solve
-  if ((M.R + M.S) * 8 >= 8 * 256) {
-    run_prog_ring<T, 8, false, false>(fwd, nullptr, 1, M.fwd_npass, W, lane, rb);
-    run_prog_ring<T, 8, false, false>(bwd, nullptr, 1, M.bwd_npass, W, lane, rb);
+    run_single<T>(SmemStream(fwd, lane), M.fwd_npass, W);
+    run_single<T>(SmemStream(bwd, lane), M.bwd_npass, W);
+  } else if (ring_fits(M)) {
+    const uint32_t rb = ring_addr(M, Wd);
+    run_single<T>(RingStream(fwd, lane, rb), M.fwd_npass, W);
+    run_single<T>(RingStream(bwd, lane, rb), M.bwd_npass, W);
   } else {
-    run_prog<T, false, false, false>(fwd, nullptr, 1, M.fwd_npass, W, lane);
-    run_prog<T, false, false, false>(bwd, nullptr, 1, M.bwd_npass, W, lane);
+    run_single<T>(GlobalStream(fwd, lane), M.fwd_npass, W);
+    run_single<T>(GlobalStream(bwd, lane), M.bwd_npass, W);
   }
 }
 
@@ -1333,7 +1351,7 @@ __device__ bool stage_tables(const unsigned char *blob, int bytes, unsigned char
 }
 
 template <typename T, int KS, bool STAGED, bool REC, bool COUPLED>
-__global__ void __launch_bounds__(MAX_WARPS_PER_BLOCK * WARP) solve_kernel(const __grid_constant__ MechDev M, const CellsDev C, const SolveParams P) {
+__global__ void __launch_bounds__(MAX_WARPS_PER_BLOCK * WARP, 1) solve_kernel(const __grid_constant__ MechDev M, const CellsDev C, const SolveParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(8) uint64_t tma_bar;
   __shared__ double grp_slot[COUPLED ? MAX_WARPS_PER_BLOCK : 1];
@@ -1654,8 +1672,8 @@ __device__ __forceinline__ void jt_and_theta(const MechDev &M, const SolveParams
   for (int k = 0; k < KS; ++k)
     if (own[k]) Wd[M.a_MU + lane + WARP * k] = v[k];
   __syncwarp();
-  run_prog<double, false, true, false>(M.nudot_ops, M.nudot_runs, M.nudot_nruns, M.nudot_npass, Wd, lane);
-  run_prog<double, false, true, false>(M.jt_ops, M.jt_runs, M.jt_nruns, M.jt_npass, Wd, lane);
+  run_prog<double, false>(GlobalStream(M.nudot_ops, lane), M.nudot_runs, M.nudot_nruns, Wd);
+  run_prog<double, false>(GlobalStream(M.jt_ops, lane), M.jt_runs, M.jt_nruns, Wd);
 #pragma unroll 2
   for (int j = lane; j < M.R; j += WARP)
     Wd[M.a_G + j] = fma(Opaque{P}.mul(scale, Wd[M.d_RT + j]), Wd[M.a_NM + j], Wd[M.a_G + j]);
@@ -1772,8 +1790,8 @@ __device__ void backward_cell(const MechDev &M, const CellsDev &C, const AdjDev 
       for (int k = 0; k < KS; ++k)
         if (cl.own[k]) Wd[M.d_Y + cl.pos[k]] = lamd[k];   // the solve vector: y's slots (y was consumed)
       __syncwarp();
-      run_prog<double, false, false, false>(M.fwdT_ops, nullptr, 1, M.fwdT_npass, Wd, lane);
-      run_prog<double, false, false, false>(M.bwdT_ops, nullptr, 1, M.bwdT_npass, Wd, lane);
+      run_single<double>(GlobalStream(M.fwdT_ops, lane), M.fwdT_npass, Wd);
+      run_single<double>(GlobalStream(M.bwdT_ops, lane), M.bwdT_npass, Wd);
 #pragma unroll
       for (int k = 0; k < KS; ++k) g[k] = cl.own[k] ? op.mul(neg_i(ss), Wd[M.d_Y + cl.pos[k]]) : 0.0;   // the programs leave -M^{-T} lambda
       __syncwarp();
@@ -1904,8 +1922,7 @@ __device__ __forceinline__ void tangent_f(const MechDev &M, const Tabs &tb, doub
     Wd[M.d_RT + j] = sj;
   }
   __syncwarp();
-  run_prog<double, false, true, false>(tab<ushort4>(tb, M.tab.f_ops), tab<uint32_t>(tb, M.tab.f_runs), M.f_nruns,
-                                              M.f_npass, Wd, lane);
+  run_prog<double, false>(GlobalStream(tab<ushort4>(tb, M.tab.f_ops), lane), tab<uint32_t>(tb, M.tab.f_runs), M.f_nruns, Wd);
 #pragma unroll
   for (int k = 0; k < KS; ++k) out[k] = own[k] ? Wd[M.d_F + lane + WARP * k] : 0.0;
   __syncwarp();

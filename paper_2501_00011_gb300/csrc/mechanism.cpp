@@ -926,23 +926,40 @@ int put(Mechanism &m, const std::vector<T> &v, const T **dst, std::string &msg) 
   return 0;
 }
 
-// Device form of a program: byte offsets (off(element index)), empty slots as
-// FMAs into the dummy slot, RECIP ops marked by c == DEV_RECIP.
+// Device form of a program (groups of two passes): byte offsets (off(element
+// index)), empty slots as FMAs into the dummy slot, RECIP ops marked by
+// c == DEV_RECIP.  pad: groups of harmless ops after the last.
 template <typename Off>
-std::vector<ushort4> device_ops_at(const HostProgram &hp, Off off, int dummy, int zero) {
-  std::vector<ushort4> v(hp.ops.size());
-  for (size_t i = 0; i < v.size(); ++i) {
-    const Op &o = hp.ops[i];
-    if (o.t == OP_EMPTY) v[i] = make_ushort4(off(dummy), off(zero), off(zero), off(zero));
-    else if (o.t & OP_RECIP) v[i] = make_ushort4(off(o.t & 0x7fff), off(o.a), 0, DEV_RECIP);
-    else v[i] = make_ushort4(off(o.t), off(o.a), off(o.b), off(o.c));
-  }
+std::vector<ushort4> device_ops_at(const HostProgram &hp, Off off, int dummy, int zero, int pad = 0) {
+  std::vector<std::pair<int, int>> g;
+  std::vector<uint32_t> runs;
+  hp.groups(g, runs);
+  const ushort4 empty = make_ushort4(off(dummy), off(zero), off(zero), off(zero));
+  std::vector<ushort4> v((g.size() + pad) * 2 * WARP, empty);
+  for (size_t i = 0; i < g.size(); ++i)
+    for (int h = 0; h < 2; ++h) {
+      const int p = h ? g[i].second : g[i].first;
+      if (p < 0) continue;
+      for (int l = 0; l < WARP; ++l) {
+        const Op &o = hp.ops[(size_t)p * WARP + l];
+        if (o.t == OP_EMPTY) continue;
+        v[(i * WARP + l) * 2 + h] = (o.t & OP_RECIP) ? make_ushort4(off(o.t & 0x7fff), off(o.a), 0, DEV_RECIP)
+                                                     : make_ushort4(off(o.t), off(o.a), off(o.b), off(o.c));
+      }
+    }
   return v;
 }
 
 // ... with byte offsets elem * index from the program's own array
-std::vector<ushort4> device_ops(const HostProgram &hp, int elem, int dummy, int zero) {
-  return device_ops_at(hp, [elem](int e) { return (unsigned short)(e * elem); }, dummy, zero);
+std::vector<ushort4> device_ops(const HostProgram &hp, int elem, int dummy, int zero, int pad = 0) {
+  return device_ops_at(hp, [elem](int e) { return (unsigned short)(e * elem); }, dummy, zero, pad);
+}
+
+std::vector<uint32_t> device_runs(const HostProgram &hp) {
+  std::vector<std::pair<int, int>> g;
+  std::vector<uint32_t> runs;
+  hp.groups(g, runs);
+  return runs;
 }
 
 // polynomial coefficients (in eta) of R(eta)_{jm} = prod_{l<m} (l - j eta)/(l+1)
@@ -1015,7 +1032,7 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
     BlobWriter bw;
     TableOffsets t;
     t.f_ops = bw.add(device_ops(m.f_prog, 8, d.d_DUMMY, d.d_ZERO));
-    t.f_runs = bw.add(m.f_prog.runs());
+    t.f_runs = bw.add(device_runs(m.f_prog));
     // the M and solve programs run on the whole per-cell slice: WL slots after Wd
     // (rounded to an even length), the pair products in Wd from the rates' first
     // slot, the solve vector in y's slots
@@ -1025,9 +1042,10 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
                               : e >= X_VIRTUAL ? x_off + (e - X_VIRTUAL) * el
                                                : wl_off + e * el);
     };
-    const std::vector<ushort4> m_dev = device_ops_at(m.m_prog, coff, d.L_DUMMY, d.L_ZERO);
+    const std::vector<ushort4> m_dev = device_ops_at(m.m_prog, coff, d.L_DUMMY, d.L_ZERO, PAD_GROUPS);
     t.fwd_ops = bw.add(device_ops_at(m.fwd_prog, coff, d.L_DUMMY, d.L_ZERO));
     t.bwd_ops = bw.add(device_ops_at(m.bwd_prog, coff, d.L_DUMMY, d.L_ZERO));
+    const int bwd_end = (int)bw.buf.size();
     std::vector<uint2> slots(R);
     for (int j = 0; j < R; ++j)
       slots[j] = make_uint2((unsigned)(m.rx_slot_idx[j * 3] * 8) | ((unsigned)(m.rx_slot_idx[j * 3 + 1] * 8) << 16),
@@ -1041,6 +1059,8 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
     std::vector<int> diag(S);
     for (int k = 0; k < S; ++k) diag[k] = m.lu_diag[k] * el;
     t.lu_diag = bw.add(diag);
+    // one readable group past the last staged program (the interpreter reads ahead)
+    while ((int)bw.buf.size() < bwd_end + GROUP_BYTES) bw.add(std::vector<uint32_t>(4, 0u));
     t.staged = (int)bw.buf.size();         // the rest is read from global memory
     std::vector<int> doff(m.d_consts_i.size()), loff(m.L_consts_i.size());
     for (size_t k = 0; k < doff.size(); ++k) doff[k] = m.d_consts_i[k] * 8;
@@ -1053,13 +1073,15 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
     t.thr3 = bw.add(thr3);
     t.g = bw.add(g);
     t.lim = bw.add(lim);
+    // ... and PAD_GROUPS when the programs are read from global memory
+    while ((int)bw.buf.size() < bwd_end + PAD_GROUPS * GROUP_BYTES) bw.add(std::vector<uint32_t>(4, 0u));
     t.bytes = (int)bw.buf.size();
     d.tab = t;
     int rc = put(m, bw.buf, &d.blob[prec], msg);
     if (!rc) rc = put(m, m_dev, &d.m_ops[prec], msg);
-    if (!rc) rc = put(m, device_ops(m.lu_prog, el, d.L_DUMMY, d.L_ZERO), &d.lu_ops[prec], msg);
-    if (!rc && prec == 0) rc = put(m, m.m_prog.runs(), &d.m_runs, msg);
-    if (!rc && prec == 0) rc = put(m, m.lu_prog.runs(), &d.lu_runs, msg);
+    if (!rc) rc = put(m, device_ops(m.lu_prog, el, d.L_DUMMY, d.L_ZERO, PAD_GROUPS), &d.lu_ops[prec], msg);
+    if (!rc && prec == 0) rc = put(m, device_runs(m.m_prog), &d.m_runs, msg);
+    if (!rc && prec == 0) rc = put(m, device_runs(m.lu_prog), &d.lu_runs, msg);
     if (rc) {
       free_mechanism(m);
       return rc;
@@ -1073,30 +1095,25 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
     std::vector<int> aoff(m.a_consts_i.size());
     for (size_t k = 0; k < aoff.size(); ++k) aoff[k] = m.a_consts_i[k] * 8;
     if ((rc = put(m, aoff, &d.a_const_off, msg)) || (rc = put(m, m.a_consts_v, &d.a_const_val, msg)) ||
-        (rc = put(m, device_ops(m.nudot_prog, 8, d.d_DUMMY, d.d_ZERO), &d.nudot_ops, msg)) ||
-        (rc = put(m, device_ops(m.jt_prog, 8, d.d_DUMMY, d.d_ZERO), &d.jt_ops, msg)) ||
-        (rc = put(m, device_ops_at(m.fwdT_prog, xoff64, d.L_DUMMY, d.L_ZERO), &d.fwdT_ops, msg)) ||
-        (rc = put(m, device_ops_at(m.bwdT_prog, xoff64, d.L_DUMMY, d.L_ZERO), &d.bwdT_ops, msg)) ||
-        (rc = put(m, m.nudot_prog.runs(), &d.nudot_runs, msg)) || (rc = put(m, m.jt_prog.runs(), &d.jt_runs, msg))) {
+        (rc = put(m, device_ops(m.nudot_prog, 8, d.d_DUMMY, d.d_ZERO, PAD_GROUPS), &d.nudot_ops, msg)) ||
+        (rc = put(m, device_ops(m.jt_prog, 8, d.d_DUMMY, d.d_ZERO, PAD_GROUPS), &d.jt_ops, msg)) ||
+        (rc = put(m, device_ops_at(m.fwdT_prog, xoff64, d.L_DUMMY, d.L_ZERO, PAD_GROUPS), &d.fwdT_ops, msg)) ||
+        (rc = put(m, device_ops_at(m.bwdT_prog, xoff64, d.L_DUMMY, d.L_ZERO, PAD_GROUPS), &d.bwdT_ops, msg)) ||
+        (rc = put(m, device_runs(m.nudot_prog), &d.nudot_runs, msg)) || (rc = put(m, device_runs(m.jt_prog), &d.jt_runs, msg))) {
       free_mechanism(m);
       return rc;
     }
     d.a_nconst = (int)m.a_consts_v.size();
-    d.nudot_npass = m.nudot_prog.n_pass();
-    d.jt_npass = m.jt_prog.n_pass();
     d.fwdT_npass = m.fwdT_prog.n_pass();
     d.bwdT_npass = m.bwdT_prog.n_pass();
-    d.nudot_nruns = (int)m.nudot_prog.runs().size();
-    d.jt_nruns = (int)m.jt_prog.runs().size();
+    d.nudot_nruns = (int)device_runs(m.nudot_prog).size();
+    d.jt_nruns = (int)device_runs(m.jt_prog).size();
   }
-  d.f_npass = m.f_prog.n_pass();
-  d.f_nruns = (int)m.f_prog.runs().size();
-  d.m_nruns = (int)m.m_prog.runs().size();
-  d.lu_nruns = (int)m.lu_prog.runs().size();
+  d.f_nruns = (int)device_runs(m.f_prog).size();
+  d.m_nruns = (int)device_runs(m.m_prog).size();
+  d.lu_nruns = (int)device_runs(m.lu_prog).size();
   d.fwd_npass = m.fwd_prog.n_pass();
   d.bwd_npass = m.bwd_prog.n_pass();
-  d.m_npass = m.m_prog.n_pass();
-  d.lu_npass = m.lu_prog.n_pass();
   d.d_nconst = (int)m.d_consts_v.size();
   d.L_nconst = (int)m.L_consts_v.size();
 
