@@ -276,7 +276,7 @@ int chem_get_state(const chem_cells *cells, double *y, int32_t mem, void *stream
  * (solver iterations).  Errors: CHEM_EINVAL, CHEM_ECUDA. */
 int chem_get_stats(const chem_cells *cells, chem_cell_stats *out, int32_t mem, void *stream);
 /* Staging counters of the last chem_solve_step / chem_solve_steps call on the
- * batch (persistent driver; every step of a graph launch): *fallbacks = blocks
+ * batch (persistent driver; counted for every step a launch takes): *fallbacks = blocks
  * whose bulk copy of the tables into shared memory was not seen to land within
  * the bounded wait (they copied the tables with ordinary loads: same results);
  * *unfinished = blocks that exited before such a late copy was seen to land

@@ -415,9 +415,10 @@ LaunchCfg launch_cfg(const chem_opts &o, double dt) {
   return cfg;
 }
 
-// One solve of every cell on stream s: queue reset (persistent driver) and
-// the solve kernel.  Stream-ordered calls only, so it can be captured.
-cudaError_t enqueue_solve(chem_cells *c, double dt, cudaStream_t s) {
+// One solve of every cell on stream s (n_steps consecutive steps of each): queue
+// reset (persistent driver) and the solve kernel.  Stream-ordered calls only, so
+// it can be captured.
+cudaError_t enqueue_solve(chem_cells *c, double dt, cudaStream_t s, int n_steps = 1) {
   CellsDev cd = solve_dev(c);
   if (c->opts.driver == CHEM_DRIVER_PERSISTENT) {
     cudaError_t e = cudaMemsetAsync(c->counters, 0, sizeof(unsigned long long), s);
@@ -436,7 +437,9 @@ cudaError_t enqueue_solve(chem_cells *c, double dt, cudaStream_t s) {
       cd.order = c->order;
     }
   }
-  return launch_solve(c->mech->m.dev, cd, launch_cfg(c->opts, dt), s);
+  LaunchCfg cfg = launch_cfg(c->opts, dt);
+  cfg.n_steps = n_steps;
+  return launch_solve(c->mech->m.dev, cd, cfg, s);
 }
 
 int check_solve_args(chem_cells *c, double dt) {
@@ -487,7 +490,13 @@ int chem_solve_steps(chem_cells *c, double dt, int32_t n_steps, void *stream) {
     if ((e = cudaStreamBeginCapture(c->capture_stream, cudaStreamCaptureModeRelaxed)) != cudaSuccess)
       return cuda_fail(e, "begin capture");
     cudaError_t le = clear_stage_counters(c, c->capture_stream);
-    for (int k = 0; k < n_steps && le == cudaSuccess; ++k) le = enqueue_solve(c, dt, c->capture_stream);
+    // independent cells take their steps one after the other inside one launch;
+    // coupled groups one launch per step
+    if (c->opts.couple_cells > 1) {
+      for (int k = 0; k < n_steps && le == cudaSuccess; ++k) le = enqueue_solve(c, dt, c->capture_stream);
+    } else if (le == cudaSuccess) {
+      le = enqueue_solve(c, dt, c->capture_stream, n_steps);
+    }
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(c->capture_stream, &g);
     if (le != cudaSuccess) {

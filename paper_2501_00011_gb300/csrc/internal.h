@@ -276,6 +276,7 @@ struct LaunchCfg {
   int blocks_per_sm;
   double rtol, atol, dt;
   int max_order, max_steps;
+  int n_steps;          // > 1: that many consecutive steps per cell in one launch (not coupled)
   long long stage_wait; // iterations of the first wait for the staged tables (chem_opts.stage_wait)
 };
 

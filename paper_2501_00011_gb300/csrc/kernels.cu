@@ -44,6 +44,7 @@ constexpr int ORDER_WARPS = 8;          // cells per block of the queue-order ke
 struct SolveParams {
   double rtol, atol, dt;
   int max_order, max_steps;
+  int n_steps = 1;     // consecutive steps of dt per cell
   int cell_bytes;      // shared memory per warp
   int wd_pad;          // Wd length rounded so WL starts 16-byte aligned
   int warps_per_block;
@@ -831,7 +832,7 @@ __device__ __forceinline__ void accept_update(const SolveParams &P, double (&D)[
 // T, P are not positive.
 template <int KS>
 __device__ __forceinline__ bool load_cell(const MechDev &M, const CellsDev &C, double *Wd, const int lane, const int64_t cell,
-                          const bool (&own)[KS], double (&y0)[KS]) {
+                          const bool (&own)[KS], double (&y0)[KS], const bool have_rates = false) {
   const int64_t NC = C.n_cells;
   const int R = M.R;
   const double Tc = C.T[cell], Pc = C.P[cell];
@@ -840,6 +841,11 @@ __device__ __forceinline__ bool load_cell(const MechDev &M, const CellsDev &C, d
   for (int k = 0; k < KS; ++k) {
     y0[k] = own[k] ? C.y[(int64_t)(lane + WARP * k) * NC + cell] : 0.0;
     if (own[k] && !isfinite(y0[k])) bad = true;
+  }
+  if (have_rates) {          // Wd[KT] holds them from the cell's step before (T, P, J and theta are the same)
+    bad = __any_sync(FULL, bad);
+    __syncwarp();
+    return bad;
   }
   if (!__any_sync(FULL, bad)) {
     const double n_air = air_number_density(Tc, Pc);
@@ -983,9 +989,9 @@ struct Recorder {
 // thr3, lim); coupled, the group's sums are first scaled by gsc = 1/(cells
 // in the group).
 template <typename T, int KS, bool STAGED, bool REC, bool COUPLED>
-__device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, const SolveParams &P, const Tabs &tb, double *Wd,
+__device__ __forceinline__ bool solve_cell(const MechDev &M, const CellsDev &C, const SolveParams &P, const Tabs &tb, double *Wd,
                            T *WL, const int lane, const int64_t cell, const Grp<COUPLED> &grp, const double invN,
-                           const double gsc) {
+                           const double gsc, const bool have_rates = false) {
   const int64_t NC = C.n_cells;
   chem_cell_stats st = {};
   int status = CHEM_CELL_OK;
@@ -1000,7 +1006,7 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
   double y0[KS];
 #pragma unroll
   for (int k = 0; k < KS; ++k) y0[k] = 0.0;
-  const bool bad = grp.any(phantom ? false : load_cell<KS>(M, C, Wd, lane, cell, cl.own, y0));
+  const bool bad = grp.any(phantom ? false : load_cell<KS>(M, C, Wd, lane, cell, cl.own, y0, have_rates));
   Recorder<KS, REC> rec(C, cell, M.S);
 
   const Opaque op{P};
@@ -1322,6 +1328,7 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
     C.stats[cell] = st;
   }
   __syncwarp();
+  return !bad;         // the inputs were usable: the rate constants in Wd are whole
 }
 
 // Stage the table blob into the first `bytes` of shared memory with one TMA
@@ -1332,7 +1339,7 @@ __device__ __forceinline__ void solve_cell(const MechDev &M, const CellsDev &C, 
 // waits (bounded again) for that copy before it exits.  Keeping the tables in
 // shared memory on both paths lets every table read use shared-memory loads.
 __device__ bool stage_tables(const unsigned char *blob, int bytes, unsigned char *smem, uint64_t *bar,
-                             unsigned long long *stage, long long limit) {
+                             unsigned long long *stage, long long limit, int n_steps) {
   if (threadIdx.x == 0) mbar_init(bar, 1);
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -1345,7 +1352,8 @@ __device__ bool stage_tables(const unsigned char *blob, int bytes, unsigned char
     uint4 *dst = reinterpret_cast<uint4 *>(smem);
     for (int i = threadIdx.x; i < bytes / 16; i += blockDim.x) dst[i] = __ldg(src + i);
     __syncthreads();
-    if (threadIdx.x == 0 && stage) atomicAdd(stage, 1ull);
+    // (a staging serves all the launch's steps and counts for each)
+    if (threadIdx.x == 0 && stage) atomicAdd(stage, (unsigned long long)n_steps);
   }
   return ok;
 }
@@ -1362,7 +1370,7 @@ __global__ void __launch_bounds__(MAX_WARPS_PER_BLOCK * WARP, 1) solve_kernel(co
   tb.gbase = M.blob[P.prec];
   bool staged_ok = true;
   if (STAGED) {
-    staged_ok = stage_tables(M.blob[P.prec], P.tab_bytes, smem, &tma_bar, C.stage, P.stage_wait);
+    staged_ok = stage_tables(M.blob[P.prec], P.tab_bytes, smem, &tma_bar, C.stage, P.stage_wait, P.n_steps);
     tb.base = smem;
   } else {
     tb.base = M.blob[P.prec];
@@ -1371,6 +1379,16 @@ __global__ void __launch_bounds__(MAX_WARPS_PER_BLOCK * WARP, 1) solve_kernel(co
   T *WL = reinterpret_cast<T *>(Wd + P.wd_pad);
   Grp<COUPLED> grp;
   const double invS = 1.0 / (double)M.S;
+  // A cell's consecutive steps one after the other: its rate constants stay in
+  // shared memory, and the batch has one load-imbalance tail instead of one per
+  // step.  Each step starts from the y it finds, as a launch of its own would; a
+  // cell whose rate constants are not all finite fails every step alike.
+  auto cell_steps = [&](const int64_t cell) {
+    bool ok = false;
+#pragma unroll 1
+    for (int k = 0; k < P.n_steps; ++k)
+      ok = solve_cell<T, KS, STAGED, REC, COUPLED>(M, C, P, tb, Wd, WL, lane, cell, grp, invS, 1.0, ok);
+  };
   if (COUPLED) {
     // groups of P.couple consecutive cells, P.warps_per_block / P.couple per
     // block, each with named barrier 1 + its index; with the queue, groups are
@@ -1405,17 +1423,17 @@ __global__ void __launch_bounds__(MAX_WARPS_PER_BLOCK * WARP, 1) solve_kernel(co
       cell = __shfl_sync(FULL, cell, 0);
       if (cell >= C.n_cells) break;
       if (C.order) cell = __ldg(C.order + cell);
-      solve_cell<T, KS, STAGED, REC, COUPLED>(M, C, P, tb, Wd, WL, lane, cell, grp, invS, 1.0);
+      cell_steps(cell);
     }
   } else {
     const int64_t cell = (int64_t)blockIdx.x * P.warps_per_block + warp;
-    if (cell < C.n_cells) solve_cell<T, KS, STAGED, REC, COUPLED>(M, C, P, tb, Wd, WL, lane, cell, grp, invS, 1.0);
+    if (cell < C.n_cells) cell_steps(cell);
   }
   // a late bulk copy must land before the block exits (its shared memory is
   // then handed to another block); one thread waits, bounded, and counts a
   // wait that ran out in stage[1]
   if (STAGED && !staged_ok && threadIdx.x == 0) {
-    if (!mbar_wait(&tma_bar, 0, STAGE_WAIT_DEFAULT) && C.stage) atomicAdd(C.stage + 1, 1ull);
+    if (!mbar_wait(&tma_bar, 0, STAGE_WAIT_DEFAULT) && C.stage) atomicAdd(C.stage + 1, (unsigned long long)P.n_steps);
   }
 }
 
@@ -2714,6 +2732,8 @@ cudaError_t launch_solve(const MechDev &M, const CellsDev &C, const LaunchCfg &c
   P.dt = cfg.dt;
   P.max_order = cfg.max_order;
   P.max_steps = cfg.max_steps;
+  P.n_steps = cfg.n_steps > 1 ? cfg.n_steps : 1;
+  if (P.n_steps > 1 && cfg.couple > 1) return cudaErrorInvalidValue;     // coupled groups take one step per launch
   P.wd_pad = (M.Wd_len + 1) & ~1;
   P.cell_bytes = (int)smem_per_cell(M, cfg.lu_precision);
   P.warps_per_block = cfg.warps_per_block;
