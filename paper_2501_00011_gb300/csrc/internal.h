@@ -136,49 +136,61 @@ struct MechDev {
 // 32 x (op of the first pass, op of the second), so one 16-byte load brings a
 // lane's ops of both.  Its run table holds one uint32 per run of equal groups
 // (kind << 28 | groups):
-//   RUN_SEQ2   two passes, one after the other
-//   RUN_FMA2   a pair: 64 mutually independent FMAs; the operands of both passes
-//              are loaded before either result is stored, so a lane has two FMAs
-//              in flight between warp synchronisations
+//   RUN_PIPE   groups of passes none of which touches what the one before it
+//              writes: each pass's operands are loaded while the FMAs of the one
+//              before are in flight
+//   RUN_PIPE1  the same, the last group with one pass (the second slot not used)
+//   RUN_SEQ    groups of two passes, the second after the first
+//   RUN_ONE    one pass (the second slot not used)
 //   RUN_RECIP  two groups, three passes, reciprocals in the first: a lane with a
 //              reciprocal spends three FP64 instructions on it and has no op in the
 //              other two, every other lane runs its three FMA ops; all ops of the
 //              unit are independent of each other
-//   RUN_FMA1   one pass (the second op slot is not used)
-constexpr uint32_t RUN_SEQ2 = 0, RUN_FMA2 = 1, RUN_RECIP = 2, RUN_FMA1 = 3;
+// A program without runs (the triangular solves) is its passes in order.
+constexpr uint32_t RUN_PIPE = 0, RUN_PIPE1 = 1, RUN_RECIP = 2, RUN_SEQ = 3, RUN_ONE = 4;
 constexpr int GROUP_BYTES = 2 * WARP * 8;
 constexpr int PAD_GROUPS = 5;     // readable groups past a program's last (the interpreters read ahead unconditionally)
 
 struct HostProgram {
   std::vector<Op> ops;   // n_pass * 32
-  // per pass: 0 single FMA pass, 1 / 2 first / second pass of a pair, 3 the
-  // first pass of a reciprocal unit (the two passes after it, marked 0, belong to it)
+  // per pass: 3 the first pass of a reciprocal unit (the two passes after it,
+  // marked 0, belong to it), 0 otherwise
   std::vector<uint8_t> unit;
+  // per pass: 1 the first pass of a run, 2 a pass that continues it (it touches
+  // nothing the pass before it writes), 0 a pass outside runs
+  std::vector<uint8_t> run;
   int n_ops = 0;
   int n_pass() const { return (int)(ops.size() / WARP); }
   // the device form's groups: the passes in each (-1: none), and the run table
   void groups(std::vector<std::pair<int, int>> &g, std::vector<uint32_t> &runs) const {
-    auto push = [&](uint32_t kind, int a, int b) {
-      g.push_back({a, b});
-      if (!runs.empty() && runs.back() >> 28 == kind) runs.back()++;
-      else runs.push_back(kind << 28 | 1u);
-    };
     for (int p = 0; p < (int)unit.size();) {
-      if (unit[p] == 1) {
-        push(RUN_FMA2, p, p + 1);
-        p += 2;
-      } else if (unit[p] == 3) {
-        push(RUN_RECIP, p, p + 1);       // runs count units: two groups each
+      if (unit[p] == 3) {
+        if (!runs.empty() && runs.back() >> 28 == RUN_RECIP) runs.back()++;      // units of two groups
+        else runs.push_back(RUN_RECIP << 28 | 1u);
+        g.push_back({p, p + 1});
         g.push_back({p + 2, -1});
         p += 3;
-      } else if (p + 1 < (int)unit.size() && unit[p + 1] == 0) {
-        push(RUN_SEQ2, p, p + 1);
-        p += 2;
-      } else {
-        push(RUN_FMA1, p, -1);
-        p += 1;
+        continue;
       }
+      // [p, e): a run; or passes that each start one (outside runs: the rest)
+      auto starts = [&](int x) { return x < (int)unit.size() && unit[x] != 3 && run[x] != 2; };
+      int e = p + 1;
+      const bool alone = !(e < (int)unit.size() && run[e] == 2);
+      if (alone)
+        while (starts(e) && !(e + 1 < (int)unit.size() && run[e + 1] == 2)) ++e;
+      else
+        while (e < (int)unit.size() && run[e] == 2) ++e;
+      const uint32_t n = (uint32_t)(e - p);
+      if (!alone) {
+        runs.push_back((n & 1 ? RUN_PIPE1 : RUN_PIPE) << 28 | (n + 1) / 2);
+      } else {
+        if (n > 1) runs.push_back(RUN_SEQ << 28 | n / 2);
+        if (n & 1) runs.push_back(RUN_ONE << 28 | 1u);
+      }
+      for (; p < e; p += 2) g.push_back({p, p + 1 < e ? p + 1 : -1});
+      p = e;
     }
+    runs.push_back(0u);        // the interpreter reads an entry ahead
   }
 };
 

@@ -276,18 +276,44 @@ struct Pass {
     A0 = unpack(wb, make_uint2(o.x, o.y));
     A1 = unpack(wb, make_uint2(o.z, o.w));
   }
+  // n groups (the last with one pass if `odd`) of a run: a pass's operands are
+  // loaded before the results of the pass before it are stored, which they do not
+  // touch, so an FMA is in flight nearly all the time
   template <class S>
-  __device__ __forceinline__ void pair(S &st) {
+  __device__ __forceinline__ void pipe(S &st, int n, const bool odd) {
     T *const tag = nullptr;
-    const T a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
-    const T a2 = lds(tag, A1.a), b2 = lds(tag, A1.b), c2 = lds(tag, A1.c);
-    const uint4 o = st.next();
-    const T v = fma(a, b, c), v2 = fma(a2, b2, c2);
-    const uint32_t t = A0.t, t2 = A1.t;
-    set(o);
-    sts(t, v);
-    sts(t2, v2);
-    __syncwarp();
+    T a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
+#pragma unroll 1
+    for (; n > 1; --n) {
+      const T v = fma(a, b, c);
+      const T a2 = lds(tag, A1.a), b2 = lds(tag, A1.b), c2 = lds(tag, A1.c);
+      const uint4 o = st.next();
+      const uint32_t t = A0.t, t2 = A1.t;
+      sts(t, v);
+      __syncwarp();
+      const T v2 = fma(a2, b2, c2);
+      set(o);
+      a = lds(tag, A0.a), b = lds(tag, A0.b), c = lds(tag, A0.c);
+      sts(t2, v2);
+      __syncwarp();
+    }
+    // the last group: what comes next may read what it writes
+    const T v = fma(a, b, c);
+    if (odd) {
+      const uint4 o = st.next();
+      sts(A0.t, v);
+      __syncwarp();
+      set(o);
+    } else {
+      const T a2 = lds(tag, A1.a), b2 = lds(tag, A1.b), c2 = lds(tag, A1.c);
+      const uint4 o = st.next();
+      sts(A0.t, v);
+      const T v2 = fma(a2, b2, c2);
+      const uint32_t t2 = A1.t;
+      set(o);
+      sts(t2, v2);
+      __syncwarp();
+    }
   }
   template <class S>
   __device__ __forceinline__ void seq(S &st) {
@@ -335,23 +361,23 @@ struct Pass {
 template <typename T, bool RECIP, class S>
 __device__ __forceinline__ void run_prog(S st, const uint32_t *runs, const int nruns, T *W) {
   Pass<T> ps{smem_addr(W)};
+  uint32_t ahead = runs[0];
   ps.set(st.first());
 #pragma unroll 1
   for (int r = 0; r < nruns; ++r) {
-    const uint32_t rr = runs[r], kind = rr >> 28;
+    const uint32_t rr = ahead, kind = rr >> 28;
     int n = (int)(rr & 0x0fffffffu);
-    if (kind == RUN_FMA2) {
-#pragma unroll 1
-      for (; n > 0; --n) ps.pair(st);
-    } else if (RECIP && kind == RUN_RECIP) {
+    ahead = runs[r + 1];
+    if (RECIP && kind == RUN_RECIP) {
 #pragma unroll 1
       for (; n > 0; --n) ps.recip(st);
-    } else if (kind == RUN_SEQ2) {
+    } else if (kind <= RUN_PIPE1) {
+      ps.pipe(st, n, kind == RUN_PIPE1);
+    } else if (kind == RUN_SEQ) {
 #pragma unroll 1
       for (; n > 0; --n) ps.seq(st);
     } else {
-#pragma unroll 1
-      for (; n > 0; --n) ps.one(st);
+      ps.one(st);
     }
   }
   st.end();

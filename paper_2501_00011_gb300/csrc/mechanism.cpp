@@ -91,8 +91,8 @@ struct Scheduler {
     const int r[1] = {a};
     add(Op{(uint16_t)(t | OP_RECIP), (uint16_t)a, 0, 0}, 1, r, 1, t);
   }
-  // wide: ops may also be packed 64 at a time into pairs of passes (when at
-  // least 64 are ready, all of them mutually independent)
+  // wide: the passes form runs (HostProgram::run) in which no pass touches what
+  // the one before it writes, and reciprocal units
   HostProgram finish(bool wide = false) const {
     const int n = (int)rec_op.size();
     std::vector<std::vector<int>> succ(n);
@@ -109,24 +109,36 @@ struct Scheduler {
       for (int s2 : succ[i]) h = std::max(h, height[s2]);
       height[i] = h + (rec_kind[i] ? RECIP_WEIGHT : 1);
     }
-    // ready ops per kind, most urgent first (then program order)
+    // ready ops per kind, most urgent first (then program order); fresh: the ops
+    // that the last pass made ready
     auto later = [&](int a, int b) { return height[a] != height[b] ? height[a] < height[b] : a > b; };
-    std::priority_queue<int, std::vector<int>, decltype(later)> ready[2] = {
-        std::priority_queue<int, std::vector<int>, decltype(later)>(later),
-        std::priority_queue<int, std::vector<int>, decltype(later)>(later)};
+    typedef std::priority_queue<int, std::vector<int>, decltype(later)> Queue;
+    Queue ready[2] = {Queue(later), Queue(later)};
+    std::vector<int> fresh;
     for (int i = 0; i < n; ++i)
       if (npred[i] == 0) ready[rec_kind[i]].push(i);
+    auto all_ready = [&]() {
+      for (int i : fresh) ready[rec_kind[i]].push(i);
+      fresh.clear();
+    };
     HostProgram hp;
     std::vector<int> pass;
     int done = 0;
+    bool in_run = false;                 // the last pass belongs to a run that this one may continue
     while (done < n) {
+      // the run goes on while a full pass is ready without the last one's results
+      // (or nothing waits for them); else all ready ops compete and a new run starts
+      bool urgent_recip = false;
+      for (int i : fresh) urgent_recip |= rec_kind[i] == 1 && (ready[0].empty() || later(ready[0].top(), i));
+      bool cont = wide && in_run && !urgent_recip && (ready[0].size() >= (size_t)WARP || (fresh.empty() && !ready[0].empty()));
+      if (cont && !ready[1].empty() && later(ready[0].top(), ready[1].top())) cont = false;
+      if (!cont) all_ready();
       int k;
       if (ready[0].empty()) k = 1;
       else if (ready[1].empty()) k = 0;
       else k = later(ready[0].top(), ready[1].top()) ? 1 : 0;
       pass.clear();
-      const size_t width = (wide && k == 0 && ready[0].size() >= 2 * (size_t)WARP) ? 2 * WARP : WARP;
-      while (!ready[k].empty() && pass.size() < width) {
+      while (!ready[k].empty() && pass.size() < (size_t)WARP) {
         pass.push_back(ready[k].top());
         ready[k].pop();
       }
@@ -147,19 +159,22 @@ struct Scheduler {
           for (int i : fill) hp.ops.push_back(rec_op[i]);
           for (size_t i = nr + fill.size(); i < (size_t)WARP; ++i) hp.ops.push_back(Op{OP_EMPTY, 0, 0, 0});
           hp.unit.push_back(sub == 0 ? 3 : 0);
+          hp.run.push_back(0);
           all.insert(all.end(), fill.begin(), fill.end());
         }
         pass = std::move(all);
       } else {
         for (int i : pass) hp.ops.push_back(rec_op[i]);
-        for (size_t i = pass.size(); i < width; ++i) hp.ops.push_back(Op{OP_EMPTY, 0, 0, 0});
-        if (width == WARP) hp.unit.push_back(0);
-        else hp.unit.insert(hp.unit.end(), {1, 2});
+        for (size_t i = pass.size(); i < (size_t)WARP; ++i) hp.ops.push_back(Op{OP_EMPTY, 0, 0, 0});
+        hp.unit.push_back(0);
+        hp.run.push_back(!wide ? 0 : cont ? 2 : 1);
       }
+      in_run = wide && k == 0;
       done += (int)pass.size();
+      all_ready();
       for (int i : pass)
         for (int s2 : succ[i])
-          if (--npred[s2] == 0) ready[rec_kind[s2]].push(s2);
+          if (--npred[s2] == 0) fresh.push_back(s2);
     }
     hp.n_ops = n_ops;
     return hp;
@@ -1106,12 +1121,12 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
     d.a_nconst = (int)m.a_consts_v.size();
     d.fwdT_npass = m.fwdT_prog.n_pass();
     d.bwdT_npass = m.bwdT_prog.n_pass();
-    d.nudot_nruns = (int)device_runs(m.nudot_prog).size();
-    d.jt_nruns = (int)device_runs(m.jt_prog).size();
+    d.nudot_nruns = (int)device_runs(m.nudot_prog).size() - 1;
+    d.jt_nruns = (int)device_runs(m.jt_prog).size() - 1;
   }
-  d.f_nruns = (int)device_runs(m.f_prog).size();
-  d.m_nruns = (int)device_runs(m.m_prog).size();
-  d.lu_nruns = (int)device_runs(m.lu_prog).size();
+  d.f_nruns = (int)device_runs(m.f_prog).size() - 1;
+  d.m_nruns = (int)device_runs(m.m_prog).size() - 1;
+  d.lu_nruns = (int)device_runs(m.lu_prog).size() - 1;
   d.fwd_npass = m.fwd_prog.n_pass();
   d.bwd_npass = m.bwd_prog.n_pass();
   d.d_nconst = (int)m.d_consts_v.size();
