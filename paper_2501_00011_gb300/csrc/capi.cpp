@@ -220,7 +220,8 @@ int chem_cells_create(const chem_mech *mech, int64_t n_cells, const chem_opts *o
       o.cells_per_block = o.couple_cells > 1 ? (wmax / o.couple_cells) * o.couple_cells   // whole groups per block
                                              : best_warps_per_block(mech->m.dev, o.lu_precision, o.driver);
     else
-      auto_shape(mech->m.dev, o.lu_precision, o.driver, o.couple_cells, n_cells, &o.cells_per_block, &o.blocks_per_sm);
+      auto_shape(mech->m.dev, o.lu_precision, o.driver, o.couple_cells, o.record_adjoint != 0, n_cells, &o.cells_per_block,
+                 &o.blocks_per_sm);
   }
   if (o.cells_per_block < 1) return fail(CHEM_EINVAL, "no launch shape fits on this device");
   if (o.record_adjoint && o.lu_precision != 64)

@@ -317,8 +317,8 @@ int occupancy(const MechDev &m, int lu_precision, int driver, int warps_per_bloc
 int best_warps_per_block(const MechDev &m, int lu_precision, int driver);
 // launch shape of a batch of n_cells in groups of `couple` whose caller gave
 // neither cells per block nor blocks per SM (0: nothing fits)
-void auto_shape(const MechDev &m, int lu_precision, int driver, int couple, int64_t n_cells, int *warps_per_block,
-                int *blocks_per_sm);
+void auto_shape(const MechDev &m, int lu_precision, int driver, int couple, bool record, int64_t n_cells,
+                int *warps_per_block, int *blocks_per_sm);
 // diagnostic: mode 0 out = f(y); mode 1 out = (I - c J(y))^{-1} b   (all [S][C] device arrays)
 cudaError_t launch_probe(const MechDev &M, const CellsDev &C, int lu_precision, int mode, double c, const double *y,
                          const double *b, double *out, cudaStream_t stream);

@@ -2172,25 +2172,30 @@ size_t pad_smem_to_blocks(size_t smem, int bps) {
 
 // Launch shape of a walk kernel.  A walk's cells each take one warp (the queue
 // hands out the longest tapes first), so while the batch has fewer than
-// NARROW_CELLS_PER_WARP cells per warp at NARROW_WARPS_PER_SM warps per SM,
-// nearly every cell has a warp of its own and the walk lasts as long as its
-// slowest cells, which run faster with fewer warps beside them on the SM: such
-// batches run at most NARROW_WARPS_PER_SM warps per SM (2,048 cells of the
-// 72-species mechanism: tangent 12.3 -> 11.2 ms, adjoint 12.5 -> 11.3 ms);
-// larger ones at the occupancy that keeps the most cells resident (shared
-// memory bounds it), ties to the larger block (fewer blocks to place).  Blocks
-// per SM are bounded by padding each block's shared memory, so the block
-// scheduler cannot stack a third block of a two-block shape on one SM while
-// another SM has none.  The kernel's dynamic shared-memory limit must be
-// raised first.
-constexpr int NARROW_WARPS_PER_SM = 8;
+// NARROW_CELLS_PER_WARP cells per warp at a few warps per SM, nearly every cell
+// has a warp of its own and the walk lasts as long as its slowest cells, which run
+// faster with fewer warps beside them on the SM.  Such batches run at most 4, or
+// else 8, warps per SM, spread over all SMs (72-species mechanism, adjoint /
+// tangent in ms at 4, 8, 12 warps per SM: 500 cells 5.4 / 5.3, 6.9 / 6.1, 7.4 /
+// 6.0; 1,000 cells 7.8 / 7.8, 9.4 / 8.8, 10.2 / 8.9; 2,048 cells 9.6 / 10.3, 8.8 /
+// 8.2, 9.5 / 10.2); larger ones at the occupancy that keeps the most cells
+// resident (shared memory bounds it), ties to the larger block (fewer blocks to
+// place).  Blocks per SM are bounded by padding each block's shared memory, so the
+// block scheduler cannot stack a third block of a two-block shape on one SM while
+// another SM has none.  The kernel's dynamic shared-memory limit must be raised
+// first.
 constexpr int NARROW_CELLS_PER_WARP = 2;
 
-bool narrow_batch(int64_t n_cells) {
+// most warps per SM of a walk over n_cells (0: no bound)
+int narrow_warps(int64_t n_cells) {
   int dev = 0, n_sm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-  return n_cells < (int64_t)NARROW_CELLS_PER_WARP * NARROW_WARPS_PER_SM * n_sm;
+  if (n_sm < 1) n_sm = 1;
+  const int64_t per_sm = (n_cells + n_sm - 1) / n_sm;
+  for (int w : {4, 8})
+    if (n_cells < (int64_t)NARROW_CELLS_PER_WARP * w * n_sm) return (int)(per_sm < w ? per_sm : w);
+  return 0;
 }
 
 struct WalkShape {
@@ -2205,16 +2210,16 @@ WalkShape walk_shape(K kernel, int cell_bytes, int max_warps, int64_t n_cells) {
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const bool narrow = narrow_batch(n_cells);
+  const int most = narrow_warps(n_cells);
   int best_w = 0, best_cells = 0, best_nb = 0;
   for (int w = 1; w <= max_warps && (long)w * cell_bytes <= (long)optin; ++w) {
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, w * WARP, (size_t)w * cell_bytes) != cudaSuccess)
       continue;
     int cells = w * nb;
-    if (narrow && cells > NARROW_WARPS_PER_SM) {
-      // the most whole blocks of w warps within the narrow bound
-      nb = NARROW_WARPS_PER_SM / w;
+    if (most > 0 && cells > most) {
+      // the most whole blocks of w warps within the bound
+      nb = most / w;
       cells = w * nb;
     }
     if (cells >= best_cells && cells > 0) {
@@ -2710,12 +2715,18 @@ int best_warps_per_block(const MechDev &M, int lu_precision, int driver) {
 // that (coupled: whole groups) spreads evenly instead, one block of
 // ceil(units / SMs) cells or groups on every SM, since a cell runs the faster
 // the fewer share its SM (72/186, first solve of 301 cells: 5.5 ms against
-// 7.3 ms as 26 full blocks of 12; 1,824 cells fill every SM either way).
-// Between one and two cells per resident warp the full occupancy stays: 8
-// cells per SM gain 8% on a first solve of 2,048 cells but lose 3% on four
-// consecutive steps, whose queue is keyed by exact costs.
-void auto_shape(const MechDev &M, int lu_precision, int driver, int couple, int64_t n_cells, int *warps_per_block,
-                int *blocks_per_sm) {
+// 7.3 ms as 26 full blocks of 12; 1,824 cells fill every SM either way).  A few
+// cells per warp later the batch still lasts about as long as its longest cells,
+// so up to two cells per resident warp the blocks hold two thirds of them, up to
+// three cells five sixths (72/186, full 12 / two thirds 8 / 10
+// cells per SM, ms: 2,048 cells first solve 8.5 / 7.7 / 8.0, repeated 9.1 / 7.8 /
+// 8.2, running 2.02 / 1.75 / 1.79; 3,001 cells 9.0 / 8.2 / 8.7, 9.3 / 8.1 / 8.8,
+// 3.1 / 2.7 / 2.8; 5,000 cells 12.3 / 12.5 / 12.3, 11.5 / 11.1 / 10.6, 2.7 / 2.4 /
+// 2.6).  A recording batch keeps the full occupancy (four recorded steps of 2,048
+// cells 13.5 / 13.8 / 14.0 ms), as do the FP32 factorisation and mechanisms small
+// enough for several blocks per SM, for which this was not measured.
+void auto_shape(const MechDev &M, int lu_precision, int driver, int couple, bool record, int64_t n_cells,
+                int *warps_per_block, int *blocks_per_sm) {
   const int full = couple > 1 ? (max_warps_per_block(M, lu_precision, driver) / couple) * couple
                               : best_warps_per_block(M, lu_precision, driver);
   *warps_per_block = full;
@@ -2725,7 +2736,14 @@ void auto_shape(const MechDev &M, int lu_precision, int driver, int couple, int6
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   if (n_sm < 1) return;
   const int64_t units = (n_cells + couple - 1) / couple;
-  const int64_t w = (units + n_sm - 1) / n_sm * couple;
+  const int64_t per_sm = (units + n_sm - 1) / n_sm * couple;
+  int64_t w = full;
+  if (per_sm < full) {
+    w = per_sm;
+  } else if (couple <= 1 && lu_precision == 64 && !record && occupancy(M, lu_precision, driver, full) == 1) {
+    if (per_sm <= 2 * full) w = 2 * full / 3;
+    else if (per_sm <= 3 * full) w = 5 * full / 6;
+  }
   if (w < 1 || w >= full) return;
   *warps_per_block = (int)w;
   *blocks_per_sm = 1;

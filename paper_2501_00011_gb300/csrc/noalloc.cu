@@ -141,7 +141,7 @@ extern "C" int chem_solve_step_noalloc(const chem_mech *mech, int64_t n_cells, c
   if (o.cells_per_block == 0) {
     int w = 0, bps = o.blocks_per_sm;
     if (bps > 0) w = best_warps_per_block(mech->m.dev, o.lu_precision, CHEM_DRIVER_PERSISTENT);
-    else auto_shape(mech->m.dev, o.lu_precision, CHEM_DRIVER_PERSISTENT, 1, n_cells, &w, &bps);
+    else auto_shape(mech->m.dev, o.lu_precision, CHEM_DRIVER_PERSISTENT, 1, false, n_cells, &w, &bps);
     o.cells_per_block = w;
     o.blocks_per_sm = bps;
   }
