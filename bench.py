@@ -463,7 +463,7 @@ def run_gpu(args):
                 "value": n3 * wl3.n_steps / (t3 / 1e3), "unit": "cells/s (cell-steps per second)",
                 "ms_per_graph": t3, "cells": n3, "steps_per_graph": wl3.n_steps,
                 "form": "persistent work queue, 6 x 600 s steps captured in one CUDA graph, per-cell photolysis, "
-                        "FP64; each step's queue keyed by the previous step's costs (a different state)",
+                        "FP64; one kernel takes every cell through its steps, the queue keyed by the batch's last solve",
                 "autotuned": {"cells_per_block": w, "blocks_per_sm": b},
                 "integrator_steps_last_600s": {"min": int(st3["steps"].min()), "median": float(np.median(st3["steps"])),
                                                "max": int(st3["steps"].max())},

@@ -246,8 +246,9 @@ int chem_cells_set_theta(chem_cells *cells, const double *theta, int32_t mem, vo
  * CHEM_ECUDA; nothing is launched on error. */
 int chem_solve_step(chem_cells *cells, double dt, void *stream);
 /* n_steps consecutive chem_solve_step calls of dt (1..CHEM_MAX_GRAPH_STEPS) as
- * one CUDA graph launch on stream: the per-step queue resets and solve
- * kernels are captured once, on an internal stream, and the graph is re-used
+ * one CUDA graph launch on stream: the queue reset, the queue order and one
+ * kernel that takes every cell through its n steps (coupled groups: one kernel
+ * per step) are captured once, on an internal stream, and the graph is re-used
  * while n_steps, dt, the launch shape and the photolysis/theta sources
  * (per-cell or mechanism J, theta set or not) stay the same; any change
  * re-captures it.  The inputs it reads (T, P, y, J, theta) are the batch's
@@ -479,7 +480,10 @@ typedef int (*chem_chunk_fn)(int64_t c0, int64_t c1, int32_t step, void *user);
  * strided copies), the solve, y back device -> host; then, on this thread,
  * fn(c0, c1, step, user) (fn may be NULL), after which that chunk's next step
  * is queued at once, so host work on one chunk overlaps the GPU's work on the
- * others and the copies overlap the solves.  Results equal those of n_steps
+ * others and the copies overlap the solves.  Without fn there is nothing to
+ * overlap: all cells run as one batch (a second device copy of the state, made
+ * by the first such run; in chunks if it does not fit), the inputs copied once,
+ * the steps in one launch.  Results equal those of n_steps
  * chem_solve_step calls on one batch with fn applied between them, bit for
  * bit.  The host arrays should be page-locked (cudaHostRegister or a pinned
  * allocation) for the copies to run asynchronously.  stats (may be NULL)

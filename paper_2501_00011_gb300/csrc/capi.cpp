@@ -26,6 +26,7 @@ struct chem_cells {
   int *order = nullptr, *order_bucket = nullptr, *order_hist = nullptr;   // persistent driver: queue order
   double *kt = nullptr;       // chem_eval_deriv_design: rate constants [R][C], allocated on first use
   bool kt_valid = false;      // ... and current for the batch's T, P, photolysis and theta
+  bool solved = false;        // a solve of the batch has been queued: its cells have costs (stats)
   bool have_state = false, use_J = false, use_theta = false;
   int device = 0;
   // adjoint (record_adjoint)
@@ -432,14 +433,15 @@ cudaError_t enqueue_solve(chem_cells *c, double dt, cudaStream_t s, int n_steps 
         return e;
       cd.order = c->order;
     } else {
-      if ((e = launch_order(c->mech->m.dev, cd, c->opts.rtol, c->opts.atol, c->order_bucket, c->order_hist, c->order,
-                            s)) != cudaSuccess)
+      if ((e = launch_order(c->mech->m.dev, cd, c->opts.rtol, c->opts.atol, c->solved, c->order_bucket, c->order_hist,
+                            c->order, s)) != cudaSuccess)
         return e;
       cd.order = c->order;
     }
   }
   LaunchCfg cfg = launch_cfg(c->opts, dt);
   cfg.n_steps = n_steps;
+  c->solved = true;
   return launch_solve(c->mech->m.dev, cd, cfg, s);
 }
 

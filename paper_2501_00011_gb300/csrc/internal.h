@@ -141,13 +141,12 @@ struct MechDev {
 //              before are in flight
 //   RUN_PIPE1  the same, the last group with one pass (the second slot not used)
 //   RUN_SEQ    groups of two passes, the second after the first
-//   RUN_ONE    one pass (the second slot not used)
 //   RUN_RECIP  two groups, three passes, reciprocals in the first: a lane with a
 //              reciprocal spends three FP64 instructions on it and has no op in the
 //              other two, every other lane runs its three FMA ops; all ops of the
 //              unit are independent of each other
 // A program without runs (the triangular solves) is its passes in order.
-constexpr uint32_t RUN_PIPE = 0, RUN_PIPE1 = 1, RUN_RECIP = 2, RUN_SEQ = 3, RUN_ONE = 4;
+constexpr uint32_t RUN_PIPE = 0, RUN_PIPE1 = 1, RUN_RECIP = 2, RUN_SEQ = 3;
 constexpr int GROUP_BYTES = 2 * WARP * 8;
 constexpr int PAD_GROUPS = 5;     // readable groups past a program's last (the interpreters read ahead unconditionally)
 
@@ -185,7 +184,7 @@ struct HostProgram {
         runs.push_back((n & 1 ? RUN_PIPE1 : RUN_PIPE) << 28 | (n + 1) / 2);
       } else {
         if (n > 1) runs.push_back(RUN_SEQ << 28 | n / 2);
-        if (n & 1) runs.push_back(RUN_ONE << 28 | 1u);
+        if (n & 1) runs.push_back(RUN_PIPE1 << 28 | 1u);
       }
       for (; p < e; p += 2) g.push_back({p, p + 1 < e ? p + 1 : -1});
       p = e;
@@ -308,7 +307,8 @@ constexpr int ORDER_HIST_INTS = 2 * ORDER_BUCKETS + 2;   // counts, cursors, key
 cudaError_t launch_order_tape(const CellsDev &c, int *bucket, int *hist, int *order, cudaStream_t stream);
 // ... and keyed by the cost of coupled groups of G cells: order[i] is a group index.
 cudaError_t launch_order_groups(const CellsDev &c, int G, int *bucket, int *hist, int *order, cudaStream_t stream);
-cudaError_t launch_order(const MechDev &m, const CellsDev &c, double rtol, double atol, int *bucket, int *hist,
+// solved: the batch has been solved before, so (nearly) every cell has a cost.
+cudaError_t launch_order(const MechDev &m, const CellsDev &c, double rtol, double atol, bool solved, int *bucket, int *hist,
                          int *order, cudaStream_t stream);
 int max_warps_per_block(const MechDev &m, int lu_precision, int driver);
 // resident blocks per SM of the solve kernel for a block of warps_per_block cells

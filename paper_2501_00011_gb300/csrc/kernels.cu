@@ -373,11 +373,9 @@ __device__ __forceinline__ void run_prog(S st, const uint32_t *runs, const int n
       for (; n > 0; --n) ps.recip(st);
     } else if (kind <= RUN_PIPE1) {
       ps.pipe(st, n, kind == RUN_PIPE1);
-    } else if (kind == RUN_SEQ) {
+    } else {
 #pragma unroll 1
       for (; n > 0; --n) ps.seq(st);
-    } else {
-      ps.one(st);
     }
   }
   st.end();
@@ -2321,31 +2319,60 @@ __device__ __forceinline__ float from_ordered_bits(unsigned u) {
 // keys: bucket[cell] receives the key's bits (float); hist[2 ORDER_BUCKETS]
 // the largest key's ordered bits, hist[2 ORDER_BUCKETS + 1] the complement of
 // the smallest's (both start at 0); a cell with bad inputs gets -inf
-template <int KS>
+// LANES: one lane per cell, for a batch that has been solved before (every cell
+// has a cost; one without, after a launch that failed, is keyed by the whole warp
+// in turn), and two atomics per warp.  Otherwise one warp per cell, since a rate
+// constant sum takes a warp 20 us.  (One warp per cell with costs took 110 us a
+// launch on average over the benchmark's batches, two same-address atomics per
+// cell; a running step of 10,000 cells 4.2 ms in all.)
+template <int KS, bool LANES>
 __global__ void __launch_bounds__(ORDER_WARPS * WARP) order_keys_kernel(const __grid_constant__ MechDev M, const CellsDev C,
                                                                           const SolveParams P, int *bucket, int *hist) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & (WARP - 1);
   const int warp = threadIdx.x / WARP;
-  const int64_t cell = (int64_t)blockIdx.x * ORDER_WARPS + warp;
-  if (cell >= C.n_cells) return;
+  const int64_t w = (int64_t)blockIdx.x * ORDER_WARPS + warp;
+  const int64_t cell = LANES ? w * WARP + lane : w;
+  if ((LANES ? w * WARP : cell) >= C.n_cells) return;
+  const bool in = cell < C.n_cells;
   double *Wd = reinterpret_cast<double *>(smem + (size_t)warp * P.cell_bytes);
-  float l = -INFINITY;                        // log2 of the key, larger first
-  const chem_cell_stats prev = C.stats[cell];
-  if (prev.steps > 0) {
-    l = (float)log2(65.0 * prev.f_evals + 100.0 * prev.solves + 560.0 * prev.jac_evals + 150.0 * prev.steps);
-  } else {
-    bool own[KS];
+  bool own[KS];
 #pragma unroll
-    for (int k = 0; k < KS; ++k) own[k] = lane + WARP * k < M.S;
+  for (int k = 0; k < KS; ++k) own[k] = lane + WARP * k < M.S;
+  // the warp's sum of the rate constants of cell c, as a key (-inf: bad inputs)
+  auto rate_key = [&](const int64_t c) {
     double y0[KS];
-    if (!load_cell<KS>(M, C, Wd, lane, cell, own, y0)) {
+    float l = -INFINITY;
+    if (!load_cell<KS>(M, C, Wd, lane, c, own, y0)) {
       double sk = 0.0;
       for (int j = lane; j < M.R; j += WARP) sk += Wd[M.d_KT + j];
       sk = warp_sum(sk);
       if (sk > 0.0 && isfinite(sk)) l = (float)log2(sk);
     }
+    __syncwarp();
+    return l;
+  };
+  float l = -INFINITY;                        // log2 of the key, larger first
+  chem_cell_stats prev = {};
+  if (in) prev = C.stats[cell];
+  if (prev.steps > 0) l = (float)log2(65.0 * prev.f_evals + 100.0 * prev.solves + 560.0 * prev.jac_evals + 150.0 * prev.steps);
+  if (LANES) {
+    for (unsigned m = __ballot_sync(FULL, in && prev.steps <= 0); m; m &= m - 1) {
+      const int src = __ffs(m) - 1;
+      const float k = rate_key(w * WARP + src);
+      if (lane == src) l = k;
+    }
+    if (in) bucket[cell] = __float_as_int(l);
+    const bool fin = in && isfinite(l);
+    const unsigned hi = __reduce_max_sync(FULL, fin ? ordered_bits(l) : 0u);
+    const unsigned lo = __reduce_max_sync(FULL, fin ? ~ordered_bits(l) : 0u);
+    if (lane == 0) {                         // (0 where no key is finite: the initial value)
+      atomicMax(reinterpret_cast<unsigned *>(hist) + 2 * ORDER_BUCKETS, hi);
+      atomicMax(reinterpret_cast<unsigned *>(hist) + 2 * ORDER_BUCKETS + 1, lo);
+    }
+    return;
   }
+  if (prev.steps <= 0) l = rate_key(cell);
   if (lane == 0) {
     bucket[cell] = __float_as_int(l);
     if (isfinite(l)) {
@@ -2405,14 +2432,24 @@ __global__ void order_group_keys_kernel(const CellsDev C, int G, int64_t n_group
   atomicAdd(hist + b, 1);
 }
 
-// exclusive prefix sum of the bucket counts into the scatter cursors
+// exclusive prefix sum of the bucket counts into the scatter cursors (one warp)
 __global__ void order_scan_kernel(int *hist) {
-  if (threadIdx.x != 0) return;
-  int acc = 0;
-  for (int b = 0; b < ORDER_BUCKETS; ++b) {
-    const int n = hist[b];
-    hist[ORDER_BUCKETS + b] = acc;
-    acc += n;
+  constexpr int PER = ORDER_BUCKETS / WARP;
+  const int lane = threadIdx.x;
+  int n[PER], sum = 0;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) sum += n[i] = hist[lane * PER + i];
+  int acc = sum;
+#pragma unroll
+  for (int o = 1; o < WARP; o <<= 1) {
+    const int v = __shfl_up_sync(FULL, acc, o);
+    if (lane >= o) acc += v;
+  }
+  acc -= sum;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    hist[ORDER_BUCKETS + lane * PER + i] = acc;
+    acc += n[i];
   }
 }
 
@@ -2424,12 +2461,14 @@ __global__ void order_scatter_kernel(const int *bucket, int *hist, int *order, i
 }
 
 template <int KS>
-cudaError_t launch_order_t(const MechDev &M, const CellsDev &C, const SolveParams &P, int *bucket, int *hist, cudaStream_t s) {
+cudaError_t launch_order_t(const MechDev &M, const CellsDev &C, const SolveParams &P, bool solved, int *bucket, int *hist,
+                           cudaStream_t s) {
   const size_t smem = (size_t)P.cell_bytes * ORDER_WARPS;
-  cudaError_t e = allow_max_smem<order_keys_kernel<KS>>();
+  cudaError_t e = solved ? allow_max_smem<order_keys_kernel<KS, true>>() : allow_max_smem<order_keys_kernel<KS, false>>();
   if (e != cudaSuccess) return e;
-  const int64_t blocks = (C.n_cells + ORDER_WARPS - 1) / ORDER_WARPS;
-  order_keys_kernel<KS><<<(unsigned)blocks, ORDER_WARPS * WARP, smem, s>>>(M, C, P, bucket, hist);
+  const int64_t per = solved ? ORDER_WARPS * WARP : ORDER_WARPS, blocks = (C.n_cells + per - 1) / per;
+  if (solved) order_keys_kernel<KS, true><<<(unsigned)blocks, ORDER_WARPS * WARP, smem, s>>>(M, C, P, bucket, hist);
+  else order_keys_kernel<KS, false><<<(unsigned)blocks, ORDER_WARPS * WARP, smem, s>>>(M, C, P, bucket, hist);
   return cudaGetLastError();
 }
 
@@ -2596,13 +2635,12 @@ __global__ void __launch_bounds__(32 * WARP) deriv_gather_kernel(const __grid_co
     reinterpret_cast<uint4 *>(gs)[i] = __ldg(reinterpret_cast<const uint4 *>(M.blob[0]) + i);
   double *sm = reinterpret_cast<double *>(gs + tb);
   // element (row, cell) -> slice of cell, slot row
-  for (int i = tid; i < M.S * D.gather_cells; i += nt) {
-    const int r = i / D.gather_cells, cl = i % D.gather_cells;
-    if (cl < nb) sm[(size_t)cl * D.cell_doubles + M.d_Y + r] = y[(int64_t)r * NC + c0 + cl];
-  }
-  for (int i = tid; i < M.R * D.gather_cells; i += nt) {
-    const int r = i / D.gather_cells, cl = i % D.gather_cells;
-    if (cl < nb) sm[(size_t)cl * D.cell_doubles + M.d_KT + r] = kt[(int64_t)r * NC + c0 + cl];
+  // (cells fastest; a thread's cell stays the same, its row goes up by nt / gather_cells)
+  const int cl = tid % D.gather_cells, r0 = tid / D.gather_cells;
+  double *const mine = sm + (size_t)cl * D.cell_doubles;
+  if (cl < nb) {
+    for (int r = r0; r < M.S; r += WARP) mine[M.d_Y + r] = y[(int64_t)r * NC + c0 + cl];
+    for (int r = r0; r < M.R; r += WARP) mine[M.d_KT + r] = kt[(int64_t)r * NC + c0 + cl];
   }
   if (warp < nb) {
     unsigned char *wd = reinterpret_cast<unsigned char *>(sm + (size_t)warp * D.cell_doubles);
@@ -2613,10 +2651,8 @@ __global__ void __launch_bounds__(32 * WARP) deriv_gather_kernel(const __grid_co
   group_sync(GATHER_BAR, D.gather_cells);
   if (warp < nb) f_core<true>(M, P, gs, sm + (size_t)warp * D.cell_doubles, lane);
   group_sync(GATHER_BAR, D.gather_cells);
-  for (int i = tid; i < M.S * D.gather_cells; i += nt) {
-    const int r = i / D.gather_cells, cl = i % D.gather_cells;
-    if (cl < nb) f[(int64_t)r * NC + c0 + cl] = sm[(size_t)cl * D.cell_doubles + M.d_F + r];
-  }
+  if (cl < nb)
+    for (int r = r0; r < M.S; r += WARP) f[(int64_t)r * NC + c0 + cl] = mine[M.d_F + r];
 }
 
 bool staged_driver(int driver) { return driver == CHEM_DRIVER_PERSISTENT; }
@@ -2936,7 +2972,7 @@ cudaError_t launch_order_tape(const CellsDev &C, int *bucket, int *hist, int *or
   return cudaGetLastError();
 }
 
-cudaError_t launch_order(const MechDev &M, const CellsDev &C, double rtol, double atol, int *bucket, int *hist,
+cudaError_t launch_order(const MechDev &M, const CellsDev &C, double rtol, double atol, bool solved, int *bucket, int *hist,
                          int *order, cudaStream_t stream) {
   if (C.n_cells <= 0) return cudaSuccess;
   SolveParams P{};
@@ -2948,10 +2984,10 @@ cudaError_t launch_order(const MechDev &M, const CellsDev &C, double rtol, doubl
   cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(int) * ORDER_HIST_INTS, stream);
   if (e != cudaSuccess) return e;
   switch ((M.S + WARP - 1) / WARP) {
-    case 1: e = launch_order_t<1>(M, C, P, bucket, hist, stream); break;
-    case 2: e = launch_order_t<2>(M, C, P, bucket, hist, stream); break;
-    case 3: e = launch_order_t<3>(M, C, P, bucket, hist, stream); break;
-    case 4: e = launch_order_t<4>(M, C, P, bucket, hist, stream); break;
+    case 1: e = launch_order_t<1>(M, C, P, solved, bucket, hist, stream); break;
+    case 2: e = launch_order_t<2>(M, C, P, solved, bucket, hist, stream); break;
+    case 3: e = launch_order_t<3>(M, C, P, solved, bucket, hist, stream); break;
+    case 4: e = launch_order_t<4>(M, C, P, solved, bucket, hist, stream); break;
     default: return cudaErrorInvalidValue;
   }
   if (e != cudaSuccess) return e;
