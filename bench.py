@@ -321,7 +321,8 @@ def run_gpu(args):
                     "solve, y back, then the host work on that chunk (one implicit vertical-diffusion step in "
                     "columns of 50 cells, numpy) while the GPU solves the other chunks; wall clock per model "
                     "step, best of 3; chunks_1 = no overlap (copies, solve, copies, host work in sequence). "
-                    "chemistry_only is one step from the initial state (the headline's work, end to end); "
+                    "chemistry_only is one step from the initial state (the headline's work, end to end; without host "
+                    "work all cells run as one batch whatever the number of chunks); "
                     "with_host_work is two steps, the second from the mixed state"}
 
     def time_adjoint(fp64_peak):
