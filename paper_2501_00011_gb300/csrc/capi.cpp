@@ -102,6 +102,25 @@ int check_device(const chem_cells *c) {
   return 0;
 }
 
+// The arrays of a new batch that start at zero, done when this returns: the
+// caller's streams, and a pipeline's own, need not wait for the default stream (a
+// cudaMemset there returns before it has run, and behind other work would run
+// during the first solve, resetting its queue and its stats).
+cudaError_t clear_batch(chem_cells *c) {
+  const size_t n = (size_t)(c->n > 0 ? c->n : 1);
+  cudaStream_t s = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(c->stats, 0, n * sizeof(chem_cell_stats), s)) == cudaSuccess &&
+      (e = cudaMemsetAsync(c->counters, 0, 4 * sizeof(unsigned long long), s)) == cudaSuccess && c->tape_n &&
+      (e = cudaMemsetAsync(c->tape_n, 0, n * sizeof(int), s)) == cudaSuccess &&
+      (e = cudaMemsetAsync(c->tape_rows, 0, n * sizeof(int), s)) == cudaSuccess)
+    e = cudaMemsetAsync(c->tape_bad, 0, n * sizeof(int), s);
+  const cudaError_t es = cudaStreamSynchronize(s);
+  cudaStreamDestroy(s);
+  return e != cudaSuccess ? e : es;
+}
+
 }  // namespace
 
 void chemgpu::set_last_error(const std::string &msg) { g_err = msg; }
@@ -274,17 +293,10 @@ int chem_cells_create(const chem_mech *mech, int64_t n_cells, const chem_opts *o
       chem_cells_destroy(c);
       return fail(CHEM_ENOMEM, std::string("cudaMalloc of the adjoint tape failed: ") + cudaGetErrorString(e));
     }
-    if ((e = cudaMemset(c->tape_n, 0, n * sizeof(int))) != cudaSuccess ||
-        (e = cudaMemset(c->tape_rows, 0, n * sizeof(int))) != cudaSuccess ||
-        (e = cudaMemset(c->tape_bad, 0, n * sizeof(int))) != cudaSuccess) {
-      chem_cells_destroy(c);
-      return cuda_fail(e, "cudaMemset");
-    }
   }
-  if ((e = cudaMemset(c->stats, 0, n * sizeof(chem_cell_stats))) != cudaSuccess ||
-      (e = cudaMemset(c->counters, 0, 4 * sizeof(unsigned long long))) != cudaSuccess) {
+  if ((e = clear_batch(c)) != cudaSuccess) {
     chem_cells_destroy(c);
-    return cuda_fail(e, "cudaMemset");
+    return cuda_fail(e, "clearing the batch");
   }
   *out = c;
   return 0;

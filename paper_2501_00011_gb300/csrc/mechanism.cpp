@@ -1229,7 +1229,9 @@ int upload_mechanism(Mechanism &m, std::string &msg) {
       return rc;
     }
   }
-  if (set_constants() != cudaSuccess) {
+  // a copy from pageable host memory may still be under way when cudaMemcpy
+  // returns; kernels on non-blocking streams do not wait for it, so this does
+  if (set_constants() != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess) {
     free_mechanism(m);
     msg = "could not set solver constants on the device";
     return CHEM_ECUDA;
