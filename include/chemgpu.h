@@ -481,9 +481,8 @@ typedef int (*chem_chunk_fn)(int64_t c0, int64_t c1, int32_t step, void *user);
  * fn(c0, c1, step, user) (fn may be NULL), after which that chunk's next step
  * is queued at once, so host work on one chunk overlaps the GPU's work on the
  * others and the copies overlap the solves.  Without fn there is nothing to
- * overlap: all cells run as one batch (a second device copy of the state, made
- * by the first such run; in chunks if it does not fit), the inputs copied once,
- * the steps in one launch.  Results equal those of n_steps
+ * overlap: all cells run as one batch, in the chunks' device memory, the inputs
+ * copied once, the steps in one launch.  Results equal those of n_steps
  * chem_solve_step calls on one batch with fn applied between them, bit for
  * bit.  The host arrays should be page-locked (cudaHostRegister or a pinned
  * allocation) for the copies to run asynchronously.  stats (may be NULL)

@@ -23,6 +23,7 @@ struct chem_cells {
   // device counters: [0] persistent work queue, [1] staging fallbacks and
   // [2] unfinished staging copies of the last solve call (CellsDev::stage), [3] spare
   unsigned long long *counters = nullptr;
+  bool view = false;          // the per-cell arrays belong to another batch (cells_create)
   int *order = nullptr, *order_bucket = nullptr, *order_hist = nullptr;   // persistent driver: queue order
   double *kt = nullptr;       // chem_eval_deriv_design: rate constants [R][C], allocated on first use
   bool kt_valid = false;      // ... and current for the batch's T, P, photolysis and theta
@@ -121,6 +122,13 @@ cudaError_t clear_batch(chem_cells *c) {
   return e != cudaSuccess ? e : es;
 }
 
+// chem_cells_create; store not NULL: the batch's cells are n_cells of those of
+// store, from cell c0 on, and its per-cell arrays the part of store's arrays that
+// holds as many cells (each array is [rows][n_cells]), with counters of its own.
+// The two are never in use at the same time.
+int cells_create(const chem_mech *mech, int64_t n_cells, const chem_opts *opts, const chem_cells *store, int64_t c0,
+                 chem_cells **out);
+
 }  // namespace
 
 void chemgpu::set_last_error(const std::string &msg) { g_err = msg; }
@@ -204,117 +212,24 @@ int chem_mechanism_structure(const chem_mech *h, int32_t *pos, uint8_t *fill) {
 }
 
 int chem_cells_create(const chem_mech *mech, int64_t n_cells, const chem_opts *opts, chem_cells **out) {
-  g_err.clear();
-  if (!out) return fail(CHEM_EINVAL, "out is NULL");
-  *out = nullptr;
-  if (!mech) return fail(CHEM_EINVAL, "mechanism is NULL");
-  if (n_cells < 0 || n_cells > ((int64_t)1 << 31)) return fail(CHEM_EINVAL, "n_cells must be in 0..2^31");
-  {
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev != mech->m.device)
-      return fail(CHEM_EINVAL, "the mechanism belongs to device " + std::to_string(mech->m.device) +
-                                   ", which must be current when a batch is created");
-  }
-  chem_opts o;
-  if (opts) o = *opts; else chem_opts_default(&o);
-  if (!(o.rtol > 0.0) || !(o.atol > 0.0)) return fail(CHEM_EINVAL, "rtol and atol must be > 0");
-  if (o.max_order < 1 || o.max_order > QMAX) return fail(CHEM_EINVAL, "max_order must be 1..5");
-  if (o.max_steps < 1) return fail(CHEM_EINVAL, "max_steps must be >= 1");
-  if (o.lu_precision != 64 && o.lu_precision != 32) return fail(CHEM_EINVAL, "lu_precision must be 64 or 32");
-  if (o.driver != CHEM_DRIVER_PLAIN && o.driver != CHEM_DRIVER_PERSISTENT) return fail(CHEM_EINVAL, "bad driver");
-  if (o.cells_per_block < 0 || o.cells_per_block > MAX_WARPS_PER_BLOCK || o.blocks_per_sm < 0) return fail(CHEM_EINVAL, "bad launch shape");
-  if (o.couple_cells < 0 || o.couple_cells > MAX_WARPS_PER_BLOCK) return fail(CHEM_EINVAL, "couple_cells out of range");
-  if (o.couple_cells == 0) o.couple_cells = 1;
-  if (o.couple_cells > 1) {
-    if (o.lu_precision != 64) return fail(CHEM_EINVAL, "coupled cells need lu_precision 64");
-    if (o.record_adjoint) return fail(CHEM_EINVAL, "coupled cells have no adjoint");
-    const int wmax = max_warps_per_block(mech->m.dev, o.lu_precision, o.driver);
-    if (o.couple_cells > wmax) return fail(CHEM_EINVAL, "couple_cells exceeds the cells a block can hold");
-    if (o.cells_per_block % o.couple_cells) return fail(CHEM_EINVAL, "cells_per_block must be a multiple of couple_cells");
-  }
-  const int wmax = max_warps_per_block(mech->m.dev, o.lu_precision, o.driver);
-  if (wmax < 1) return fail(CHEM_EINVAL, "mechanism working set does not fit in shared memory");
-  if (o.cells_per_block > wmax) return fail(CHEM_EINVAL, "cells_per_block exceeds the shared-memory limit");
-  if (o.cells_per_block == 0) {
-    if (o.blocks_per_sm > 0)
-      o.cells_per_block = o.couple_cells > 1 ? (wmax / o.couple_cells) * o.couple_cells   // whole groups per block
-                                             : best_warps_per_block(mech->m.dev, o.lu_precision, o.driver);
-    else
-      auto_shape(mech->m.dev, o.lu_precision, o.driver, o.couple_cells, o.record_adjoint != 0, n_cells, &o.cells_per_block,
-                 &o.blocks_per_sm);
-  }
-  if (o.cells_per_block < 1) return fail(CHEM_EINVAL, "no launch shape fits on this device");
-  if (o.record_adjoint && o.lu_precision != 64)
-    return fail(CHEM_EINVAL, "record_adjoint needs lu_precision 64 (the adjoint differentiates the FP64 iteration)");
-  if (o.record_adjoint && (o.tape_steps < 0 || o.tape_steps > CHEM_MAX_TAPE_ROWS))
-    return fail(CHEM_EINVAL, "tape_steps out of range");
-  if (o.stage_wait < -1) return fail(CHEM_EINVAL, "stage_wait must be -1, 0 or positive");
-
-  chem_cells *c = new (std::nothrow) chem_cells();
-  if (!c) return fail(CHEM_ENOMEM, "host allocation failed");
-  c->mech = mech;
-  c->n = n_cells;
-  c->opts = o;
-  cudaGetDevice(&c->device);
-  const int S = mech->m.S, R = mech->m.R;
-  const size_t n = (size_t)(n_cells > 0 ? n_cells : 1);
-  cudaError_t e = cudaSuccess;
-  if ((e = cudaMalloc(&c->T, n * sizeof(double))) != cudaSuccess ||
-      (e = cudaMalloc(&c->P, n * sizeof(double))) != cudaSuccess ||
-      (e = cudaMalloc(&c->y, n * S * sizeof(double))) != cudaSuccess ||
-      (e = cudaMalloc(&c->stats, n * sizeof(chem_cell_stats))) != cudaSuccess ||
-      (e = cudaMalloc(&c->counters, 4 * sizeof(unsigned long long))) != cudaSuccess ||
-      (e = cudaMalloc(&c->theta, (R > 0 ? R : 1) * sizeof(double))) != cudaSuccess ||
-      (mech->m.n_phot > 0 && (e = cudaMalloc(&c->J, n * mech->m.n_phot * sizeof(double))) != cudaSuccess)) {
-    chem_cells_destroy(c);
-    return fail(CHEM_ENOMEM, std::string("cudaMalloc failed: ") + cudaGetErrorString(e));
-  }
-  if ((o.driver == CHEM_DRIVER_PERSISTENT || o.record_adjoint) &&
-      ((e = cudaMalloc(&c->order, n * sizeof(int))) != cudaSuccess ||
-       (e = cudaMalloc(&c->order_bucket, n * sizeof(int))) != cudaSuccess ||
-       (e = cudaMalloc(&c->order_hist, ORDER_HIST_INTS * sizeof(int))) != cudaSuccess)) {
-    chem_cells_destroy(c);
-    return fail(CHEM_ENOMEM, std::string("cudaMalloc of the queue order failed: ") + cudaGetErrorString(e));
-  }
-  if (o.record_adjoint) {
-    c->row_cap = o.tape_steps > 0 ? o.tape_steps : 2000;
-    c->tape_cap = 3 * c->row_cap + 64;
-    const size_t E = (size_t)c->tape_cap, RC = (size_t)c->row_cap;
-    if ((e = cudaMalloc(&c->tape_kq, n * E * sizeof(int))) != cudaSuccess ||
-        (e = cudaMalloc(&c->tape_val, n * E * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&c->tape_n, n * sizeof(int))) != cudaSuccess ||
-        (e = cudaMalloc(&c->tape_rows, n * sizeof(int))) != cudaSuccess ||
-        (e = cudaMalloc(&c->tape_bad, n * sizeof(int))) != cudaSuccess ||
-        (e = cudaMalloc(&c->ytape, n * RC * S * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&c->gcell, n * (R > 0 ? R : 1) * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&c->dLdy, n * S * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&c->dLdy0, n * S * sizeof(double))) != cudaSuccess ||
-        (e = cudaMalloc(&c->dLdtheta, (R > 0 ? R : 1) * sizeof(double))) != cudaSuccess) {
-      chem_cells_destroy(c);
-      return fail(CHEM_ENOMEM, std::string("cudaMalloc of the adjoint tape failed: ") + cudaGetErrorString(e));
-    }
-  }
-  if ((e = clear_batch(c)) != cudaSuccess) {
-    chem_cells_destroy(c);
-    return cuda_fail(e, "clearing the batch");
-  }
-  *out = c;
-  return 0;
+  return cells_create(mech, n_cells, opts, nullptr, 0, out);
 }
 
 void chem_cells_destroy(chem_cells *c) {
   if (!c) return;
   if (c->graph) cudaGraphExecDestroy(c->graph);
   if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
-  cudaFree(c->T);
-  cudaFree(c->P);
-  cudaFree(c->y);
-  cudaFree(c->J);
+  if (!c->view) {
+    cudaFree(c->T);
+    cudaFree(c->P);
+    cudaFree(c->y);
+    cudaFree(c->J);
+    cudaFree(c->stats);
+    cudaFree(c->order);
+    cudaFree(c->order_bucket);
+  }
   cudaFree(c->theta);
-  cudaFree(c->stats);
   cudaFree(c->counters);
-  cudaFree(c->order);
-  cudaFree(c->order_bucket);
   cudaFree(c->order_hist);
   cudaFree(c->kt);
   cudaFree(c->tape_kq);
@@ -390,6 +305,120 @@ int chem_cells_set_theta(chem_cells *c, const double *theta, int32_t mem, void *
 }  // extern "C"
 
 namespace {
+
+int cells_create(const chem_mech *mech, int64_t n_cells, const chem_opts *opts, const chem_cells *store, int64_t c0,
+                 chem_cells **out) {
+  g_err.clear();
+  if (!out) return fail(CHEM_EINVAL, "out is NULL");
+  *out = nullptr;
+  if (!mech) return fail(CHEM_EINVAL, "mechanism is NULL");
+  if (n_cells < 0 || n_cells > ((int64_t)1 << 31)) return fail(CHEM_EINVAL, "n_cells must be in 0..2^31");
+  {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev != mech->m.device)
+      return fail(CHEM_EINVAL, "the mechanism belongs to device " + std::to_string(mech->m.device) +
+                                   ", which must be current when a batch is created");
+  }
+  chem_opts o;
+  if (opts) o = *opts; else chem_opts_default(&o);
+  if (!(o.rtol > 0.0) || !(o.atol > 0.0)) return fail(CHEM_EINVAL, "rtol and atol must be > 0");
+  if (o.max_order < 1 || o.max_order > QMAX) return fail(CHEM_EINVAL, "max_order must be 1..5");
+  if (o.max_steps < 1) return fail(CHEM_EINVAL, "max_steps must be >= 1");
+  if (o.lu_precision != 64 && o.lu_precision != 32) return fail(CHEM_EINVAL, "lu_precision must be 64 or 32");
+  if (o.driver != CHEM_DRIVER_PLAIN && o.driver != CHEM_DRIVER_PERSISTENT) return fail(CHEM_EINVAL, "bad driver");
+  if (o.cells_per_block < 0 || o.cells_per_block > MAX_WARPS_PER_BLOCK || o.blocks_per_sm < 0) return fail(CHEM_EINVAL, "bad launch shape");
+  if (o.couple_cells < 0 || o.couple_cells > MAX_WARPS_PER_BLOCK) return fail(CHEM_EINVAL, "couple_cells out of range");
+  if (o.couple_cells == 0) o.couple_cells = 1;
+  if (o.couple_cells > 1) {
+    if (o.lu_precision != 64) return fail(CHEM_EINVAL, "coupled cells need lu_precision 64");
+    if (o.record_adjoint) return fail(CHEM_EINVAL, "coupled cells have no adjoint");
+    const int wmax = max_warps_per_block(mech->m.dev, o.lu_precision, o.driver);
+    if (o.couple_cells > wmax) return fail(CHEM_EINVAL, "couple_cells exceeds the cells a block can hold");
+    if (o.cells_per_block % o.couple_cells) return fail(CHEM_EINVAL, "cells_per_block must be a multiple of couple_cells");
+  }
+  const int wmax = max_warps_per_block(mech->m.dev, o.lu_precision, o.driver);
+  if (wmax < 1) return fail(CHEM_EINVAL, "mechanism working set does not fit in shared memory");
+  if (o.cells_per_block > wmax) return fail(CHEM_EINVAL, "cells_per_block exceeds the shared-memory limit");
+  if (o.cells_per_block == 0) {
+    if (o.blocks_per_sm > 0)
+      o.cells_per_block = o.couple_cells > 1 ? (wmax / o.couple_cells) * o.couple_cells   // whole groups per block
+                                             : best_warps_per_block(mech->m.dev, o.lu_precision, o.driver);
+    else
+      auto_shape(mech->m.dev, o.lu_precision, o.driver, o.couple_cells, o.record_adjoint != 0, n_cells, &o.cells_per_block,
+                 &o.blocks_per_sm);
+  }
+  if (o.cells_per_block < 1) return fail(CHEM_EINVAL, "no launch shape fits on this device");
+  if (o.record_adjoint && o.lu_precision != 64)
+    return fail(CHEM_EINVAL, "record_adjoint needs lu_precision 64 (the adjoint differentiates the FP64 iteration)");
+  if (o.record_adjoint && (o.tape_steps < 0 || o.tape_steps > CHEM_MAX_TAPE_ROWS))
+    return fail(CHEM_EINVAL, "tape_steps out of range");
+  if (o.stage_wait < -1) return fail(CHEM_EINVAL, "stage_wait must be -1, 0 or positive");
+
+  chem_cells *c = new (std::nothrow) chem_cells();
+  if (!c) return fail(CHEM_ENOMEM, "host allocation failed");
+  c->mech = mech;
+  c->n = n_cells;
+  c->opts = o;
+  cudaGetDevice(&c->device);
+  const int S = mech->m.S, R = mech->m.R;
+  const size_t n = (size_t)(n_cells > 0 ? n_cells : 1);
+  cudaError_t e = cudaSuccess;
+  const bool queue = o.driver == CHEM_DRIVER_PERSISTENT || o.record_adjoint;
+  if (store) {
+    c->view = true;
+    c->T = store->T + c0;
+    c->P = store->P + c0;
+    c->y = store->y + c0 * S;
+    c->J = store->J ? store->J + c0 * mech->m.n_phot : nullptr;
+    c->stats = store->stats + c0;
+    if (queue) {
+      c->order = store->order + c0;
+      c->order_bucket = store->order_bucket + c0;
+    }
+  } else if ((e = cudaMalloc(&c->T, n * sizeof(double))) != cudaSuccess ||
+             (e = cudaMalloc(&c->P, n * sizeof(double))) != cudaSuccess ||
+             (e = cudaMalloc(&c->y, n * S * sizeof(double))) != cudaSuccess ||
+             (e = cudaMalloc(&c->stats, n * sizeof(chem_cell_stats))) != cudaSuccess ||
+             (mech->m.n_phot > 0 && (e = cudaMalloc(&c->J, n * mech->m.n_phot * sizeof(double))) != cudaSuccess)) {
+    chem_cells_destroy(c);
+    return fail(CHEM_ENOMEM, std::string("cudaMalloc failed: ") + cudaGetErrorString(e));
+  }
+  if ((e = cudaMalloc(&c->counters, 4 * sizeof(unsigned long long))) != cudaSuccess ||
+      (e = cudaMalloc(&c->theta, (R > 0 ? R : 1) * sizeof(double))) != cudaSuccess) {
+    chem_cells_destroy(c);
+    return fail(CHEM_ENOMEM, std::string("cudaMalloc failed: ") + cudaGetErrorString(e));
+  }
+  if (queue && ((!c->order && (e = cudaMalloc(&c->order, n * sizeof(int))) != cudaSuccess) ||
+                (!c->order_bucket && (e = cudaMalloc(&c->order_bucket, n * sizeof(int))) != cudaSuccess) ||
+                (e = cudaMalloc(&c->order_hist, ORDER_HIST_INTS * sizeof(int))) != cudaSuccess)) {
+    chem_cells_destroy(c);
+    return fail(CHEM_ENOMEM, std::string("cudaMalloc of the queue order failed: ") + cudaGetErrorString(e));
+  }
+  if (o.record_adjoint) {
+    c->row_cap = o.tape_steps > 0 ? o.tape_steps : 2000;
+    c->tape_cap = 3 * c->row_cap + 64;
+    const size_t E = (size_t)c->tape_cap, RC = (size_t)c->row_cap;
+    if ((e = cudaMalloc(&c->tape_kq, n * E * sizeof(int))) != cudaSuccess ||
+        (e = cudaMalloc(&c->tape_val, n * E * sizeof(double))) != cudaSuccess ||
+        (e = cudaMalloc(&c->tape_n, n * sizeof(int))) != cudaSuccess ||
+        (e = cudaMalloc(&c->tape_rows, n * sizeof(int))) != cudaSuccess ||
+        (e = cudaMalloc(&c->tape_bad, n * sizeof(int))) != cudaSuccess ||
+        (e = cudaMalloc(&c->ytape, n * RC * S * sizeof(double))) != cudaSuccess ||
+        (e = cudaMalloc(&c->gcell, n * (R > 0 ? R : 1) * sizeof(double))) != cudaSuccess ||
+        (e = cudaMalloc(&c->dLdy, n * S * sizeof(double))) != cudaSuccess ||
+        (e = cudaMalloc(&c->dLdy0, n * S * sizeof(double))) != cudaSuccess ||
+        (e = cudaMalloc(&c->dLdtheta, (R > 0 ? R : 1) * sizeof(double))) != cudaSuccess) {
+      chem_cells_destroy(c);
+      return fail(CHEM_ENOMEM, std::string("cudaMalloc of the adjoint tape failed: ") + cudaGetErrorString(e));
+    }
+  }
+  if ((e = clear_batch(c)) != cudaSuccess) {
+    chem_cells_destroy(c);
+    return cuda_fail(e, "clearing the batch");
+  }
+  *out = c;
+  return 0;
+}
 
 CellsDev solve_dev(chem_cells *c) {
   CellsDev cd{};
@@ -1065,16 +1094,17 @@ int chem_get_tape(const chem_cells *c, int64_t cell, int32_t *kind, int32_t *q, 
 // ---------------------------------------------------------------- pipeline
 // Host-resident state, chunked: per chunk its own batch and stream, so the
 // copies of one chunk overlap the solves of the others and the host's work on
-// a chunk that is back overlaps the GPU's work on the rest.
+// a chunk that is back overlaps the GPU's work on the rest.  The device memory is
+// one batch of all cells, which a run without host work uses as it is; the
+// chunks' batches are parts of it (a run takes its inputs from the host and waits
+// for its streams, so the two never meet).
 
 struct chem_pipeline {
   const chem_mech *mech = nullptr;
   int64_t n = 0;
-  chem_opts opts{};                        // as given (the whole batch picks its own launch shape)
-  chem_cells *whole = nullptr;             // all cells as one batch, made by the first run without host work
-  bool no_whole = false;                   // ... which found no memory for it
+  chem_cells *whole = nullptr;             // all cells as one batch
   std::vector<int64_t> c0;                 // chunk k is cells [c0[k], c0[k + 1])
-  std::vector<chem_cells *> sub;
+  std::vector<chem_cells *> sub;           // (one chunk: whole itself)
   std::vector<cudaStream_t> stream;
   std::vector<cudaEvent_t> done;
 };
@@ -1087,7 +1117,8 @@ void chem_pipeline_destroy(chem_pipeline *p) {
     if (e) cudaEventDestroy(e);
   for (cudaStream_t s : p->stream)
     if (s) cudaStreamDestroy(s);
-  for (chem_cells *c : p->sub) chem_cells_destroy(c);
+  for (chem_cells *c : p->sub)
+    if (c != p->whole) chem_cells_destroy(c);
   chem_cells_destroy(p->whole);
   delete p;
 }
@@ -1107,7 +1138,6 @@ int chem_pipeline_create(const chem_mech *mech, int64_t n_cells, int32_t n_chunk
   if (!p) return fail(CHEM_ENOMEM, "host allocation failed");
   p->mech = mech;
   p->n = n_cells;
-  if (opts) p->opts = *opts; else chem_opts_default(&p->opts);
   const int K = n_cells > 0 ? n_chunks : 1;
   const int64_t base = n_cells / K, extra = n_cells % K;
   p->c0.push_back(0);
@@ -1115,12 +1145,17 @@ int chem_pipeline_create(const chem_mech *mech, int64_t n_cells, int32_t n_chunk
   p->sub.assign(K, nullptr);
   p->stream.assign(K, nullptr);
   p->done.assign(K, nullptr);
+  int rc = chem_cells_create(mech, n_cells, opts, &p->whole);
+  for (int k = 0; k < K && rc == 0; ++k) {
+    if (K == 1) p->sub[k] = p->whole;
+    else rc = cells_create(mech, p->c0[k + 1] - p->c0[k], opts, p->whole, p->c0[k], &p->sub[k]);
+  }
+  if (rc) {
+    const std::string msg = g_err;
+    chem_pipeline_destroy(p);
+    return fail(rc, msg);
+  }
   for (int k = 0; k < K; ++k) {
-    if (int rc = chem_cells_create(mech, p->c0[k + 1] - p->c0[k], opts, &p->sub[k])) {
-      const std::string msg = g_err;
-      chem_pipeline_destroy(p);
-      return fail(rc, msg);
-    }
     cudaError_t e;
     if ((e = cudaStreamCreateWithFlags(&p->stream[k], cudaStreamNonBlocking)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&p->done[k], cudaEventDisableTiming)) != cudaSuccess) {
@@ -1197,19 +1232,12 @@ int chem_pipeline_run(chem_pipeline *p, const double *T, const double *P, const 
   cudaError_t e = cudaSuccess;
   int rc = 0;
   if (!fn && K > 1) {
-    if (!p->whole && !p->no_whole && chem_cells_create(p->mech, p->n, &p->opts, &p->whole) != 0) {
-      p->no_whole = true;                  // no memory for a second copy of the state: in chunks
-      cudaGetLastError();
-      g_err.clear();
-    }
-    if (p->whole) {
-      if (int drc = check_device(p->whole)) return drc;
-      e = pipeline_whole(p, T, P, J, y, dt, n_steps, stats);
-      const cudaError_t es = cudaStreamSynchronize(p->stream[0]);
-      if (e == cudaSuccess) e = es;
-      if (e != cudaSuccess) return cuda_fail(e, "pipeline");
-      return 0;
-    }
+    if (int drc = check_device(p->whole)) return drc;
+    e = pipeline_whole(p, T, P, J, y, dt, n_steps, stats);
+    const cudaError_t es = cudaStreamSynchronize(p->stream[0]);
+    if (e == cudaSuccess) e = es;
+    if (e != cudaSuccess) return cuda_fail(e, "pipeline");
+    return 0;
   }
   for (int k = 0; k < K && e == cudaSuccess; ++k) e = pipeline_enqueue(p, k, T, P, J, y, dt);
   // visit the chunks in queue order; a chunk's next step goes in as soon as its callback returns

@@ -190,10 +190,55 @@ static int pipeline_is_ordered() {
   return 0;
 }
 
+// A run allocates nothing and a pipeline holds one copy of its cells, whatever the
+// host does between the steps; a run that fails for another reason says so, and
+// the next one is as before.
+static int pipeline_memory() {
+  chem_mech *m = mechanism();
+  const chem_opts o = persistent();
+  const size_t base = fake::live;
+  const int n = 1000, K = 8;
+  chem_cells *c = nullptr;
+  CHECK(chem_cells_create(m, n, &o, &c) == 0);
+  const size_t one = fake::live - base;
+  chem_cells_destroy(c);
+  CHECK(fake::live == base);
+  chem_pipeline *p = nullptr;
+  CHECK(chem_pipeline_create(m, n, K, &o, &p) == 0);
+  const size_t held = fake::live, calls = fake::n_malloc;
+  CHECK(held - base <= one + K * (ORDER_HIST_INTS * sizeof(int) + 128));
+  Host h(n);
+  fake::device = 1;                                // another device is current
+  CHECK(h.run(p, 1, nullptr) == CHEM_EINVAL);
+  fake::device = 0;
+  for (int with = 0; with < 2; ++with) {
+    solves.clear();
+    CHECK(h.run(p, 1, with ? host_chunk : nullptr) == 0);
+    CHECK(fake::live == held && fake::n_malloc == calls);
+    CHECK(solves.size() == (with ? (size_t)K : 1u));
+    for (double v : h.y) CHECK(v == 1.0 + with);
+  }
+  chem_pipeline_destroy(p);
+  CHECK(fake::live == base);
+  for (int fit = 0; fit < (int)(calls); ++fit) {   // no memory for the allocation after `fit`
+    fake::fail_malloc = fit;
+    const int rc = chem_pipeline_create(m, n, K, &o, &p);
+    fake::fail_malloc = -1;
+    if (rc == 0) {
+      chem_pipeline_destroy(p);
+      break;
+    }
+    CHECK(rc == CHEM_ENOMEM && fake::live == base);
+  }
+  chem_mechanism_destroy(m);
+  return 0;
+}
+
 int main(int argc, char **argv) {
   const std::string what = argc > 1 ? argv[1] : "";
   if (what == "create_is_complete") return create_is_complete();
   if (what == "pipeline_is_ordered") return pipeline_is_ordered();
+  if (what == "pipeline_memory") return pipeline_memory();
   std::printf("unknown scenario\n");
   return 2;
 }
