@@ -234,11 +234,34 @@ static int pipeline_memory() {
   return 0;
 }
 
+// The chunks of a pipeline run side by side: each has the launch shape of all cells
+// together (or the one the caller gave), not that of a batch alone on the device.
+static int pipeline_shape() {
+  chem_mech *m = mechanism();
+  for (int given = 0; given < 2; ++given)
+    for (int n : {40, 100, 1000}) {
+      chem_opts o = persistent();
+      if (given) o.cells_per_block = 7;
+      chem_pipeline *p = nullptr;
+      CHECK(chem_pipeline_create(m, n, 4, &o, &p) == 0);
+      Host h(n);
+      solves.clear();
+      CHECK(h.run(p, 1, nullptr) == 0 && h.run(p, 1, host_chunk) == 0);
+      CHECK(solves.size() == 5 && solves[0].n == n);
+      for (const Solve &x : solves) CHECK(x.warps == solves[0].warps && x.bps == solves[0].bps);
+      CHECK(solves[0].warps == (given ? 7 : n < 120 ? n / 10 : 12));
+      chem_pipeline_destroy(p);
+    }
+  chem_mechanism_destroy(m);
+  return 0;
+}
+
 int main(int argc, char **argv) {
   const std::string what = argc > 1 ? argv[1] : "";
   if (what == "create_is_complete") return create_is_complete();
   if (what == "pipeline_is_ordered") return pipeline_is_ordered();
   if (what == "pipeline_memory") return pipeline_memory();
+  if (what == "pipeline_shape") return pipeline_shape();
   std::printf("unknown scenario\n");
   return 2;
 }
