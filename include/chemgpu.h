@@ -251,7 +251,8 @@ int chem_solve_step(chem_cells *cells, double dt, void *stream);
  * per step) are captured once, on an internal stream, and the graph is re-used
  * while n_steps, dt, the launch shape and the photolysis/theta sources
  * (per-cell or mechanism J, theta set or not) stay the same; any change
- * re-captures it.  The inputs it reads (T, P, y, J, theta) are the batch's
+ * re-captures it, and so does, once, the first call after the batch's first
+ * solve (persistent driver: the queue is then ordered by the cells' costs).  The inputs it reads (T, P, y, J, theta) are the batch's
  * own buffers, so set_state / set_photolysis / set_theta between launches
  * take effect.  Results are identical to n_steps chem_solve_step calls.
  * Asynchronous.  Errors: CHEM_EINVAL, CHEM_ESTATE, CHEM_ECUDA. */

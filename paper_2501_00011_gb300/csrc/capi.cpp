@@ -14,6 +14,14 @@
 
 using namespace chemgpu;
 
+// chem_solve_steps: a captured graph and what it was captured for
+struct StepsGraph {
+  cudaGraphExec_t exec = nullptr;
+  int steps = 0, w = 0, bps = 0;
+  double dt = 0.0;
+  bool J = false, theta = false;
+};
+
 struct chem_cells {
   const chem_mech *mech = nullptr;
   int64_t n = 0;
@@ -27,19 +35,18 @@ struct chem_cells {
   int *order = nullptr, *order_bucket = nullptr, *order_hist = nullptr;   // persistent driver: queue order
   double *kt = nullptr;       // chem_eval_deriv_design: rate constants [R][C], allocated on first use
   bool kt_valid = false;      // ... and current for the batch's T, P, photolysis and theta
-  bool solved = false;        // a solve of the batch has been queued: its cells have costs (stats)
+  bool solved = false;        // a solve of the batch has been launched: its cells have costs (stats)
   bool have_state = false, use_J = false, use_theta = false;
   int device = 0;
   // adjoint (record_adjoint)
   int *tape_kq = nullptr, *tape_n = nullptr, *tape_bad = nullptr, *tape_rows = nullptr;
   double *tape_val = nullptr;
   int tape_cap = 0, row_cap = 0;
-  // chem_solve_steps: the captured graph and what it was captured for
+  // chem_solve_steps: [1] once the cells have costs, whose queue order is made by
+  // another kernel (launch_order: solved); the first call's graph, which may still
+  // be running when the second call captures, stays
   cudaStream_t capture_stream = nullptr;
-  cudaGraphExec_t graph = nullptr;
-  int graph_steps = 0, graph_w = 0, graph_bps = 0;
-  double graph_dt = 0.0;
-  bool graph_J = false, graph_theta = false;
+  StepsGraph graph[2];
   double *ytape = nullptr, *gcell = nullptr, *dLdy = nullptr, *dLdy0 = nullptr, *dLdtheta = nullptr;
 };
 
@@ -217,7 +224,8 @@ int chem_cells_create(const chem_mech *mech, int64_t n_cells, const chem_opts *o
 
 void chem_cells_destroy(chem_cells *c) {
   if (!c) return;
-  if (c->graph) cudaGraphExecDestroy(c->graph);
+  for (StepsGraph &g : c->graph)
+    if (g.exec) cudaGraphExecDestroy(g.exec);
   if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
   if (!c->view) {
     cudaFree(c->T);
@@ -491,7 +499,6 @@ cudaError_t enqueue_solve(chem_cells *c, double dt, cudaStream_t s, int n_steps 
   }
   LaunchCfg cfg = launch_cfg(c->opts, dt);
   cfg.n_steps = n_steps;
-  c->solved = true;
   return launch_solve(c->mech->m.dev, cd, cfg, s);
 }
 
@@ -519,6 +526,7 @@ int chem_solve_step(chem_cells *c, double dt, void *stream) {
   cudaError_t e = clear_stage_counters(c, (cudaStream_t)stream);
   if (e == cudaSuccess) e = enqueue_solve(c, dt, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "solve kernel launch");
+  c->solved = true;
   return 0;
 }
 
@@ -529,13 +537,15 @@ int chem_solve_steps(chem_cells *c, double dt, int32_t n_steps, void *stream) {
   if (n_steps < 1 || n_steps > CHEM_MAX_GRAPH_STEPS) return fail(CHEM_EINVAL, "n_steps out of range");
   if (c->n == 0) return 0;
   cudaError_t e;
-  const bool same = c->graph && c->graph_steps == n_steps && c->graph_dt == dt &&
-                    c->graph_w == c->opts.cells_per_block && c->graph_bps == c->opts.blocks_per_sm &&
-                    c->graph_J == c->use_J && c->graph_theta == c->use_theta;
+  // only the queue of independent cells is keyed in two ways
+  const bool by_cost = c->solved && c->opts.driver == CHEM_DRIVER_PERSISTENT && c->opts.couple_cells <= 1;
+  StepsGraph &gr = c->graph[by_cost ? 1 : 0];
+  const bool same = gr.exec && gr.steps == n_steps && gr.dt == dt && gr.w == c->opts.cells_per_block &&
+                    gr.bps == c->opts.blocks_per_sm && gr.J == c->use_J && gr.theta == c->use_theta;
   if (!same) {
-    if (c->graph) {
-      cudaGraphExecDestroy(c->graph);
-      c->graph = nullptr;
+    if (gr.exec) {
+      cudaGraphExecDestroy(gr.exec);
+      gr.exec = nullptr;
     }
     if (!c->capture_stream && (e = cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking)) != cudaSuccess)
       return cuda_fail(e, "capture stream");
@@ -557,20 +567,21 @@ int chem_solve_steps(chem_cells *c, double dt, int32_t n_steps, void *stream) {
       return cuda_fail(le, "capture of the solve steps");
     }
     if (e != cudaSuccess) return cuda_fail(e, "end capture");
-    e = cudaGraphInstantiate(&c->graph, g, 0);
+    e = cudaGraphInstantiate(&gr.exec, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) {
-      c->graph = nullptr;
+      gr.exec = nullptr;
       return cuda_fail(e, "graph instantiate");
     }
-    c->graph_steps = n_steps;
-    c->graph_dt = dt;
-    c->graph_w = c->opts.cells_per_block;
-    c->graph_bps = c->opts.blocks_per_sm;
-    c->graph_J = c->use_J;
-    c->graph_theta = c->use_theta;
+    gr.steps = n_steps;
+    gr.dt = dt;
+    gr.w = c->opts.cells_per_block;
+    gr.bps = c->opts.blocks_per_sm;
+    gr.J = c->use_J;
+    gr.theta = c->use_theta;
   }
-  if ((e = cudaGraphLaunch(c->graph, (cudaStream_t)stream)) != cudaSuccess) return cuda_fail(e, "graph launch");
+  if ((e = cudaGraphLaunch(gr.exec, (cudaStream_t)stream)) != cudaSuccess) return cuda_fail(e, "graph launch");
+  c->solved = true;
   return 0;
 }
 
@@ -988,6 +999,7 @@ int chem_sensitivity_checkpointed(chem_cells *c, const double *states, int32_t n
           (e = cudaMemsetAsync(c->tape_bad, 0, n * sizeof(int), s)) != cudaSuccess ||
           (e = enqueue_solve(c, dt, s)) != cudaSuccess)
         return cuda_fail(e, "checkpointed re-solve");
+      c->solved = true;
     }
     CellsDev ca = cd;
     if ((e = launch_order_tape(ca, c->order_bucket, c->order_hist, c->order, s)) != cudaSuccess ||
@@ -1196,8 +1208,9 @@ cudaError_t pipeline_whole(chem_pipeline *p, const double *T, const double *P, c
     return e;
   c->have_state = true;
   c->kt_valid = false;
-  if ((e = enqueue_solve(c, dt, s, n_steps)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(y, c->y, n * S, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+  if ((e = enqueue_solve(c, dt, s, n_steps)) != cudaSuccess) return e;
+  c->solved = true;
+  if ((e = cudaMemcpyAsync(y, c->y, n * S, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
       (stats && (e = cudaMemcpyAsync(stats, c->stats, (size_t)p->n * sizeof(chem_cell_stats), cudaMemcpyDeviceToHost, s)) !=
                     cudaSuccess))
     return e;
@@ -1223,6 +1236,7 @@ cudaError_t pipeline_enqueue(chem_pipeline *p, int k, const double *T, const dou
   c->have_state = true;
   c->kt_valid = false;
   if ((e = enqueue_solve(c, dt, s)) != cudaSuccess) return e;
+  c->solved = true;
   if ((e = cudaMemcpy2DAsync(y + c0, ld, c->y, w, w, S, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
   return cudaEventRecord(p->done[k], s);
 }

@@ -256,12 +256,43 @@ static int pipeline_shape() {
   return 0;
 }
 
+// The queue order is keyed by the whole-warp kernel for a first solve and by lanes
+// once the cells have costs, also when the steps are a graph; a solve that was not
+// launched leaves no costs.
+static int graph_order() {
+  chem_mech *m = mechanism();
+  const chem_opts o = persistent();
+  chem_cells *c = nullptr;
+  CHECK(chem_cells_create(m, 50, &o, &c) == 0);
+  cudaStream_t s;
+  cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+  std::vector<double> T(50, 300.0), P(50, 1e5), y(150, 0.0);
+  CHECK(chem_cells_set_state(c, T.data(), P.data(), y.data(), CHEM_MEM_HOST, s) == 0);
+  solve_error = cudaErrorLaunchOutOfResources;
+  CHECK(chem_solve_step(c, 600.0, s) == CHEM_ECUDA);
+  CHECK(chem_solve_steps(c, 600.0, 3, s) == CHEM_ECUDA);
+  solve_error = cudaSuccess;
+  for (int call = 0; call < 4; ++call) {
+    solves.clear();
+    CHECK(chem_solve_steps(c, 600.0, 3, s) == 0);
+    CHECK(solves.size() == 1 && solves[0].steps == 3 && solves[0].lanes == (call > 0));
+  }
+  CHECK(chem_solve_step(c, 600.0, s) == 0 && solves.back().lanes);
+  CHECK(chem_solve_steps(c, 600.0, 2, s) == 0 && solves.back().steps == 2 && solves.back().lanes);
+  CHECK(chem_get_state(c, y.data(), CHEM_MEM_HOST, s) == 0);
+  for (double v : y) CHECK(v == 15.0);
+  chem_cells_destroy(c);
+  chem_mechanism_destroy(m);
+  return 0;
+}
+
 int main(int argc, char **argv) {
   const std::string what = argc > 1 ? argv[1] : "";
   if (what == "create_is_complete") return create_is_complete();
   if (what == "pipeline_is_ordered") return pipeline_is_ordered();
   if (what == "pipeline_memory") return pipeline_memory();
   if (what == "pipeline_shape") return pipeline_shape();
+  if (what == "graph_order") return graph_order();
   std::printf("unknown scenario\n");
   return 2;
 }
