@@ -141,9 +141,9 @@ typedef struct {
   int32_t driver;                  /* CHEM_DRIVER_* */
   int32_t cells_per_block;         /* warps (= concurrent cells) per block; 0 = auto: 1 for the
                                       plain driver, for the persistent one the most resident
-                                      cells per SM, fewer for a batch of at most three times as
-                                      many, and a batch smaller than that spread evenly over the
-                                      SMs (chem_autotune measures instead) */
+                                      cells per SM, at least 8 of them for a batch of at most 36
+                                      cells per SM, and a batch smaller than fills them spread
+                                      evenly over the SMs (chem_autotune measures instead) */
   int32_t blocks_per_sm;           /* persistent driver: resident blocks per SM; 0 = auto (as
                                       many as fit); fewer than fit are kept to by padding each
                                       block's shared memory, so the blocks spread over the SMs */

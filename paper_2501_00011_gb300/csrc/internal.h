@@ -315,6 +315,30 @@ int max_warps_per_block(const MechDev &m, int lu_precision, int driver);
 int occupancy(const MechDev &m, int lu_precision, int driver, int warps_per_block);
 // cells per block that maximises resident cells per SM (0 if nothing fits)
 int best_warps_per_block(const MechDev &m, int lu_precision, int driver);
+// Warps (cells) per SM of a persistent batch, of `full` that fit in a block, in
+// groups of `couple`.  A batch with fewer cells than that spreads evenly, one block
+// of ceil(units / SMs) cells or groups on every SM, since a cell runs the faster the
+// fewer share its SM (72/186, first solve of 301 cells: 5.5 ms against 7.3 ms as 26
+// full blocks of 12).  A few cells per warp later the batch still lasts about as
+// long as its longest cells; up to 24 cells per SM `narrow` batches take two warps
+// for each of the SM's four FP64 units, up to 36 ten warps.  ms of a first solve /
+// repeated / running, by warps per SM:
+//   72/186 (12 fit)   2,048 cells  12: 8.5/9.1/2.0    8: 7.7/7.8/1.8   10: 8.0/8.2/1.8
+//                     3,001 cells  12: 9.0/9.3/3.1    8: 8.2/8.1/2.7   10: 8.7/8.8/2.8
+//                     5,000 cells  12: 12.3/11.5/2.7  8: 12.5/11.1/2.4 10: 12.3/10.6/2.6
+//   50/130 (12 fit)   3,000 cells  12: 7.0/7.4/1.7    8: 7.0/6.4/1.8   10: 7.1/6.8/1.7
+// Never below that: with one warp a unit stands idle while it waits (100/260, where 8 fit: 1,700 cells 8: 11.9/9.3/2.4,
+// 5: 13.1/8.9/2.5; 2,400 cells 8: 13.2/12.7/2.9, 5: 15.4/13.3/3.0; 128/330, where 4
+// fit: 1,000 cells 4: 62.4/55.7/4.3, 2: 66.5/54.0/5.1).
+constexpr int NARROW_WARPS = 8, NARROW_WARPS_MORE = 10;      // up to 24, up to 36 cells per SM
+inline int shape_warps(int full, int couple, int64_t n_cells, int n_sm, bool narrow) {
+  const int64_t units = (n_cells + couple - 1) / couple;
+  const int64_t per_sm = (units + n_sm - 1) / n_sm * couple;
+  if (per_sm < full) return (int)per_sm;
+  if (narrow && per_sm <= 24) return full < NARROW_WARPS ? full : NARROW_WARPS;
+  if (narrow && per_sm <= 36) return full < NARROW_WARPS_MORE ? full : NARROW_WARPS_MORE;
+  return full;
+}
 // launch shape of a batch of n_cells in groups of `couple` whose caller gave
 // neither cells per block nor blocks per SM (0: nothing fits)
 void auto_shape(const MechDev &m, int lu_precision, int driver, int couple, bool record, int64_t n_cells,

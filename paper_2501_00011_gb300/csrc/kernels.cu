@@ -2746,21 +2746,11 @@ int best_warps_per_block(const MechDev &M, int lu_precision, int driver) {
   return best_w;
 }
 
-// Launch shape of a batch whose caller gave none.  The persistent driver fills
-// the SMs with best_warps_per_block cells each; a batch with fewer cells than
-// that (coupled: whole groups) spreads evenly instead, one block of
-// ceil(units / SMs) cells or groups on every SM, since a cell runs the faster
-// the fewer share its SM (72/186, first solve of 301 cells: 5.5 ms against
-// 7.3 ms as 26 full blocks of 12; 1,824 cells fill every SM either way).  A few
-// cells per warp later the batch still lasts about as long as its longest cells,
-// so up to two cells per resident warp the blocks hold two thirds of them, up to
-// three cells five sixths (72/186, full 12 / two thirds 8 / 10
-// cells per SM, ms: 2,048 cells first solve 8.5 / 7.7 / 8.0, repeated 9.1 / 7.8 /
-// 8.2, running 2.02 / 1.75 / 1.79; 3,001 cells 9.0 / 8.2 / 8.7, 9.3 / 8.1 / 8.8,
-// 3.1 / 2.7 / 2.8; 5,000 cells 12.3 / 12.5 / 12.3, 11.5 / 11.1 / 10.6, 2.7 / 2.4 /
-// 2.6).  A recording batch keeps the full occupancy (four recorded steps of 2,048
-// cells 13.5 / 13.8 / 14.0 ms), as do the FP32 factorisation and mechanisms small
-// enough for several blocks per SM, for which this was not measured.
+// Launch shape of a batch whose caller gave none (shape_warps, with what fits on
+// the device).  Narrowing is for the FP64 factorisation of independent cells where
+// one block fills an SM: a recording batch keeps the full occupancy (four recorded
+// steps of 2,048 cells 13.5 / 13.8 / 14.0 ms at 12 / 10 / 8 per SM), as do the FP32
+// factorisation and blocks that share an SM, for which it was not measured.
 void auto_shape(const MechDev &M, int lu_precision, int driver, int couple, bool record, int64_t n_cells,
                 int *warps_per_block, int *blocks_per_sm) {
   const int full = couple > 1 ? (max_warps_per_block(M, lu_precision, driver) / couple) * couple
@@ -2771,17 +2761,10 @@ void auto_shape(const MechDev &M, int lu_precision, int driver, int couple, bool
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   if (n_sm < 1) return;
-  const int64_t units = (n_cells + couple - 1) / couple;
-  const int64_t per_sm = (units + n_sm - 1) / n_sm * couple;
-  int64_t w = full;
-  if (per_sm < full) {
-    w = per_sm;
-  } else if (couple <= 1 && lu_precision == 64 && !record && occupancy(M, lu_precision, driver, full) == 1) {
-    if (per_sm <= 2 * full) w = 2 * full / 3;
-    else if (per_sm <= 3 * full) w = 5 * full / 6;
-  }
+  const bool narrow = couple <= 1 && lu_precision == 64 && !record && occupancy(M, lu_precision, driver, full) == 1;
+  const int w = shape_warps(full, couple, n_cells, n_sm, narrow);
   if (w < 1 || w >= full) return;
-  *warps_per_block = (int)w;
+  *warps_per_block = w;
   *blocks_per_sm = 1;
 }
 

@@ -5,6 +5,8 @@
 // usage: hostside <scenario>; exits 0 when the scenario holds, and prints why not.
 #include "fakecuda.h"
 
+#include <algorithm>
+
 #include "internal.h"
 
 using namespace chemgpu;
@@ -286,6 +288,27 @@ static int graph_order() {
   return 0;
 }
 
+// Launch shapes for every block size that a mechanism's cells may fit in: a batch
+// is narrowed to two warps per FP64 unit and never below, whole groups stay whole,
+// and a batch that cannot fill its blocks spreads over the SMs.
+static int shape_rule() {
+  const int n_sm = 152;
+  for (int full = 1; full <= MAX_WARPS_PER_BLOCK; ++full)
+    for (int64_t n = 1; n < 60 * n_sm; n += 37) {
+      const int64_t per = (n + n_sm - 1) / n_sm;
+      const int w = shape_warps(full, 1, n, n_sm, true), wide = shape_warps(full, 1, n, n_sm, false);
+      CHECK(wide == (per < full ? per : full));
+      if (per < full || per > 36) CHECK(w == wide);
+      else CHECK(w == std::min(full, per <= 24 ? 8 : 10));
+    }
+  for (int couple : {2, 3, 5})
+    for (int64_t n = couple; n < 5000; n += couple) {
+      const int full = MAX_WARPS_PER_BLOCK / couple * couple, w = shape_warps(full, couple, n, n_sm, false);
+      CHECK(w >= couple && w <= full && w % couple == 0 && (w == full || (int64_t)w * n_sm >= n));
+    }
+  return 0;
+}
+
 int main(int argc, char **argv) {
   const std::string what = argc > 1 ? argv[1] : "";
   if (what == "create_is_complete") return create_is_complete();
@@ -293,6 +316,7 @@ int main(int argc, char **argv) {
   if (what == "pipeline_memory") return pipeline_memory();
   if (what == "pipeline_shape") return pipeline_shape();
   if (what == "graph_order") return graph_order();
+  if (what == "shape_rule") return shape_rule();
   std::printf("unknown scenario\n");
   return 2;
 }
