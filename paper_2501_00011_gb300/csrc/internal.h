@@ -282,6 +282,7 @@ constexpr long long STAGE_WAIT_DEFAULT = 1LL << 22;
 struct LaunchCfg {
   int lu_precision;     // 64 / 32
   int driver;           // CHEM_DRIVER_*
+  bool dense;           // dense_solve of the batch (a pipeline's chunk: of all its cells)
   int couple;           // > 1: cells integrated in coupled groups of this many (one block each)
   int warps_per_block;
   int blocks_per_sm;
@@ -312,9 +313,16 @@ cudaError_t launch_order(const MechDev &m, const CellsDev &c, double rtol, doubl
                          int *order, cudaStream_t stream);
 int max_warps_per_block(const MechDev &m, int lu_precision, int driver);
 // resident blocks per SM of the solve kernel for a block of warps_per_block cells
-int occupancy(const MechDev &m, int lu_precision, int driver, int warps_per_block);
+int occupancy(const MechDev &m, int lu_precision, int driver, bool dense, int warps_per_block);
+// the batch runs the kernel with fewer registers and more cells per SM
+// (solve_registers): above 80 cells per SM, where it is the faster one with either
+// driver (10,000 cells, 66 per SM, 20/40 and 32/80 first solve / repeated, persistent:
+// 5.9/4.8 and 9.7/6.9 ms without, 5.3/4.5 and 9.0/8.5 with; 14,000: 7.9/6.5 and
+// 12.4/9.4, 6.8/5.6 and 11.5/9.3)
+constexpr int DENSE_CELLS_PER_SM = 80;
+bool dense_solve(const MechDev &m, int lu_precision, int64_t n_cells);
 // cells per block that maximises resident cells per SM (0 if nothing fits)
-int best_warps_per_block(const MechDev &m, int lu_precision, int driver);
+int best_warps_per_block(const MechDev &m, int lu_precision, int driver, bool dense);
 // Warps (cells) per SM of a persistent batch, of `full` that fit in a block, in
 // groups of `couple`.  A batch with fewer cells than that spreads evenly, one block
 // of ceil(units / SMs) cells or groups on every SM, since a cell runs the faster the
@@ -341,7 +349,7 @@ inline int shape_warps(int full, int couple, int64_t n_cells, int n_sm, bool nar
 }
 // launch shape of a batch of n_cells in groups of `couple` whose caller gave
 // neither cells per block nor blocks per SM (0: nothing fits)
-void auto_shape(const MechDev &m, int lu_precision, int driver, int couple, bool record, int64_t n_cells,
+void auto_shape(const MechDev &m, int lu_precision, int driver, bool dense, int couple, bool record, int64_t n_cells,
                 int *warps_per_block, int *blocks_per_sm);
 // diagnostic: mode 0 out = f(y); mode 1 out = (I - c J(y))^{-1} b   (all [S][C] device arrays)
 cudaError_t launch_probe(const MechDev &M, const CellsDev &C, int lu_precision, int mode, double c, const double *y,

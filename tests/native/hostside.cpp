@@ -14,6 +14,7 @@ using namespace chemgpu;
 struct Solve {
   int64_t n;
   int warps, bps, steps;
+  bool dense;
   bool lanes;           // the queue order was made by lanes (launch_order: solved)
 };
 static std::vector<Solve> solves;
@@ -33,10 +34,11 @@ cudaError_t set_constants() { return cudaSuccess; }
 size_t smem_per_cell(const MechDev &, int) { return 16384; }
 size_t staged_bytes(const MechDev &, int) { return 0; }
 int max_warps_per_block(const MechDev &, int, int) { return 12; }
-int best_warps_per_block(const MechDev &, int, int driver) { return driver == CHEM_DRIVER_PERSISTENT ? 12 : 1; }
-int occupancy(const MechDev &, int, int, int w) { return w <= 12 ? 12 / w : 0; }
+int best_warps_per_block(const MechDev &, int, int driver, bool) { return driver == CHEM_DRIVER_PERSISTENT ? 12 : 1; }
+int occupancy(const MechDev &, int, int, bool, int w) { return w <= 12 ? 12 / w : 0; }
 // the cells of a batch spread over 10 SMs
-void auto_shape(const MechDev &, int, int driver, int, bool, int64_t n, int *w, int *bps) {
+bool dense_solve(const MechDev &, int prec, int64_t n) { return prec == 32 && n > 10 * DENSE_CELLS_PER_SM; }
+void auto_shape(const MechDev &, int, int driver, bool, int, bool, int64_t n, int *w, int *bps) {
   const int64_t per = (n + 9) / 10;
   if (driver != CHEM_DRIVER_PERSISTENT) { *w = 1; return; }
   *w = per < 12 ? (int)(per < 1 ? 1 : per) : 12;
@@ -81,7 +83,7 @@ cudaError_t launch_solve(const MechDev &m, const CellsDev &c, const LaunchCfg &c
     }
     for (int64_t i = 0; i < cd.n_cells * S; ++i) cd.y[i] += k;
     for (int64_t i = 0; i < cd.n_cells; ++i) cd.stats[i].steps = k;
-    solves.push_back({cd.n_cells, f.warps_per_block, f.blocks_per_sm, k, order_lanes});
+    solves.push_back({cd.n_cells, f.warps_per_block, f.blocks_per_sm, k, f.dense, order_lanes});
   });
   return cudaSuccess;
 }
@@ -243,14 +245,14 @@ static int pipeline_shape() {
   for (int given = 0; given < 2; ++given)
     for (int n : {40, 100, 1000}) {
       chem_opts o = persistent();
-      if (given) o.cells_per_block = 7;
+      if (given) o.cells_per_block = 7, o.lu_precision = 32;
       chem_pipeline *p = nullptr;
       CHECK(chem_pipeline_create(m, n, 4, &o, &p) == 0);
       Host h(n);
       solves.clear();
       CHECK(h.run(p, 1, nullptr) == 0 && h.run(p, 1, host_chunk) == 0);
       CHECK(solves.size() == 5 && solves[0].n == n);
-      for (const Solve &x : solves) CHECK(x.warps == solves[0].warps && x.bps == solves[0].bps);
+      for (const Solve &x : solves) CHECK(x.warps == solves[0].warps && x.bps == solves[0].bps && x.dense == (given && n == 1000));
       CHECK(solves[0].warps == (given ? 7 : n < 120 ? n / 10 : 12));
       chem_pipeline_destroy(p);
     }
