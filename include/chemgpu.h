@@ -365,7 +365,8 @@ int chem_get_tape(const chem_cells *cells, int64_t cell, int32_t *kind, int32_t 
                   int32_t capacity, int32_t *n_events, int32_t *n_rows);
 
 /* Designs of the derivative f(y) for chem_eval_deriv_design. */
-#define CHEM_DERIV_GATHER 0       /* this library's: one warp per cell, the compiled f program, no atomics */
+#define CHEM_DERIV_GATHER 0       /* this library's: tiles of 32 cells, one lane per cell, and one warp per cell
+                                     (the compiled f program) for the rest and small batches; no atomics */
 #define CHEM_DERIV_ATOMIC_AOS 1   /* the paper's: one thread per reaction and cell, FP64 atomic adds into f,
                                      reaction data as an array of structures */
 #define CHEM_DERIV_ATOMIC_SOA 2   /* the same with the reaction data as a structure of arrays */

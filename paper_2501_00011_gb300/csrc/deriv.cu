@@ -5,8 +5,8 @@
 // its contributions to the species' rates of change with atomic additions;
 // reorganising the reaction data for the GPU gave a further speedup.  This
 // file builds that design (reaction data as an array of structures or as a
-// structure of arrays) so it can be measured against this library's gather,
-// one warp per cell running the compiled f program (kernels.cu), on the same
+// structure of arrays) so it can be measured against this library's own
+// (kernels.cu: tiles of 32 cells and the compiled f program, no atomics) on the same
 // inputs: the rate constants of the batch computed once, y and f in HBM.
 #include <cuda_runtime.h>
 

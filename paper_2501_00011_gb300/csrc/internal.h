@@ -28,7 +28,7 @@ constexpr int TAN_WARPS_PER_BLOCK = 4;   // ... and of the tangent walk (a large
 // scheduler guarantees that no location written in a pass is read or written
 // by another op of the same pass, so the passes run without intra-pass races.
 // On the host an op holds element indices:
-//   FMA op:    W[t] = fma(W[a], W[b], W[c])      (NEG program: fma(-W[a], W[b], W[c]))
+//   FMA op:    W[t] = fma(W[a], W[b], W[c])
 //   RECIP op:  W[t & 0x7fff] = -1 / W[a]         (t has bit 15 set)
 //   empty:     t == 0xffff
 // On the device the same op holds BYTE offsets into the cell's work array,
@@ -369,7 +369,8 @@ cudaError_t launch_count_flags(const int *flag, int64_t n, unsigned long long *a
 cudaError_t launch_rates(const MechDev &m, const CellsDev &c, double *kt, cudaStream_t stream);
 cudaError_t launch_deriv_design(const MechDev &m, const CellsDev &c, int design, const double *kt, const double *y,
                                 double *f, cudaStream_t stream);
-// kernels.cu: the gather design (one warp per cell, the compiled f program)
+// kernels.cu: this library's design, without atomics (tiles of 32 cells, one lane per
+// cell; the compiled f program, one warp per cell, for the rest)
 cudaError_t launch_deriv_gather(const MechDev &m, const CellsDev &c, const double *kt, const double *y, double *f,
                                 cudaStream_t stream);
 

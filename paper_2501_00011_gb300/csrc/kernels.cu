@@ -92,9 +92,6 @@ __device__ __forceinline__ double recip_nr(double x) {
   const double e = fma(-x, r, 1.0);
   return fma(r, fma(e, e, e), r);
 }
-__device__ __forceinline__ double lu_recip(double x) { return recip_nr(x); }
-__device__ __forceinline__ float lu_recip(float x) { return __frcp_rn(x); }
-
 template <typename T>
 __device__ __forceinline__ T &at(unsigned char *base, unsigned off) {
   return *reinterpret_cast<T *>(base + off);
@@ -659,7 +656,7 @@ __device__ __forceinline__ void mlu_core(const MechDev &M, const SolveParams &P,
   __syncwarp();
   // The M program runs on the whole per-cell slice (its operands are the pair
   // products in Wd and the LU slots, constants and temporaries in WL), its ops
-  // read from L2 two passes ahead.  The LU program's ops are streamed through a
+  // read from L2 two groups ahead.  The LU program's ops are streamed through a
   // ring in the rates and f slots of Wd, dead once M is formed (too small a
   // region: read from L2 as well).
   run_prog<T, false>(GlobalStream(M.m_ops[prec], lane), M.m_runs, M.m_nruns, reinterpret_cast<T *>(Wd));
