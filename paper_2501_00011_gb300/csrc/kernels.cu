@@ -2522,7 +2522,8 @@ constexpr int GATHER_WARPS = 16;                // most gather warps of a block
 struct DerivSplit {
   int64_t n_tiles;         // tiles of 32 cells, dealt to the blocks in turn, then to a block's groups
   int tile_warps;          // of a block: TILE_GROUPS * TILE_WARPS, or 0 without tiles
-  int gather_cells;        // gather warps (one cell each) per block
+  int gather_cells;        // cells of a block by the gather, one warp each
+  int gather_warps;        // warps that bring their tables and inputs in
   int cell_doubles;        // a gather cell's slice
   int tile_doubles;        // a tile buffer
 };
@@ -2649,22 +2650,30 @@ __global__ void __launch_bounds__(32 * WARP) deriv_gather_kernel(const __grid_co
   }
   warp -= D.tile_warps;
   const int64_t c0 = D.n_tiles * TILE_CELLS + (int64_t)blockIdx.x * D.gather_cells;
-  if (c0 >= NC) return;                         // all the block's gather warps
+  if (c0 >= NC) return;                         // all the block's gather warps (gather_warps >= gather_cells)
   const int nb = (int)((NC - c0) < D.gather_cells ? (NC - c0) : D.gather_cells);    // cells of this block
   // the hot table prefix (f program, reactant slots), then the cells' slices
   unsigned char *const gs = smem + (D.tile_warps ? (size_t)TILE_GROUPS * D.tile_doubles * sizeof(double) : 0);
-  const int tid = warp * WARP + lane, nt = D.gather_cells * WARP;
+  const int tid = warp * WARP + lane, nt = D.gather_warps * WARP;
   const int tb = M.tab.staged;
-  for (int i = tid; i < tb / 16; i += nt)
-    reinterpret_cast<uint4 *>(gs)[i] = __ldg(reinterpret_cast<const uint4 *>(M.blob[0]) + i);
+  // (what f reads of it, each section at its place; the op that the interpreter reads
+  // past the program's end is not run)
+  auto stage = [&](int from, int bytes) {
+    for (int i = from / 16 + tid; i < (from + bytes + 15) / 16; i += nt)
+      reinterpret_cast<uint4 *>(gs)[i] = __ldg(reinterpret_cast<const uint4 *>(M.blob[0]) + i);
+  };
+  stage(M.tab.f_ops, M.tab.f_runs - M.tab.f_ops + (M.f_nruns + 1) * (int)sizeof(uint32_t));
+  stage(M.tab.rx_slots, M.R * (int)sizeof(uint2));
   double *sm = reinterpret_cast<double *>(gs + tb);
   // element (row, cell) -> slice of cell, slot row
-  // (cells fastest; a thread's cell stays the same, its row goes up by nt / gather_cells)
-  const int cl = tid % D.gather_cells, r0 = tid / D.gather_cells;
+  // (cells fastest; a thread's cell stays the same, its row goes up by the rows in
+  // flight; the threads of a last, incomplete row rest)
+  const int cl = tid % D.gather_cells, r0 = tid / D.gather_cells, dr = nt / D.gather_cells;
   double *const mine = sm + (size_t)cl * D.cell_doubles;
-  if (cl < nb) {
-    for (int r = r0; r < M.S; r += WARP) mine[M.d_Y + r] = y[(int64_t)r * NC + c0 + cl];
-    for (int r = r0; r < M.R; r += WARP) mine[M.d_KT + r] = kt[(int64_t)r * NC + c0 + cl];
+  const bool moves = cl < nb && r0 < dr;
+  if (moves) {
+    for (int r = r0; r < M.S; r += dr) mine[M.d_Y + r] = y[(int64_t)r * NC + c0 + cl];
+    for (int r = r0; r < M.R; r += dr) mine[M.d_KT + r] = kt[(int64_t)r * NC + c0 + cl];
   }
   if (warp < nb) {
     unsigned char *wd = reinterpret_cast<unsigned char *>(sm + (size_t)warp * D.cell_doubles);
@@ -2672,11 +2681,11 @@ __global__ void __launch_bounds__(32 * WARP) deriv_gather_kernel(const __grid_co
     for (int k = lane; k < M.d_nconst; k += WARP)
       at<double>(wd, reinterpret_cast<const int *>(gb + M.tab.dconst_off)[k]) = reinterpret_cast<const double *>(gb + M.tab.dconst_val)[k];
   }
-  group_sync(GATHER_BAR, D.gather_cells);
+  group_sync(GATHER_BAR, D.gather_warps);
   if (warp < nb) f_core<true>(M, P, gs, sm + (size_t)warp * D.cell_doubles, lane);
-  group_sync(GATHER_BAR, D.gather_cells);
-  if (cl < nb)
-    for (int r = r0; r < M.S; r += WARP) f[(int64_t)r * NC + c0 + cl] = mine[M.d_F + r];
+  group_sync(GATHER_BAR, D.gather_warps);
+  if (moves)
+    for (int r = r0; r < M.S; r += dr) f[(int64_t)r * NC + c0 + cl] = mine[M.d_F + r];
 }
 
 bool staged_driver(int driver) { return driver == CHEM_DRIVER_PERSISTENT; }
@@ -2948,6 +2957,11 @@ cudaError_t launch_deriv_gather(const MechDev &M, const CellsDev &C, const doubl
     if (fit < 1) return cudaErrorInvalidValue;
     const int64_t per_sm = (rest + n_sm - 1) / n_sm;
     D.gather_cells = (int)(per_sm < fit ? per_sm : fit);
+    // with few cells per block the copy of the tables takes most of the time, so the
+    // block has all its warps all the same (one warp per cell copying the whole
+    // prefix: 10 cells of 72 species 18.8 us, 10.9 so; of 128 species 27.1, 11.2;
+    // 10,000 of 128 species, which have no tiles, 82.5 with the whole prefix, 78.5)
+    D.gather_warps = used ? 32 - TILE_GROUPS * TILE_WARPS : GATHER_WARPS;
     const int64_t need = (rest + D.gather_cells - 1) / D.gather_cells;
     blocks = D.n_tiles > 0 && need < n_sm ? n_sm : need;      // with tiles per_sm <= fit, so need <= n_sm
   }
@@ -2957,7 +2971,7 @@ cudaError_t launch_deriv_gather(const MechDev &M, const CellsDev &C, const doubl
                                   : 0);
   const cudaError_t e = allow_max_smem<deriv_gather_kernel>();
   if (e != cudaSuccess) return e;
-  deriv_gather_kernel<<<(unsigned)blocks, (D.tile_warps + D.gather_cells) * WARP, smem, stream>>>(M, C.n_cells, kt, y, f, D,
+  deriv_gather_kernel<<<(unsigned)blocks, (D.tile_warps + D.gather_warps) * WARP, smem, stream>>>(M, C.n_cells, kt, y, f, D,
                                                                                                 SolveParams{});
   return cudaGetLastError();
 }

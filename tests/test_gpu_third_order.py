@@ -45,9 +45,11 @@ def _workload(name, n, seed=41):
     return synth.Workload(m.name + "_3rd", m, cells, 600.0, 1, 1e-4, 1e-10)
 
 
-# too few cells for a tile; one round of 32 cells on every SM and its edges; a ragged rest
+# too few cells for a tile, with 1, 3 and 7 per block (3 and 7 do not divide its threads);
+# one round of 32 cells on every SM and its edges; a ragged rest
 @pytest.mark.parametrize("name", list(MECHS))
-@pytest.mark.parametrize("rounds,rest", [(0, 1), (0, 33), (1, -1), (1, 1), (1, 3333), (2, 271)])
+@pytest.mark.parametrize("rounds,rest", [(0, 1), (0, 33), (0, 437), (0, 1063), (1, -1), (1, 1), (1, 437), (1, 3333),
+                                         (2, 271)])
 def test_tiles_equal_the_f_program(oracle_lib, cg, name, rounds, rest):
     prop = torch.cuda.get_device_properties(0)
     n = rounds * 32 * prop.multi_processor_count + rest
