@@ -31,7 +31,7 @@ struct chem_cells {
   // device counters: [0] persistent work queue, [1] staging fallbacks and
   // [2] unfinished staging copies of the last solve call (CellsDev::stage), [3] spare
   unsigned long long *counters = nullptr;
-  bool dense = false;         // dense_solve of the batch's cells (a view's: of its store's)
+  int regs = 168;             // solve_registers of the batch's cells (a view's: of its store's)
   bool view = false;          // the per-cell arrays belong to another batch (cells_create)
   int *order = nullptr, *order_bucket = nullptr, *order_hist = nullptr;   // persistent driver: queue order
   double *kt = nullptr;       // chem_eval_deriv_design: rate constants [R][C], allocated on first use
@@ -348,7 +348,7 @@ int cells_create(const chem_mech *mech, int64_t n_cells, const chem_opts *opts, 
   const int wmax = max_warps_per_block(mech->m.dev, o.lu_precision, o.driver);
   if (wmax < 1) return fail(CHEM_EINVAL, "mechanism working set does not fit in shared memory");
   if (o.cells_per_block > wmax) return fail(CHEM_EINVAL, "cells_per_block exceeds the shared-memory limit");
-  const bool dense = store ? store->dense : dense_solve(mech->m.dev, o.lu_precision, n_cells);
+  const int regs = store ? store->regs : solve_registers(mech->m.dev, o.lu_precision, o.driver, o.couple_cells, n_cells);
   if (o.cells_per_block == 0 && store) {
     // batches of one pipeline run side by side: the shape of all their cells, which
     // bounds the warps per SM for all of them (a shape of its own would spread each
@@ -361,9 +361,9 @@ int cells_create(const chem_mech *mech, int64_t n_cells, const chem_opts *opts, 
   if (o.cells_per_block == 0) {
     if (o.blocks_per_sm > 0)
       o.cells_per_block = o.couple_cells > 1 ? (wmax / o.couple_cells) * o.couple_cells   // whole groups per block
-                                             : best_warps_per_block(mech->m.dev, o.lu_precision, o.driver, dense);
+                                             : best_warps_per_block(mech->m.dev, o.lu_precision, o.driver, regs);
     else
-      auto_shape(mech->m.dev, o.lu_precision, o.driver, dense, o.couple_cells, o.record_adjoint != 0, n_cells,
+      auto_shape(mech->m.dev, o.lu_precision, o.driver, regs, o.couple_cells, o.record_adjoint != 0, n_cells,
                  &o.cells_per_block, &o.blocks_per_sm);
   }
   if (o.cells_per_block < 1) return fail(CHEM_EINVAL, "no launch shape fits on this device");
@@ -378,7 +378,7 @@ int cells_create(const chem_mech *mech, int64_t n_cells, const chem_opts *opts, 
   c->mech = mech;
   c->n = n_cells;
   c->opts = o;
-  c->dense = dense;
+  c->regs = regs;
   cudaGetDevice(&c->device);
   const int S = mech->m.S, R = mech->m.R;
   const size_t n = (size_t)(n_cells > 0 ? n_cells : 1);
@@ -465,7 +465,7 @@ CellsDev solve_dev(chem_cells *c) {
 LaunchCfg launch_cfg(const chem_cells *c, double dt) {
   const chem_opts &o = c->opts;
   LaunchCfg cfg{};
-  cfg.dense = c->dense;
+  cfg.regs = c->regs;
   cfg.lu_precision = o.lu_precision;
   cfg.driver = o.driver;
   cfg.couple = o.couple_cells;
@@ -648,7 +648,7 @@ int chem_autotune(chem_cells *c, double dt, int64_t n_sample, int32_t *cells_per
   float best = 0.0f;
   int best_w = 0, best_b = 0;
   for (int w = 1; w <= wmax && rc == 0; ++w) {
-    const int occ = occupancy(M, prec, drv, c->dense, w);
+    const int occ = occupancy(M, prec, drv, c->regs, w);
     if (occ < 1) continue;
     const int nb = drv == CHEM_DRIVER_PERSISTENT ? occ : 1;
     for (int b = 1; b <= nb && rc == 0; ++b) {

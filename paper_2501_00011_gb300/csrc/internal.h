@@ -282,7 +282,7 @@ constexpr long long STAGE_WAIT_DEFAULT = 1LL << 22;
 struct LaunchCfg {
   int lu_precision;     // 64 / 32
   int driver;           // CHEM_DRIVER_*
-  bool dense;           // dense_solve of the batch (a pipeline's chunk: of all its cells)
+  int regs;             // solve_registers of the batch (a pipeline's chunk: of all its cells)
   int couple;           // > 1: cells integrated in coupled groups of this many (one block each)
   int warps_per_block;
   int blocks_per_sm;
@@ -313,16 +313,30 @@ cudaError_t launch_order(const MechDev &m, const CellsDev &c, double rtol, doubl
                          int *order, cudaStream_t stream);
 int max_warps_per_block(const MechDev &m, int lu_precision, int driver);
 // resident blocks per SM of the solve kernel for a block of warps_per_block cells
-int occupancy(const MechDev &m, int lu_precision, int driver, bool dense, int warps_per_block);
-// the batch runs the kernel with fewer registers and more cells per SM
-// (solve_registers): above 80 cells per SM, where it is the faster one with either
-// driver (10,000 cells, 66 per SM, 20/40 and 32/80 first solve / repeated, persistent:
-// 5.9/4.8 and 9.7/6.9 ms without, 5.3/4.5 and 9.0/8.5 with; 14,000: 7.9/6.5 and
-// 12.4/9.4, 6.8/5.6 and 11.5/9.3)
-constexpr int DENSE_CELLS_PER_SM = 80;
-bool dense_solve(const MechDev &m, int lu_precision, int64_t n_cells);
+int occupancy(const MechDev &m, int lu_precision, int driver, int regs, int warps_per_block);
+// Registers of a solve kernel's thread.  A sub-partition's 16,384 hold 3 warps at up
+// to 168 (a block of 12 warps on the SM), 4 at 128, 6 at 80.  Shared memory holds 12
+// cells or fewer of 72 species and more, so those kernels take 168.  Of up to 32
+// species it holds 24 and more (ms of a first solve, 20/40, at 168 / 128 / 80):
+//   plain driver, more than 12 cells per SM: 128 (FP64: 2,000 cells 2.6 / 2.5 / 2.7,
+//   20,000 13.8 / 13.3 / 12.7, 50,000 32.5 / 31.3 / 29.2; but 10 cells at rtol 1e-8
+//   3.55 / 3.59 / 4.10, which is why fewer keep 168);
+//   FP32 factorisation, more than 80 cells per SM: 80, since what a warp waits for is
+//   latency, not the FP64 unit (plain: 5,000 cells 4.0 / 3.7 / 3.7, 10,000 6.8 / 6.0 /
+//   5.9, 20,000 12.7 / 11.0 / 10.3, 50,000 29.9 / 25.6 / 23.6; persistent: 2,000 cells
+//   2.0 / 2.0 / 2.3, 10,000 5.9 / 5.6 / 5.3 and repeated 4.8 / 4.4 / 4.5, with 32/80
+//   6.9 / 7.7 / 8.5, 14,000 7.9 / 7.3 / 6.8, 50,000 25.3 / 23.5 / 21.6);
+//   the persistent FP64 kernel 168: its narrow batches gain more from few warps
+//   (repeated solve: 3,500 cells 2.7 / 3.3 / 3.3, 20,000 11.3 / 10.9 / 10.8).
+inline int register_rule(int n_species, int lu_precision, int driver, int couple, int64_t n_cells, int n_sm) {
+  if (n_species > WARP || couple > 1) return 168;
+  if (lu_precision == 32 && n_cells > (int64_t)80 * n_sm) return 80;
+  if (driver == CHEM_DRIVER_PLAIN && n_cells > (int64_t)12 * n_sm) return 128;
+  return 168;
+}
+int solve_registers(const MechDev &m, int lu_precision, int driver, int couple, int64_t n_cells);
 // cells per block that maximises resident cells per SM (0 if nothing fits)
-int best_warps_per_block(const MechDev &m, int lu_precision, int driver, bool dense);
+int best_warps_per_block(const MechDev &m, int lu_precision, int driver, int regs);
 // Warps (cells) per SM of a persistent batch, of `full` that fit in a block, in
 // groups of `couple`.  A batch with fewer cells than that spreads evenly, one block
 // of ceil(units / SMs) cells or groups on every SM, since a cell runs the faster the
@@ -349,7 +363,7 @@ inline int shape_warps(int full, int couple, int64_t n_cells, int n_sm, bool nar
 }
 // launch shape of a batch of n_cells in groups of `couple` whose caller gave
 // neither cells per block nor blocks per SM (0: nothing fits)
-void auto_shape(const MechDev &m, int lu_precision, int driver, bool dense, int couple, bool record, int64_t n_cells,
+void auto_shape(const MechDev &m, int lu_precision, int driver, int regs, int couple, bool record, int64_t n_cells,
                 int *warps_per_block, int *blocks_per_sm);
 // diagnostic: mode 0 out = f(y); mode 1 out = (I - c J(y))^{-1} b   (all [S][C] device arrays)
 cudaError_t launch_probe(const MechDev &M, const CellsDev &C, int lu_precision, int mode, double c, const double *y,

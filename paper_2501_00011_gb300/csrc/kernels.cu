@@ -1379,27 +1379,12 @@ __device__ bool stage_tables(const unsigned char *blob, int bytes, unsigned char
   return ok;
 }
 
-// Registers of a solve kernel's thread.  A sub-partition's 16,384 hold 3 warps at up
-// to 168 (a block of 12 warps on the SM), 4 at 128, 6 at 80.  72 species and more
-// fill an SM's shared memory with 12 cells or fewer, so their kernels take 168.  Up
-// to 32 species (KS = 1), where shared memory holds 24 and more:
-//   plain driver, 128: 16 cells per SM for a few spilled bytes (20/40, FP64, first
-//   solve in ms at 168 / 128 / 80: 2,000 cells 2.6 / 2.5 / 2.7, 20,000 13.8 / 13.3 /
-//   12.7, 50,000 32.5 / 31.3 / 29.2; 10 cells 1.05 / 1.06 / 1.22);
-//   FP32 factorisation in large batches (dense_solve), 80: 24 cells per SM, since
-//   what a warp waits for is latency, not the FP64 unit (20/40, plain: 5,000 cells
-//   4.0 / 3.7 / 3.7, 10,000 6.8 / 6.0 / 5.9, 20,000 12.7 / 11.0 / 10.3, 50,000 29.9 /
-//   25.6 / 23.6; persistent: 10,000 5.9 / 5.6 / 5.3, 20,000 10.8 / 10.1 / 9.4, 50,000
-//   25.3 / 23.5 / 21.6, but 2,000 2.0 / 2.0 / 2.3);
-//   the persistent FP64 kernel, 168: its narrow batches gain more from few warps
-//   (20/40, repeated solve: 3,500 cells 2.7 / 3.3 / 3.3, 20,000 11.3 / 10.9 / 10.8).
-// (Without a bound the compiler gave some of these kernels 80 and others 150.)
-constexpr int solve_registers(int ks, bool staged, bool coupled, bool dense) {
-  return dense ? 80 : ks == 1 && !staged && !coupled ? 128 : 168;
-}
-
-template <typename T, int KS, bool STAGED, bool REC, bool COUPLED, bool DENSE>
-__global__ void __maxnreg__(solve_registers(KS, STAGED, COUPLED, DENSE)) solve_kernel(const __grid_constant__ MechDev M, const CellsDev C, const SolveParams P) {
+// REGS: the registers a thread may have (solve_registers).  Without a bound the
+// compiler gave some of these kernels 80 and others 150.  At 168 those for up to 96
+// species keep everything in registers but for a few bytes of the plain ones; those
+// for 97 to 128 spill 88 to 370 bytes.
+template <typename T, int KS, bool STAGED, bool REC, bool COUPLED, int REGS>
+__global__ void __maxnreg__(REGS) solve_kernel(const __grid_constant__ MechDev M, const CellsDev C, const SolveParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(8) uint64_t tma_bar;
   __shared__ double grp_slot[COUPLED ? MAX_WARPS_PER_BLOCK : 1];
@@ -1545,7 +1530,7 @@ cudaError_t launch_probe_t(const MechDev &M, const CellsDev &C, const SolveParam
   return cudaGetLastError();
 }
 
-template <typename T, int KS, bool STAGED, bool REC, bool COUPLED, bool DENSE>
+template <typename T, int KS, bool STAGED, bool REC, bool COUPLED, int REGS>
 cudaError_t configure_t() {
   static bool configured[64] = {false};
   int dev = 0;
@@ -1554,75 +1539,78 @@ cudaError_t configure_t() {
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   cudaFuncAttributes fa;
-  cudaError_t e = cudaFuncGetAttributes(&fa, solve_kernel<T, KS, STAGED, REC, COUPLED, DENSE>);
+  cudaError_t e = cudaFuncGetAttributes(&fa, solve_kernel<T, KS, STAGED, REC, COUPLED, REGS>);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(solve_kernel<T, KS, STAGED, REC, COUPLED, DENSE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  e = cudaFuncSetAttribute(solve_kernel<T, KS, STAGED, REC, COUPLED, REGS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            optin - (int)fa.sharedSizeBytes);
   if (e == cudaSuccess && dev < 64) configured[dev] = true;
   return e;
 }
 
-template <typename T, int KS, bool STAGED, bool DENSE>
+template <typename T, int KS, bool STAGED, int REGS = 168>
 int occupancy_t(int warps_per_block, size_t smem) {
-  if (configure_t<T, KS, STAGED, false, false, DENSE>() != cudaSuccess) return 0;
+  if (configure_t<T, KS, STAGED, false, false, REGS>() != cudaSuccess) return 0;
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, solve_kernel<T, KS, STAGED, false, false, DENSE>,
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, solve_kernel<T, KS, STAGED, false, false, REGS>,
                                                     warps_per_block * WARP, smem) != cudaSuccess)
     return 0;
   return n;
 }
 
-template <typename T, int KS, bool STAGED, bool REC, bool COUPLED, bool DENSE = false>
+template <typename T, int KS, bool STAGED, bool REC, bool COUPLED, int REGS = 168>
 cudaError_t launch_rec_t(const MechDev &M, const CellsDev &C, const SolveParams &P, int blocks, cudaStream_t stream) {
   const size_t smem = P.smem_bytes > 0 ? (size_t)P.smem_bytes : (size_t)P.tab_bytes + (size_t)P.cell_bytes * P.warps_per_block;
-  cudaError_t e = configure_t<T, KS, STAGED, REC, COUPLED, DENSE>();
+  cudaError_t e = configure_t<T, KS, STAGED, REC, COUPLED, REGS>();
   if (e != cudaSuccess) return e;
-  solve_kernel<T, KS, STAGED, REC, COUPLED, DENSE><<<blocks, P.warps_per_block * WARP, smem, stream>>>(M, C, P);
+  solve_kernel<T, KS, STAGED, REC, COUPLED, REGS><<<blocks, P.warps_per_block * WARP, smem, stream>>>(M, C, P);
   return cudaGetLastError();
 }
 
 // The recording kernel and the coupled (multi-cell) kernel exist for the
-// FP64 iteration only, the dense one for the FP32 factorisation of up to 32
-// species; they do not combine.
-template <typename T, int KS>
-constexpr bool has_dense = std::is_same<T, float>::value && KS == 1;
-
+// FP64 iteration only; they do not combine.  Fewer registers than 168: kernels of up
+// to 32 species (KS = 1), 128 with the plain driver, 80 with the FP32 factorisation.
 template <typename T, int KS, bool STAGED>
-cudaError_t launch_t(const MechDev &M, const CellsDev &C, const SolveParams &P, int blocks, bool coupled, bool dense,
+cudaError_t launch_t(const MechDev &M, const CellsDev &C, const SolveParams &P, int blocks, bool coupled, int regs,
                      cudaStream_t stream) {
   if constexpr (std::is_same<T, double>::value) {
     if (C.tape_n && coupled) return cudaErrorInvalidValue;
-    if (C.tape_n) return launch_rec_t<T, KS, STAGED, true, false>(M, C, P, blocks, stream);
     if (coupled) return launch_rec_t<T, KS, STAGED, false, true>(M, C, P, blocks, stream);
+    if constexpr (KS == 1 && !STAGED)
+      if (C.tape_n && regs == 128) return launch_rec_t<T, KS, STAGED, true, false, 128>(M, C, P, blocks, stream);
+    if (C.tape_n) return launch_rec_t<T, KS, STAGED, true, false>(M, C, P, blocks, stream);
   } else {
     if (C.tape_n || coupled) return cudaErrorInvalidValue;
+    if constexpr (KS == 1)
+      if (regs == 80) return launch_rec_t<T, KS, STAGED, false, false, 80>(M, C, P, blocks, stream);
   }
-  if constexpr (has_dense<T, KS>)
-    if (dense) return launch_rec_t<T, KS, STAGED, false, false, true>(M, C, P, blocks, stream);
+  if constexpr (KS == 1 && !STAGED)
+    if (regs == 128) return launch_rec_t<T, KS, STAGED, false, false, 128>(M, C, P, blocks, stream);
   return launch_rec_t<T, KS, STAGED, false, false>(M, C, P, blocks, stream);
 }
 
 template <typename T, bool STAGED>
-int occupancy_ks(const MechDev &M, bool dense, int warps_per_block, size_t smem) {
-  if constexpr (has_dense<T, 1>)
-    if (dense) return occupancy_t<T, 1, STAGED, true>(warps_per_block, smem);
+int occupancy_ks(const MechDev &M, int regs, int warps_per_block, size_t smem) {
+  if constexpr (std::is_same<T, float>::value)
+    if (regs == 80) return occupancy_t<T, 1, STAGED, 80>(warps_per_block, smem);
+  if constexpr (!STAGED)
+    if (regs == 128) return occupancy_t<T, 1, STAGED, 128>(warps_per_block, smem);
   switch ((M.S + WARP - 1) / WARP) {
-    case 1: return occupancy_t<T, 1, STAGED, false>(warps_per_block, smem);
-    case 2: return occupancy_t<T, 2, STAGED, false>(warps_per_block, smem);
-    case 3: return occupancy_t<T, 3, STAGED, false>(warps_per_block, smem);
-    case 4: return occupancy_t<T, 4, STAGED, false>(warps_per_block, smem);
+    case 1: return occupancy_t<T, 1, STAGED>(warps_per_block, smem);
+    case 2: return occupancy_t<T, 2, STAGED>(warps_per_block, smem);
+    case 3: return occupancy_t<T, 3, STAGED>(warps_per_block, smem);
+    case 4: return occupancy_t<T, 4, STAGED>(warps_per_block, smem);
     default: return 0;
   }
 }
 
 template <typename T, bool STAGED>
-cudaError_t launch_ks(const MechDev &M, const CellsDev &C, const SolveParams &P, int blocks, bool coupled, bool dense,
+cudaError_t launch_ks(const MechDev &M, const CellsDev &C, const SolveParams &P, int blocks, bool coupled, int regs,
                       cudaStream_t stream) {
   switch ((M.S + WARP - 1) / WARP) {
-    case 1: return launch_t<T, 1, STAGED>(M, C, P, blocks, coupled, dense, stream);
-    case 2: return launch_t<T, 2, STAGED>(M, C, P, blocks, coupled, dense, stream);
-    case 3: return launch_t<T, 3, STAGED>(M, C, P, blocks, coupled, dense, stream);
-    case 4: return launch_t<T, 4, STAGED>(M, C, P, blocks, coupled, dense, stream);
+    case 1: return launch_t<T, 1, STAGED>(M, C, P, blocks, coupled, regs, stream);
+    case 2: return launch_t<T, 2, STAGED>(M, C, P, blocks, coupled, regs, stream);
+    case 3: return launch_t<T, 3, STAGED>(M, C, P, blocks, coupled, regs, stream);
+    case 4: return launch_t<T, 4, STAGED>(M, C, P, blocks, coupled, regs, stream);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -2751,36 +2739,35 @@ cudaError_t set_constants() {
   return cudaMemcpyToSymbol(c_igam, igam, sizeof(igam));
 }
 
-bool dense_solve(const MechDev &M, int lu_precision, int64_t n_cells) {
-  if (M.S > WARP || lu_precision != 32) return false;
+int solve_registers(const MechDev &M, int lu_precision, int driver, int couple, int64_t n_cells) {
   int dev = 0, n_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-  return n_cells > (int64_t)DENSE_CELLS_PER_SM * n_sm;
+  return register_rule(M.S, lu_precision, driver, couple, n_cells, n_sm);
 }
 
-int occupancy(const MechDev &M, int lu_precision, int driver, bool dense, int warps_per_block) {
+int occupancy(const MechDev &M, int lu_precision, int driver, int regs, int warps_per_block) {
   const size_t smem = staged_bytes(M, driver) + smem_per_cell(M, lu_precision) * (size_t)warps_per_block;
   const bool f32 = lu_precision == 32;
   if (staged_driver(driver))
-    return f32 ? occupancy_ks<float, true>(M, dense, warps_per_block, smem)
-               : occupancy_ks<double, true>(M, dense, warps_per_block, smem);
-  return f32 ? occupancy_ks<float, false>(M, dense, warps_per_block, smem)
-             : occupancy_ks<double, false>(M, dense, warps_per_block, smem);
+    return f32 ? occupancy_ks<float, true>(M, regs, warps_per_block, smem)
+               : occupancy_ks<double, true>(M, regs, warps_per_block, smem);
+  return f32 ? occupancy_ks<float, false>(M, regs, warps_per_block, smem)
+             : occupancy_ks<double, false>(M, regs, warps_per_block, smem);
 }
 
-int best_warps_per_block(const MechDev &M, int lu_precision, int driver, bool dense) {
+int best_warps_per_block(const MechDev &M, int lu_precision, int driver, int regs) {
   const int wmax = max_warps_per_block(M, lu_precision, driver);
   // The plain driver runs one cell per block: a block retires only when its
   // slowest cell does, and that tail costs more than the odd extra resident
   // cell a larger block may fit (72/186, 10,000 cells: 49.6 ms at 1 cell per
   // block against 64.1 ms at 11).
-  if (!staged_driver(driver)) return (wmax >= 1 && occupancy(M, lu_precision, driver, dense, 1) >= 1) ? 1 : 0;
+  if (!staged_driver(driver)) return (wmax >= 1 && occupancy(M, lu_precision, driver, regs, 1) >= 1) ? 1 : 0;
   // The persistent driver stages the tables once per block: most resident
   // cells per SM, ties to the larger block.
   int best_w = 0, best_cells = 0;
   for (int w = 1; w <= wmax; ++w) {
-    const int cells = w * occupancy(M, lu_precision, driver, dense, w);
+    const int cells = w * occupancy(M, lu_precision, driver, regs, w);
     if (cells > 0 && cells >= best_cells) {
       best_cells = cells;
       best_w = w;
@@ -2794,17 +2781,17 @@ int best_warps_per_block(const MechDev &M, int lu_precision, int driver, bool de
 // one block fills an SM: a recording batch keeps the full occupancy (four recorded
 // steps of 2,048 cells 13.5 / 13.8 / 14.0 ms at 12 / 10 / 8 per SM), as do the FP32
 // factorisation and blocks that share an SM, for which it was not measured.
-void auto_shape(const MechDev &M, int lu_precision, int driver, bool dense, int couple, bool record, int64_t n_cells,
+void auto_shape(const MechDev &M, int lu_precision, int driver, int regs, int couple, bool record, int64_t n_cells,
                 int *warps_per_block, int *blocks_per_sm) {
   const int full = couple > 1 ? (max_warps_per_block(M, lu_precision, driver) / couple) * couple
-                              : best_warps_per_block(M, lu_precision, driver, dense);
+                              : best_warps_per_block(M, lu_precision, driver, regs);
   *warps_per_block = full;
   if (!staged_driver(driver) || full < 1) return;
   int dev = 0, n_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   if (n_sm < 1) return;
-  const bool narrow = couple <= 1 && lu_precision == 64 && !record && occupancy(M, lu_precision, driver, dense, full) == 1;
+  const bool narrow = couple <= 1 && lu_precision == 64 && !record && occupancy(M, lu_precision, driver, regs, full) == 1;
   const int w = shape_warps(full, couple, n_cells, n_sm, narrow);
   if (w < 1 || w >= full) return;
   *warps_per_block = w;
@@ -2858,7 +2845,7 @@ cudaError_t launch_solve(const MechDev &M, const CellsDev &C, const LaunchCfg &c
   int blocks;
   P.smem_bytes = 0;
   if (cfg.driver == CHEM_DRIVER_PERSISTENT) {
-    const int natural = occupancy(M, cfg.lu_precision, cfg.driver, cfg.dense, cfg.warps_per_block);
+    const int natural = occupancy(M, cfg.lu_precision, cfg.driver, cfg.regs, cfg.warps_per_block);
     int bps = cfg.blocks_per_sm > 0 ? cfg.blocks_per_sm : natural;
     if (bps < 1) bps = 1;
     // fewer resident blocks than fit: pad the blocks' shared memory so that
@@ -2873,8 +2860,8 @@ cudaError_t launch_solve(const MechDev &M, const CellsDev &C, const LaunchCfg &c
   const bool f32 = cfg.lu_precision == 32;
   const bool coupled = cfg.couple > 1;      // warps_per_block is then the group size
   if (staged)
-    return f32 ? launch_ks<float, true>(M, C, P, blocks, coupled, cfg.dense, stream) : launch_ks<double, true>(M, C, P, blocks, coupled, cfg.dense, stream);
-  return f32 ? launch_ks<float, false>(M, C, P, blocks, coupled, cfg.dense, stream) : launch_ks<double, false>(M, C, P, blocks, coupled, cfg.dense, stream);
+    return f32 ? launch_ks<float, true>(M, C, P, blocks, coupled, cfg.regs, stream) : launch_ks<double, true>(M, C, P, blocks, coupled, cfg.regs, stream);
+  return f32 ? launch_ks<float, false>(M, C, P, blocks, coupled, cfg.regs, stream) : launch_ks<double, false>(M, C, P, blocks, coupled, cfg.regs, stream);
 }
 
 cudaError_t launch_adjoint(const MechDev &M, const CellsDev &C, const AdjDev &A, cudaStream_t stream) {

@@ -138,11 +138,11 @@ extern "C" int chem_solve_step_noalloc(const chem_mech *mech, int64_t n_cells, c
   const int wmax = max_warps_per_block(mech->m.dev, o.lu_precision, CHEM_DRIVER_PERSISTENT);
   if (wmax < 1) return fail(CHEM_EINVAL, "mechanism working set does not fit in shared memory");
   if (o.cells_per_block > wmax) return fail(CHEM_EINVAL, "cells_per_block exceeds the shared-memory limit");
-  const bool dense = dense_solve(mech->m.dev, o.lu_precision, n_cells);
+  const int regs = solve_registers(mech->m.dev, o.lu_precision, CHEM_DRIVER_PERSISTENT, 1, n_cells);
   if (o.cells_per_block == 0) {
     int w = 0, bps = o.blocks_per_sm;
-    if (bps > 0) w = best_warps_per_block(mech->m.dev, o.lu_precision, CHEM_DRIVER_PERSISTENT, dense);
-    else auto_shape(mech->m.dev, o.lu_precision, CHEM_DRIVER_PERSISTENT, dense, 1, false, n_cells, &w, &bps);
+    if (bps > 0) w = best_warps_per_block(mech->m.dev, o.lu_precision, CHEM_DRIVER_PERSISTENT, regs);
+    else auto_shape(mech->m.dev, o.lu_precision, CHEM_DRIVER_PERSISTENT, regs, 1, false, n_cells, &w, &bps);
     o.cells_per_block = w;
     o.blocks_per_sm = bps;
   }
@@ -166,7 +166,7 @@ extern "C" int chem_solve_step_noalloc(const chem_mech *mech, int64_t n_cells, c
   LaunchCfg cfg{};
   cfg.lu_precision = o.lu_precision;
   cfg.driver = CHEM_DRIVER_PERSISTENT;
-  cfg.dense = dense;
+  cfg.regs = regs;
   cfg.warps_per_block = o.cells_per_block;
   cfg.blocks_per_sm = o.blocks_per_sm;
   cfg.rtol = o.rtol;

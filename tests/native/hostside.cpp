@@ -14,7 +14,7 @@ using namespace chemgpu;
 struct Solve {
   int64_t n;
   int warps, bps, steps;
-  bool dense;
+  int regs;
   bool lanes;           // the queue order was made by lanes (launch_order: solved)
 };
 static std::vector<Solve> solves;
@@ -34,11 +34,11 @@ cudaError_t set_constants() { return cudaSuccess; }
 size_t smem_per_cell(const MechDev &, int) { return 16384; }
 size_t staged_bytes(const MechDev &, int) { return 0; }
 int max_warps_per_block(const MechDev &, int, int) { return 12; }
-int best_warps_per_block(const MechDev &, int, int driver, bool) { return driver == CHEM_DRIVER_PERSISTENT ? 12 : 1; }
-int occupancy(const MechDev &, int, int, bool, int w) { return w <= 12 ? 12 / w : 0; }
+int best_warps_per_block(const MechDev &, int, int driver, int) { return driver == CHEM_DRIVER_PERSISTENT ? 12 : 1; }
+int occupancy(const MechDev &, int, int, int, int w) { return w <= 12 ? 12 / w : 0; }
 // the cells of a batch spread over 10 SMs
-bool dense_solve(const MechDev &, int prec, int64_t n) { return prec == 32 && n > 10 * DENSE_CELLS_PER_SM; }
-void auto_shape(const MechDev &, int, int driver, bool, int, bool, int64_t n, int *w, int *bps) {
+int solve_registers(const MechDev &m, int prec, int driver, int couple, int64_t n) { return register_rule(m.S, prec, driver, couple, n, 10); }
+void auto_shape(const MechDev &, int, int driver, int, int, bool, int64_t n, int *w, int *bps) {
   const int64_t per = (n + 9) / 10;
   if (driver != CHEM_DRIVER_PERSISTENT) { *w = 1; return; }
   *w = per < 12 ? (int)(per < 1 ? 1 : per) : 12;
@@ -83,7 +83,7 @@ cudaError_t launch_solve(const MechDev &m, const CellsDev &c, const LaunchCfg &c
     }
     for (int64_t i = 0; i < cd.n_cells * S; ++i) cd.y[i] += k;
     for (int64_t i = 0; i < cd.n_cells; ++i) cd.stats[i].steps = k;
-    solves.push_back({cd.n_cells, f.warps_per_block, f.blocks_per_sm, k, f.dense, order_lanes});
+    solves.push_back({cd.n_cells, f.warps_per_block, f.blocks_per_sm, k, f.regs, order_lanes});
   });
   return cudaSuccess;
 }
@@ -252,7 +252,7 @@ static int pipeline_shape() {
       solves.clear();
       CHECK(h.run(p, 1, nullptr) == 0 && h.run(p, 1, host_chunk) == 0);
       CHECK(solves.size() == 5 && solves[0].n == n);
-      for (const Solve &x : solves) CHECK(x.warps == solves[0].warps && x.bps == solves[0].bps && x.dense == (given && n == 1000));
+      for (const Solve &x : solves) CHECK(x.warps == solves[0].warps && x.bps == solves[0].bps && x.regs == (given && n == 1000 ? 80 : 168));
       CHECK(solves[0].warps == (given ? 7 : n < 120 ? n / 10 : 12));
       chem_pipeline_destroy(p);
     }
@@ -311,6 +311,23 @@ static int shape_rule() {
   return 0;
 }
 
+// Registers of the solve kernels: 168 but for up to 32 species, where large plain
+// batches take 128 and large batches of the FP32 factorisation 80.
+static int register_choice() {
+  const int P = CHEM_DRIVER_PLAIN, Q = CHEM_DRIVER_PERSISTENT;
+  for (int S : {1, 20, 32, 33, 72, 128})
+    for (int prec : {64, 32})
+      for (int drv : {P, Q})
+        for (int64_t n : {1, 1824, 1825, 12160, 12161, 1000000}) {
+          const int r = register_rule(S, prec, drv, 1, n, 152);
+          if (S > 32) CHECK(r == 168);
+          else if (prec == 32 && n > 12160) CHECK(r == 80);
+          else CHECK(r == (drv == P && n > 1824 ? 128 : 168));
+          CHECK(register_rule(S, prec, drv, 2, n, 152) == 168);
+        }
+  return 0;
+}
+
 int main(int argc, char **argv) {
   const std::string what = argc > 1 ? argv[1] : "";
   if (what == "create_is_complete") return create_is_complete();
@@ -319,6 +336,7 @@ int main(int argc, char **argv) {
   if (what == "pipeline_shape") return pipeline_shape();
   if (what == "graph_order") return graph_order();
   if (what == "shape_rule") return shape_rule();
+  if (what == "register_choice") return register_choice();
   std::printf("unknown scenario\n");
   return 2;
 }

@@ -1,5 +1,5 @@
-"""The solve kernel with fewer registers, which large FP32-factorisation batches of up
-to 32 species run: the same results, cell by cell, as the kernel smaller ones run."""
+"""The solve kernels with fewer registers, which large batches of up to 32 species run:
+the same results, cell by cell, as the kernels of smaller batches."""
 import numpy as np
 import pytest
 
@@ -17,8 +17,8 @@ def cg():
     return chemgpu
 
 
-def _solve(cg, mech, wl, n, driver, steps=1):
-    c = cg.Cells(mech, n, rtol=wl.rtol, atol=wl.atol, driver=driver, lu_precision=32)
+def _solve(cg, mech, wl, n, driver, steps=1, prec=32, **kw):
+    c = cg.Cells(mech, n, rtol=wl.rtol, atol=wl.atol, driver=driver, lu_precision=prec, **kw)
     c.set_state(wl.cells.T[:n], wl.cells.P[:n], np.ascontiguousarray(wl.cells.y[:, :n]))
     if steps == 1:
         c.solve_step(wl.dt)
@@ -47,3 +47,16 @@ def test_large_batch_equals_its_cells_in_small_batches(cg, driver, extra):
         ys, ss = _solve(cg, mech, sub, part, driver, steps)
         assert np.array_equal(y[:, c0:c0 + part].view(np.int64), ys.view(np.int64))
         assert np.array_equal(st[c0:c0 + part], ss)
+
+
+# the plain driver's last batch of 12 cells per SM and the first above it
+@pytest.mark.parametrize("kw", [{}, {"prec": 32}, {"record_adjoint": True, "tape_steps": 1500}],
+                         ids=["fp64", "fp32", "recording"])
+def test_plain_batch_equals_its_cells_in_small_batches(cg, kw):
+    n = 12 * torch.cuda.get_device_properties(0).multi_processor_count + 1
+    wl = synth.workload_small(n_cells=n)
+    mech = cg.Mechanism(wl.mech)
+    kw = {"prec": 64, **kw}
+    y, st = _solve(cg, mech, wl, n, "plain", **kw)
+    ys, ss = _solve(cg, mech, wl, n - 1, "plain", **kw)
+    assert np.array_equal(y[:, :n - 1].view(np.int64), ys.view(np.int64)) and np.array_equal(st[:n - 1], ss)

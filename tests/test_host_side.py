@@ -21,7 +21,7 @@ def exe(tmp_path_factory):
 
 
 @pytest.mark.parametrize("scenario", ["create_is_complete", "pipeline_is_ordered", "pipeline_memory",
-                                      "pipeline_shape", "graph_order", "shape_rule"])
+                                      "pipeline_shape", "graph_order", "shape_rule", "register_choice"])
 def test_host_side(exe, scenario):
     r = subprocess.run([exe, scenario], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
