@@ -2644,8 +2644,9 @@ __global__ void __launch_bounds__(32 * WARP) deriv_gather_kernel(const __grid_co
   unsigned char *const gs = smem + (D.tile_warps ? (size_t)TILE_GROUPS * D.tile_doubles * sizeof(double) : 0);
   const int tid = warp * WARP + lane, nt = D.gather_warps * WARP;
   const int tb = M.tab.staged;
-  // (what f reads of it, each section at its place; the op that the interpreter reads
-  // past the program's end is not run)
+  // (what f reads of it, each section at its place: 10,000 cells of 128 species, which
+  // have no tiles, 82.5 us with the whole prefix, 78.5 so; the op that the interpreter
+  // reads past the program's end is not run)
   auto stage = [&](int from, int bytes) {
     for (int i = from / 16 + tid; i < (from + bytes + 15) / 16; i += nt)
       reinterpret_cast<uint4 *>(gs)[i] = __ldg(reinterpret_cast<const uint4 *>(M.blob[0]) + i);
@@ -2944,11 +2945,12 @@ cudaError_t launch_deriv_gather(const MechDev &M, const CellsDev &C, const doubl
     if (fit < 1) return cudaErrorInvalidValue;
     const int64_t per_sm = (rest + n_sm - 1) / n_sm;
     D.gather_cells = (int)(per_sm < fit ? per_sm : fit);
-    // with few cells per block the copy of the tables takes most of the time, so the
-    // block has all its warps all the same (one warp per cell copying the whole
-    // prefix: 10 cells of 72 species 18.8 us, 10.9 so; of 128 species 27.1, 11.2;
-    // 10,000 of 128 species, which have no tiles, 82.5 with the whole prefix, 78.5)
-    D.gather_warps = used ? 32 - TILE_GROUPS * TILE_WARPS : GATHER_WARPS;
+    // without tiles the copy of the tables takes most of the time of a block with few
+    // cells, so it has all its warps all the same (one warp per cell copying the whole
+    // prefix: 10 cells of 72 species 18.8 us, 10.9 so; of 128 species 27.1, 11.2);
+    // beside tiles the copy passes under their work, and more warps would take issue
+    // slots from it (10,000 cells, 24.5 us with 8 warps for 2 cells, 22.6 with 2)
+    D.gather_warps = used ? D.gather_cells : GATHER_WARPS;
     const int64_t need = (rest + D.gather_cells - 1) / D.gather_cells;
     blocks = D.n_tiles > 0 && need < n_sm ? n_sm : need;      // with tiles per_sm <= fit, so need <= n_sm
   }
