@@ -2501,8 +2501,8 @@ cudaError_t launch_order_t(const MechDev &M, const CellsDev &C, const SolveParam
 //   gather  more warps run the compiled f program, one warp per cell (36
 //           instructions): the cells beyond the last whole round of one tile per
 //           SM, spread over the SMs, and batches too small for tiles.
-// 10,000 cells: 24.9 us a call against 38.9 us with every cell by the gather in
-// blocks of 16 cells.
+// 10,000 cells: 22.7 us a call among others (24.4 with a wait after each) against
+// 38.9 us with every cell by the gather in blocks of 16 cells.
 constexpr int TILE_CELLS = WARP;
 constexpr int GATHER_BAR = 1, TILE_BAR = 2;     // named barriers: the gather warps, the first tile group
 constexpr int GATHER_WARPS = 16;                // most gather warps of a block
