@@ -536,7 +536,8 @@ def run_gpu(args):
                 "cells": C, "designs": designs,
                 "note": "f(y) only, rate constants precomputed; median of 10 launches with L2 flushed between; "
                         "hbm_gbs counts y and k~ read and f written once per cell (the atomic designs re-read y "
-                        "per reaction and add through L2)"}
+                        "per reaction and add through L2); gather_warp_per_cell: this library's design, tiles of "
+                        "32 cells with a lane per cell and the compiled f program, a warp per cell, for the rest"}
         if "coupled_cells" in extras_sel:
             # the paper's multi-cell system: groups of G consecutive cells integrated as one system
             coupled = {}
